@@ -80,9 +80,13 @@ BatchShape g_shape = default_batch_shape();
 BatchShape default_batch_shape() {
     BatchShape s;
     s.threads = 256;
-    s.blocks_per_sm = 4;
-    s.offload = 3;  // every product in the integer pipelines: 6910 GB/s against 6767
-                    // with half the sums there, on the 4096-segment batch (GB300)
+    // The last blocks to finish set the time of a large batch, and the fewer
+    // tiles a block owns the better the block scheduler evens them out: on the
+    // 4096-segment batch (79k tiles, GB300) 4, 8, 16, 32 blocks per SM took
+    // 1153, 1124, 1087, 1075 us; smaller batches have fewer blocks than that.
+    s.blocks_per_sm = 32;
+    s.offload = 3;  // every product in the integer pipelines: 1075 us there, against
+                    // 1103 with half the sums (at its best grid)
     for (int b = 0; b < kBuckets; ++b) {
         s.tile_elems[b] = b < 13 ? 0 : 8192;
         s.unroll_log2[b] = 2;
@@ -616,7 +620,7 @@ int batch_tune_impl(int bmin, int bmax, unsigned flags, wxpy_batch_tune_result *
         double best_us = 1e30;
         int best_bps = shape.blocks_per_sm, best_of = shape.offload;
         for (int of : {0, 1, 3})
-            for (int bps : {1, 2, 4, 8}) {
+            for (int bps : {2, 4, 8, 32}) {
                 BatchShape cand = shape;
                 cand.blocks_per_sm = bps;
                 cand.offload = of;

@@ -155,21 +155,26 @@ __device__ __forceinline__ void wxpy_vec_emu(double alpha, const double (&x)[VW]
 }
 
 // The same with alpha's split `ca` at hand: EMU == 3 computes every product
-// RN(alpha*x) in the integer pipelines (fp64_mul.cuh; operands it leaves out
-// take the hardware multiply, out of line) and every sum on the FP64
-// pipeline, which then carries one instruction per element.
+// RN(alpha*x) in the integer pipelines (fp64_mul.cuh; a vector with an operand
+// it leaves out takes the hardware multiply, out of line) and every sum on the
+// FP64 pipeline, which then carries one instruction per element.
 template <int VW, int EMU>
 __device__ __forceinline__ void wxpy_vec_emu(double alpha, const MulCoef &ca, const double (&x)[VW],
                                              const double (&y)[VW], double (&w)[VW], int base) {
     if constexpr (EMU == 3) {
+        uint32_t away = ca.win != 0 ? 0u : 1u << 31;
+        uint64_t p[VW];
 #pragma unroll
-        for (int k = 0; k < VW; ++k) {
-            const uint64_t xb = (uint64_t)__double_as_longlong(x[k]);
-            bool slow = false;
-            uint64_t pb = mul_rn_core(ca, xb, slow);
-            if (slow) pb = mul_rn_hw_bits((uint64_t)__double_as_longlong(alpha), xb);  // out of line
-            w[k] = __dadd_rn(__longlong_as_double((long long)pb), y[k]);
+        for (int k = 0; k < VW; ++k)
+            p[k] = mul_rn_quick(ca, (uint64_t)__double_as_longlong(x[k]), away);
+        if ((int32_t)away < 0) {
+#pragma unroll
+            for (int k = 0; k < VW; ++k)  // out of line
+                p[k] = mul_rn_hw_bits((uint64_t)__double_as_longlong(alpha),
+                                      (uint64_t)__double_as_longlong(x[k]));
         }
+#pragma unroll
+        for (int k = 0; k < VW; ++k) w[k] = __dadd_rn(__longlong_as_double((long long)p[k]), y[k]);
     } else {
         wxpy_vec_emu<VW, EMU>(alpha, x, y, w, base);
     }

@@ -31,31 +31,47 @@ WX_MUL_FN uint32_t funnel_r(uint32_t lo, uint32_t hi, uint32_t sh) {
 #endif
 }
 
-// RN(a * b) in the integer pipelines (multiply-adds on the FMA pipeline,
-// about thirty ALU operations) -- less than half the ALU cost of add_rn_bits,
-// so a product is the cheaper operation to move off the FP64 pipeline.
+// RN(a * b) in the integer pipelines (multiply-adds on the FMA pipeline, the
+// rest on the ALU).
 //
 // Method (the definition of a correctly rounded product).  For normal
 // operands, split each 53-bit significand (hidden bit included) into a 21-bit
 // high and a 32-bit low limb; four 32x32-bit products give the exact 106-bit
 // product P = top 2^64 + w1 2^32 + w0, with P in [2^104, 2^106) and t = 1 when
-// P >= 2^105.  The unrounded significand is P >> (52 + t), the round bit is
-// bit 51 + t of P, and every bit below it is sticky; round to nearest, ties to
-// even.  The biased exponent is ea + eb - 1023 + t.  The result is assembled
-// by adding the 53-bit significand, hidden bit included, to
-// sign | (exponent - 1) << 52, so a rounding carry to 2^53 lands in the
-// exponent field by itself.  Operands that are zero, subnormal, infinite or
-// NaN, and products whose exponent leaves [1, 0x7FD] (a subnormal, or a
-// possible overflow), are flagged for the hardware instruction.
+// P >= 2^105.  The unrounded significand M is P >> (52 + t); g holds the 32
+// bits of P below it.  Adding 2^31 to g carries into M exactly when the
+// discarded part is at least one half, and g becomes 0 exactly when its own 32
+// bits are one half: the discarded part is then one half if w0 is 0 as well
+// (g reaches into w0, so the bits of w0 below g are zero exactly when w0 is),
+// and that tie goes to even by clearing the lowest bit of the rounded-up M.
+// The biased exponent is ea + eb - 1023 + t.  The result is assembled by
+// adding M, hidden bit included, to sign | (exponent - 1) << 52, so a rounding
+// carry to 2^53 lands in the exponent field by itself.
 
 // One operand split once for many products (a coefficient: prepared on the
 // host, read from the kernel's parameter space by every product).
 struct MulCoef {
-    uint32_t hi;  // high significand limb with the hidden bit (21 bits)
-    uint32_t lo;  // low significand limb (32 bits)
-    int32_t e;    // biased exponent - 1024; 2^20 when the operand is not normal
-    uint32_t k;   // sign << 31 plus (biased exponent - 1024) << 20, modulo 2^32
+    uint32_t hi;   // high significand limb with the hidden bit (21 bits)
+    uint32_t lo;   // low significand limb (32 bits)
+    int32_t e;     // biased exponent - 1024; 2^20 when the operand is not normal
+    uint32_t k;    // sign << 31 plus (biased exponent - 1024) << 20, modulo 2^32
+    uint32_t win;  // mul_rn_quick: first exponent field of the other operand's window, << 21
 };
+
+// The exponent window of mul_rn_quick: the 1024 exponent fields from first on,
+// every one of which gives a product in the normal range whatever t and the
+// rounding; 0 when the coefficient has no such window (it is not normal, or
+// 2^1020 or more in magnitude).  The window starts as near to 512 (values from
+// 2^-511) as the coefficient's exponent allows.
+WX_MUL_FN int mul_window_first(uint64_t ua) {
+    const int ea = (int)((ua >> 52) & 0x7FFu);
+    if (ea == 0 || ea == 0x7FF) return 0;
+    const int lo = 1024 - ea > 1 ? 1024 - ea : 1;               // result exponent field >= 1
+    const int top = 0x7FB + 1024 - ea;                          // .. and <= 0x7FD with t = 1
+    const int hi = (top < 0x7FE ? top : 0x7FE) - 1023;
+    if (lo > hi) return 0;
+    return lo > 512 ? lo : hi < 512 ? hi : 512;
+}
 
 WX_MUL_FN MulCoef mul_coef_of(uint64_t ua) {
     const uint32_t ah = (uint32_t)(ua >> 32);
@@ -65,61 +81,108 @@ WX_MUL_FN MulCoef mul_coef_of(uint64_t ua) {
     c.lo = (uint32_t)ua;
     c.e = ea - 1u >= 0x7FEu ? (1 << 20) : (int32_t)ea - 1024;
     c.k = (ah & 0x80000000u) + ((uint32_t)((int32_t)ea - 1024) << 20);
+    c.win = (uint32_t)mul_window_first(ua) << 21;
     return c;
 }
 
+// Rounds the 106-bit product top:w1:w0 and adds it to base (sign and exponent
+// field - 1 - t); *t_out is t.
+WX_MUL_FN uint64_t round_product(uint64_t top, uint32_t w1, uint32_t w0, uint32_t base,
+                                 uint32_t *t_out) {
+    const uint32_t tl = (uint32_t)top, th = (uint32_t)(top >> 32);
+    const uint32_t sh = (th >> 9) + 20u;  // 20 + t: bit 105 of P is bit 9 of th
+    const uint32_t ml = funnel_r(w1, tl, sh);
+    const uint32_t mh = funnel_r(tl, th, sh);  // < 2^21, hidden bit at bit 20
+    const uint32_t g = funnel_r(w0, w1, sh);
+    const uint32_t hw = (base - (20u << 20)) + (sh << 20) + mh;
+    uint32_t gs, lo, hi;
+#ifdef __CUDA_ARCH__
+    asm("add.cc.u32 %0, %3, 0x80000000;\n\t"
+        "addc.cc.u32 %1, %4, 0;\n\t"
+        "addc.u32 %2, %5, 0;"
+        : "=r"(gs), "=r"(lo), "=r"(hi)
+        : "r"(g), "r"(ml), "r"(hw));
+#else
+    gs = g + 0x80000000u;
+    lo = ml + (g >> 31);
+    hi = hw + (uint32_t)(lo < ml);
+#endif
+    lo = (gs | w0) == 0u ? lo & ~1u : lo;
+    *t_out = sh - 20u;
+    return ((uint64_t)hi << 32) | lo;
+}
+
 // The fast path of RN(c * b): the result's bits, and `slow` set when the
-// operands or the result leave it (the bits are then meaningless).
+// operands or the result leave it (the bits are then meaningless): operands
+// that are zero, subnormal, infinite or NaN, and products whose unrounded
+// exponent field leaves [1, 0x7FD] (a subnormal, or a possible overflow).
 WX_MUL_FN uint64_t mul_rn_core(const MulCoef &c, uint64_t ub, bool &slow) {
     const uint32_t bh = (uint32_t)(ub >> 32), bl = (uint32_t)ub;
     const uint32_t eb = (bh >> 20) & 0x7FFu;
     const uint32_t b1 = (bh & 0xFFFFFu) | 0x100000u;
     const uint64_t p00 = (uint64_t)c.lo * bl;
-    const uint64_t m1 = (uint64_t)c.hi * bl + (p00 >> 32);              // < 2^53 + 2^32
-    const uint64_t m2 = (uint64_t)c.lo * b1 + (uint32_t)m1;             // < 2^53 + 2^32
-    const uint64_t top = (uint64_t)c.hi * b1 + (m1 >> 32) + (m2 >> 32);  // P >> 64, < 2^42
-    const uint32_t w0 = (uint32_t)p00, w1 = (uint32_t)m2;
-    const uint32_t tl = (uint32_t)top, th = (uint32_t)(top >> 32);
-    const uint32_t t = th >> 9;                     // bit 105 of P
-    const uint32_t sh = 20 + t;                     // significand = (top:w1) >> sh
-    const uint32_t m0l = funnel_r(w1, tl, sh);
-    const uint32_t m0h = funnel_r(tl, th, sh);  // < 2^21, hidden bit at bit 20
-    const uint32_t rnd = (w1 >> (sh - 1)) & 1u;
-    const uint32_t stk = (w0 | (w1 << (33 - sh))) != 0u;
-    const uint32_t inc = rnd & (stk | m0l);
+    const uint64_t x = (uint64_t)c.hi * bl + (uint64_t)c.lo * b1 + (p00 >> 32);  // < 2^55
+    const uint64_t top = (uint64_t)c.hi * b1 + (x >> 32);                        // < 2^42
+    uint32_t t;
+    // sign and exponent: the two signs add modulo 2 in bit 31
+    const uint64_t bits =
+        round_product(top, (uint32_t)x, (uint32_t)p00, c.k + (bh & 0xFFF00000u), &t);
     const int32_t ebase = c.e + (int32_t)(eb + t);  // result exponent - 1
     slow = slow || (eb - 1u >= 0x7FEu) || ((uint32_t)ebase >= 0x7FDu);
-    // sign and exponent: the two signs add modulo 2 in bit 31
-    const uint32_t hw = c.k + (bh & 0xFFF00000u) + (t << 20) + m0h;
-    return (((uint64_t)hw << 32) | m0l) + inc;
+    return bits;
 }
 
-// RN(a * a): the same method with both operands one value, so the split is
-// taken once and the two cross products are one, doubled: P = A1^2 2^64 +
-// 2 A1 A0 2^32 + A0^2 for the limbs A1 (21 bits, hidden bit included) and A0
-// (32 bits).  The sign is always clear; the biased exponent is
-// 2 ea - 1023 + t.  `slow` as in mul_rn_core.
+// The same product with the cheapest range check, for kernels whose products
+// set the pace: ORs into `away` a word whose top bit is set when b's exponent
+// field lies outside the coefficient's window (mul_window_first; zeros,
+// subnormals, infinities and NaN always do, since a window lies in
+// [1, 0x7FE]); the bits are then meaningless.  The coefficient must have a
+// window.
+WX_MUL_FN uint64_t mul_rn_quick(const MulCoef &c, uint64_t ub, uint32_t &away) {
+    const uint32_t bh = (uint32_t)(ub >> 32), bl = (uint32_t)ub;
+    const uint32_t b1 = (bh & 0xFFFFFu) | 0x100000u;
+    away |= (bh << 1) - c.win;
+    const uint64_t p00 = (uint64_t)c.lo * bl;
+    const uint64_t x = (uint64_t)c.hi * bl + (uint64_t)c.lo * b1 + (p00 >> 32);
+    const uint64_t top = (uint64_t)c.hi * b1 + (x >> 32);
+    uint32_t t;
+    return round_product(top, (uint32_t)x, (uint32_t)p00, c.k + (bh & 0xFFF00000u), &t);
+}
+
+// RN(a * b) of two data operands, with a cheap range check: `slow` is set when
+// either exponent field is outside [512, 1534] (magnitudes 2^-511 up to 2^512),
+// where every product is in the normal range.
+WX_MUL_FN uint64_t mul_rn_quick2(uint64_t ua, uint64_t ub, bool &slow) {
+    const uint32_t ah = (uint32_t)(ua >> 32), al = (uint32_t)ua;
+    const uint32_t bh = (uint32_t)(ub >> 32), bl = (uint32_t)ub;
+    const uint32_t a1 = (ah & 0xFFFFFu) | 0x100000u, b1 = (bh & 0xFFFFFu) | 0x100000u;
+    slow |= ((ah << 1) - (512u << 21) >= (1023u << 21)) | ((bh << 1) - (512u << 21) >= (1023u << 21));
+    const uint64_t p00 = (uint64_t)al * bl;
+    const uint64_t x = (uint64_t)a1 * bl + (uint64_t)al * b1 + (p00 >> 32);
+    const uint64_t top = (uint64_t)a1 * b1 + (x >> 32);
+    uint32_t t;
+    return round_product(top, (uint32_t)x, (uint32_t)p00,
+                         (ah & 0xFFF00000u) + (bh & 0xFFF00000u) - (1024u << 20), &t);
+}
+
+// RN(a * a): both operands one value, so the split is taken once and the two
+// cross products are one, doubled: P = A1^2 2^64 + 2 A1 A0 2^32 + A0^2 for the
+// limbs A1 (21 bits, hidden bit included) and A0 (32 bits).  The sign is
+// always clear, so the top word of the result tells by itself whether the
+// exponent field left [1, 0x7FD]: 2 ea - 1024 + t runs from -1024 (zero,
+// subnormal) to 3071 (infinity, NaN), which as a field of 12 bits names each
+// value once, and the hidden bit adds one to it.  `slow` as in mul_rn_core.
 WX_MUL_FN uint64_t sqr_rn_core(uint64_t ua, bool &slow) {
     const uint32_t ah = (uint32_t)(ua >> 32), a0 = (uint32_t)ua;
-    const uint32_t ea = (ah >> 20) & 0x7FFu;
     const uint32_t a1 = (ah & 0xFFFFFu) | 0x100000u;
     const uint64_t p00 = (uint64_t)a0 * a0;
-    const uint64_t x = (uint64_t)a1 * a0;                    // < 2^53
-    const uint64_t m1 = (x << 1) + (p00 >> 32);              // < 2^54 + 2^32
-    const uint64_t top = (uint64_t)a1 * a1 + (m1 >> 32);     // P >> 64, < 2^42
-    const uint32_t w0 = (uint32_t)p00, w1 = (uint32_t)m1;
-    const uint32_t tl = (uint32_t)top, th = (uint32_t)(top >> 32);
-    const uint32_t t = th >> 9;
-    const uint32_t sh = 20 + t;
-    const uint32_t m0l = funnel_r(w1, tl, sh);
-    const uint32_t m0h = funnel_r(tl, th, sh);
-    const uint32_t rnd = (w1 >> (sh - 1)) & 1u;
-    const uint32_t stk = (w0 | (w1 << (33 - sh))) != 0u;
-    const uint32_t inc = rnd & (stk | m0l);
-    const int32_t ebase = 2 * (int32_t)ea - 1024 + (int32_t)t;  // result exponent - 1
-    slow = slow || (ea - 1u >= 0x7FEu) || ((uint32_t)ebase >= 0x7FDu);
-    const uint32_t hw = ((uint32_t)ebase << 20) + m0h;
-    return (((uint64_t)hw << 32) | m0l) + inc;
+    const uint64_t x = (uint64_t)(a1 << 1) * a0 + (p00 >> 32);  // < 2^55
+    const uint64_t top = (uint64_t)a1 * a1 + (x >> 32);           // P >> 64, < 2^42
+    uint32_t t;
+    const uint64_t bits = round_product(top, (uint32_t)x, (uint32_t)p00,
+                                        ((ah << 1) & 0xFFE00000u) - (1024u << 20), &t);
+    slow = slow || (uint32_t)(bits >> 32) - 0x100000u >= 0x7FD00000u;
+    return bits;
 }
 
 #ifdef __CUDACC__

@@ -560,7 +560,8 @@ int launch_reduce(int64_t n, double alpha, const double *x, const double *y, dou
     uint64_t ab;
     std::memcpy(&ab, &alpha, 8);
     a.ca = mul_coef_of(ab);
-    a.mul_sixteenths = cfg.mul;
+    // an alpha without an exponent window (zero, say): FP64 products
+    a.mul_sixteenths = a.ca.win != 0 ? cfg.mul : 0;
     a.drop_chunk = g_reduce_drop.load();
     uintptr_t any = (uintptr_t)x | (uintptr_t)y | (uintptr_t)w | (KIND == 1 ? (uintptr_t)z : 0);
     const bool vec = (any & 31u) == 0;

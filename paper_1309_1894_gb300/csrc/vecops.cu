@@ -22,7 +22,7 @@
 // has 3 products and 2 sums per element (32 bytes of traffic), maxpy with m
 // terms 2m operations per 8(m + 2) bytes.  Both are FP64-bound far below the
 // HBM roofline unless part of the arithmetic moves to the integer pipelines
-// (fp64_emu.cuh, fp64_mul.cuh).  A product costs about thirty ALU operations
+// (fp64_emu.cuh, fp64_mul.cuh).  A product costs about twenty ALU operations
 // there and a sum about seventy-five, so products are the cheaper ones to
 // move: a runtime fraction (in sixteenths) of each warp's loop iterations
 // computes all of its products in the integer pipeline, the rest in FP64;
@@ -72,7 +72,10 @@ __device__ __forceinline__ double double_of(uint64_t b) { return __longlong_as_d
 // p[j] = RN(c_j * e[F + j]), j < K, F = NIN - K (the data operands follow any
 // others).  PM = 1: integer-pipeline products, one out-of-line fallback to the
 // hardware instruction for the whole element when any of them leaves the
-// fast path.
+// fast path.  At n = 2^26 (GB300) the windowed products (mul_rn_quick) took
+// axpbypcz from 0.92 to 0.965 of the measured peak and maxpy with 4 / 8 terms
+// from 0.87 / 0.74 to 0.89 / 0.755, against the fully checked ones; there the
+// sums keep the FP64 pipeline at the rate a plain chain of sums reaches.
 template <int PM, int K, int NIN>
 __device__ __forceinline__ void products(const Coefs &c, const double (&e)[NIN], double (&p)[K]) {
     constexpr int F = NIN - K;
@@ -80,11 +83,11 @@ __device__ __forceinline__ void products(const Coefs &c, const double (&e)[NIN],
 #pragma unroll
         for (int j = 0; j < K; ++j) p[j] = __dmul_rn(c.d[j], e[F + j]);
     } else {
-        bool slow = false;
+        uint32_t away = 0;
         uint64_t b[K];
 #pragma unroll
-        for (int j = 0; j < K; ++j) b[j] = mul_rn_core(c.m[j], bits_of(e[F + j]), slow);
-        if (slow) {
+        for (int j = 0; j < K; ++j) b[j] = mul_rn_quick(c.m[j], bits_of(e[F + j]), away);
+        if ((int32_t)away < 0) {
 #pragma unroll
             for (int j = 0; j < K; ++j) b[j] = mul_rn_hw_bits(bits_of(c.d[j]), bits_of(e[F + j]));
         }
@@ -94,14 +97,14 @@ __device__ __forceinline__ void products(const Coefs &c, const double (&e)[NIN],
 }
 
 // The fast path of the integer-pipeline products alone: p[j] as in
-// products<1>, with `slow` set when any of them left the fast path (its
-// bits are then meaningless and the caller recomputes the element).
+// products<1>, with the top bit of `away` set when any of them left the fast
+// path (its bits are then meaningless and the caller recomputes the element).
 template <int K, int NIN>
 __device__ __forceinline__ void products_fast(const Coefs &c, const double (&e)[NIN], double (&p)[K],
-                                              bool &slow) {
+                                              uint32_t &away) {
     constexpr int F = NIN - K;
 #pragma unroll
-    for (int j = 0; j < K; ++j) p[j] = double_of(mul_rn_core(c.m[j], bits_of(e[F + j]), slow));
+    for (int j = 0; j < K; ++j) p[j] = double_of(mul_rn_quick(c.m[j], bits_of(e[F + j]), away));
 }
 
 template <int OFF>
@@ -115,9 +118,9 @@ struct AxpbyOp {
         return add_sel<OFF>(p[0], p[1], 1);
     }
     __device__ __forceinline__ static double apply_fast(const Coefs &c, const double (&e)[kIn],
-                                                        bool &slow) {
+                                                        uint32_t &away) {
         double p[2];
-        products_fast(c, e, p, slow);
+        products_fast(c, e, p, away);
         return add_sel<OFF>(p[0], p[1], 1);
     }
 };
@@ -134,9 +137,9 @@ struct AxpbypczOp {
         return add_sel<OFF>(s1, p[2], OFF == 1 ? 0 : 1);
     }
     __device__ __forceinline__ static double apply_fast(const Coefs &c, const double (&e)[kIn],
-                                                        bool &slow) {
+                                                        uint32_t &away) {
         double p[3];
-        products_fast(c, e, p, slow);
+        products_fast(c, e, p, away);
         const double s1 = add_sel<OFF>(p[0], p[1], 1);
         return add_sel<OFF>(s1, p[2], OFF == 1 ? 0 : 1);
     }
@@ -156,9 +159,9 @@ struct MaxpyOp {
         return acc;
     }
     __device__ __forceinline__ static double apply_fast(const Coefs &c, const double (&e)[kIn],
-                                                        bool &slow) {
+                                                        uint32_t &away) {
         double p[M];
-        products_fast(c, e, p, slow);
+        products_fast(c, e, p, away);
         double acc = e[0];
 #pragma unroll
         for (int j = 0; j < M; ++j) acc = add_sel<OFF>(acc, p[j], j + 1);
@@ -369,7 +372,7 @@ template <class Op, int PM, int TE>
 __device__ __forceinline__ void staged_tile(const Coefs &cf, const double *sb, double *out, int len,
                                             int c) {
     constexpr int NIN = Op::kIn;
-    bool slow = false;
+    uint32_t away = 0;
 #pragma unroll
     for (int j = 0; j < TE / 512; ++j) {
         const int p = 2 * c + 512 * j;
@@ -383,14 +386,14 @@ __device__ __forceinline__ void staged_tile(const Coefs &cf, const double *sb, d
                 double e[NIN];
 #pragma unroll
                 for (int k = 0; k < NIN; ++k) e[k] = v[k][q];
-                if constexpr (PM == 1) r[q] = Op::apply_fast(cf, e, slow);
+                if constexpr (PM == 1) r[q] = Op::apply_fast(cf, e, away);
                 else r[q] = Op::template apply<0>(cf, e);
             }
             st_global_v2_cs(out + p, r[0], r[1]);
         }
     }
     if constexpr (PM == 1) {
-        if (slow)
+        if ((int32_t)away < 0)
             staged_tile_fp64<Op, TE>(cf.d[0], cf.d[1], cf.d[2], cf.d[3], cf.d[4], cf.d[5], cf.d[6],
                                      cf.d[7], sb, out, len, c);
     }
@@ -535,6 +538,8 @@ int launch_ew(const double *const *in, double *out, int64_t n, const double *coe
         uint64_t b;
         std::memcpy(&b, &a.cf.d[k], 8);
         a.cf.m[k] = mul_coef_of(b);
+        // a coefficient without an exponent window (zero, say): FP64 products
+        if (k < ncoef && a.cf.m[k].win == 0) a.pm = 0;
     }
     cudaError_t e = injected_launch_error();
     if (e == cudaSuccess && (diff & 31u) == 0) {
