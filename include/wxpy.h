@@ -341,8 +341,11 @@ int wxpy_vecops_status(void);
  * vectors and result, owned by the caller; the call overwrites it, so calls in
  * flight at the same time need separate workspaces.  Nothing is allocated.
  * When x, y, w (and z) are all 32-byte aligned, the kernel of the current
- * configuration (wxpy_reduce_variant) reads them as 32-byte vectors;
- * otherwise every element is read and written on its own (same bits).
+ * configuration (wxpy_reduce_variant) reads them as 32-byte vectors; when
+ * they share an offset past 32 bytes the default kernel does so too;
+ * otherwise every element is read and written on its own (same bits).  Two
+ * kernels are launched (one when n <= 8192), the second summing the tile sums
+ * in the workspace.
  * Errors: WXPY_EINVAL (bad argument, workspace too small), WXPY_EOVERLAP,
  * WXPY_ECUDA. */
 int64_t wxpy_reduce_workspace_bytes(int64_t n);
@@ -368,9 +371,10 @@ int wxpy_reduce_pipes(int mul_sixteenths);
  * Same bits either way.  Process-wide. */
 int wxpy_reduce_sum_levels(int levels);
 
-/* The kernel of wxpy_norm2 / wxpy_dot for 32-byte co-aligned pointers
- * (other alignments always take the element path): 0 register-loaded (a
- * block of 256 threads per tile, 32-byte loads into registers); 1, 2, 3
+/* The kernel of wxpy_norm2 / wxpy_dot for 32-byte aligned pointers (other
+ * alignments always take kernel 0): 0 register-loaded (a block of 256 threads
+ * per tile, 32-byte loads into registers; on few tiles, and with no integer
+ * tree levels asked for, a cluster of blocks per tile); 1, 2, 3
  * staged through a shared-memory ring of bulk copies with (ring stages,
  * resident blocks per SM) = (4, 2), (3, 3), (2, 3); 4, 5, 6 warp-tiled (one
  * warp per tile, no block barrier; rows loaded together, resident 128-thread

@@ -13,11 +13,12 @@
 // blocks, four per SM; a block takes a tile, thread t the 32-byte vectors at
 // 1024k + 4t (k = 0..7), so element i = 1024k + 4t + q has bits 12..10 = k,
 // 9..7 = warp, 6..2 = lane, 1..0 = q.  The halving tree reduces bits from the
-// top down, each level where its operands live: bits 12..10 inside the
-// thread, 9..7 across warps through shared memory, 6..2 by warp shuffles,
-// 1..0 inside lane 0.  With pointers that are not 32-byte co-aligned (and for
-// the last, ragged tile) the same threads read and write every element on its
-// own.  For norm2, the first 0..3 in-thread levels may run as the integer-
+// top down: bits 12..10 inside the thread, 9..7 by the threads of four warps
+// from shared memory, 6..0 by one warp (column_sum).  Pointers that share an
+// offset past 32 bytes are read as aligned vectors too (kShifted); with
+// pointers whose offsets differ (and for the last, ragged tile) every element
+// is read and written on its own.  Calls of few tiles take the cluster form of
+// reduce_split.cu instead.  For norm2, the first 0..3 in-thread levels may run as the integer-
 // pipeline sum of non-negative values (fp64_addpos.cuh).
 //
 // Staged kernels (variants 1..3, co-aligned pointers).  One producer warp
@@ -43,8 +44,8 @@
 // bounded (bulk.cuh); one that runs out ends the kernel and is reported by
 // wxpy_reduce_status().
 //
-// Either way the tile sums go to a workspace, and the last block to finish
-// (an atomic ticket, no waiting) sums them with the same tree.
+// Every way the tile sums go to a workspace, and a second kernel sums them with
+// the same tree (reduce_split.cu).
 //
 // Pipes: per element two products (alpha*x and the term) and, on average, two
 // sums (the update's and one tree level).  A share of the tiles (mul_sixteenths,
@@ -63,92 +64,173 @@
 #include "bulk.cuh"
 #include "internal.h"
 #include "reduce_common.cuh"
+#include "single_kernel.cuh"
 
 namespace wx {
 namespace {
 
 constexpr int kThreads = 256;
 
-// The sum of tile `tile`; valid in thread 0.  red: 256 x 4 doubles of shared memory.
+// How a tile's elements are dealt to the threads.
+enum Deal {
+    kElements,  // one by one: any alignment, and the last, ragged tile
+    kVectors,   // 32-byte vectors: every pointer 32-byte aligned
+    kShifted    // 32-byte vectors: every pointer the same 8, 16 or 24 bytes past 32
+};
+
+// Terms of this thread's four elements of one row (1024 elements from `row`);
+// w stored, +0 terms past n.  The tree asks only that every row deals its
+// positions alike:
+//   kVectors   positions 4t .. 4t + 3
+//   kShifted   positions 4t - s .. 4t - s + 3, s elements past the boundary, so
+//              that they are an aligned vector; thread 0's first s positions wrap
+//              to the end of the row, and only its accesses are single ones
+//   kElements  positions 128 warp + lane + 32 q, so that the 8-byte accesses of
+//              a warp are contiguous
+template <int KIND, bool EMU, int DEAL>
+__device__ __forceinline__ void row_terms(const ReduceArgs &a, int64_t row, double (&t)[4]) {
+    if constexpr (DEAL == kVectors) {
+        vector_terms<KIND, EMU, true>(a, row + 4 * threadIdx.x, t);
+    } else if constexpr (DEAL == kShifted) {
+        const int64_t i = row + 4 * (int)threadIdx.x - a.shift;
+        double x[4], y[4], z[4], w[4];
+        if (threadIdx.x != 0) {
+            ld4(a.x + i, x);
+            ld4(a.y + i, y);
+            if constexpr (KIND == 1) ld4(a.z + i, z);
+        } else {
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const int64_t e = i + q + (q < a.shift ? 1024 : 0);
+                x[q] = a.x[e];
+                y[q] = a.y[e];
+                if constexpr (KIND == 1) z[q] = a.z[e];
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) element<KIND, EMU>(a, x[q], y[q], KIND == 1 ? z[q] : 0.0, w[q], t[q]);
+        if (threadIdx.x != 0) {
+            st4(a.w + i, w);
+        } else {
+#pragma unroll
+            for (int q = 0; q < 4; ++q) a.w[i + q + (q < a.shift ? 1024 : 0)] = w[q];
+        }
+    } else {
+        const int64_t i0 = row + 128 * (threadIdx.x >> 5) + (threadIdx.x & 31);
+        constexpr int G = EMU ? 2 : 1;  // elements loaded together
+#pragma unroll
+        for (int g = 0; g < 4; g += G) {
+            double x[G], y[G], z[G];
+#pragma unroll
+            for (int q = 0; q < G; ++q) {
+                const int64_t i = i0 + 32 * (g + q);
+                if (i < a.n) {
+                    x[q] = a.x[i];
+                    y[q] = a.y[i];
+                    if constexpr (KIND == 1) z[q] = a.z[i];
+                }
+            }
+#pragma unroll
+            for (int q = 0; q < G; ++q) {
+                const int64_t i = i0 + 32 * (g + q);
+                t[g + q] = 0.0;
+                if (i < a.n) {
+                    double w;
+                    element<KIND, EMU>(a, x[q], y[q], KIND == 1 ? z[q] : 0.0, w, t[g + q]);
+                    a.w[i] = w;
+                }
+            }
+        }
+    }
+}
+
+// The sum of tile `tile`; valid in thread 0.  red: 1024 doubles of shared memory,
+// the node of position p of the rows at red[p]; node: 128 doubles.
 // SUML (norm2 only): the first SUML of the three in-thread tree levels run as
 // integer-pipeline sums of non-negative values.
-template <int KIND, bool VEC, bool EMU, int SUML = 0>
-__device__ double tile_sum(const ReduceArgs &a, int64_t tile, double (*red)[4]) {
+template <int KIND, int DEAL, bool EMU, int SUML = 0>
+__device__ double tile_sum(const ReduceArgs &a, int64_t tile, double *red, double *node) {
     static_assert(SUML == 0 || KIND == 0, "integer tree sums need non-negative terms");
     const int t = threadIdx.x, lane = t & 31;
-    const int64_t t0 = tile * kTile + 4 * t;
-    // bits 12..10: r[j] = tree over k = j, j+4 (bit 12), then j, j+2 (bit 11), then bit 10
-    // j in the order 0, 2, 1, 3: each pair (0, 2), (1, 3) is summed (bit 11)
-    // as soon as both are formed, so at most two level-1 vectors are live
-    double p[2][4];
-#pragma unroll
+    const int64_t t0 = tile * kTile;
+    // bits 12..10: rows j and j + 4 (bit 12), then j and j + 2 (bit 11), then bit 10,
+    // with j in the order 0, 2, 1, 3: each pair (0, 2), (1, 3) is summed as soon as
+    // both are formed, so at most two level-1 vectors are live
+    constexpr int kUnroll = DEAL == kElements ? 1 : 2;
+    double pc[4] = {}, pp[4] = {};
+#pragma unroll kUnroll
     for (int h = 0; h < 2; ++h) {
-        double r[2][4];
-#pragma unroll
+        double rc[4] = {}, rp[4] = {};
+#pragma unroll kUnroll
         for (int m = 0; m < 2; ++m) {
             const int j = h + 2 * m;
             double lo[4], hi[4];
-            vector_terms<KIND, EMU, VEC>(a, t0 + 1024 * j, lo);
-            vector_terms<KIND, EMU, VEC>(a, t0 + 1024 * (j + 4), hi);
+            row_terms<KIND, EMU, DEAL>(a, t0 + 1024 * j, lo);
+            row_terms<KIND, EMU, DEAL>(a, t0 + 1024 * (j + 4), hi);
 #pragma unroll
-            for (int q = 0; q < 4; ++q) r[m][q] = tree_add<(SUML >= 1)>(lo[q], hi[q]);
+            for (int q = 0; q < 4; ++q) {
+                rp[q] = rc[q];
+                rc[q] = tree_add<(SUML >= 1)>(lo[q], hi[q]);
+            }
         }
 #pragma unroll
-        for (int q = 0; q < 4; ++q) p[h][q] = tree_add<(SUML >= 2)>(r[0][q], r[1][q]);
+        for (int q = 0; q < 4; ++q) {
+            pp[q] = pc[q];
+            pc[q] = tree_add<(SUML >= 2)>(rp[q], rc[q]);
+        }
     }
     double v[4];
 #pragma unroll
-    for (int q = 0; q < 4; ++q) v[q] = tree_add<(SUML >= 3)>(p[0][q], p[1][q]);
-    // bits 9..7: threads t and t + 128, t + 64, t + 32 through shared memory
+    for (int q = 0; q < 4; ++q) v[q] = tree_add<(SUML >= 3)>(pp[q], pc[q]);
+    if constexpr (DEAL == kVectors) {
+        double2 *d = reinterpret_cast<double2 *>(red + 4 * t);
+        d[0] = make_double2(v[0], v[1]);
+        d[1] = make_double2(v[2], v[3]);
+    } else if constexpr (DEAL == kShifted) {
 #pragma unroll
-    for (int q = 0; q < 4; ++q) red[t][q] = v[q];
-    __syncthreads();
-    if (t < 128) {
+        for (int q = 0; q < 4; ++q) red[(4 * t + q - a.shift) & 1023] = v[q];
+    } else {
 #pragma unroll
-        for (int q = 0; q < 4; ++q) red[t][q] = __dadd_rn(red[t][q], red[t + 128][q]);
-    }
-    __syncthreads();
-    if (t < 64) {
-#pragma unroll
-        for (int q = 0; q < 4; ++q) red[t][q] = __dadd_rn(red[t][q], red[t + 64][q]);
+        for (int q = 0; q < 4; ++q) red[128 * (t >> 5) + lane + 32 * q] = v[q];
     }
     __syncthreads();
     double s = 0.0;
-    if (t < 32) {
-#pragma unroll
-        for (int q = 0; q < 4; ++q) v[q] = __dadd_rn(red[t][q], red[t + 32][q]);
-        // bits 6..2: lanes L and L + 16, 8, 4, 2, 1
-#pragma unroll
-        for (int sh = 16; sh >= 1; sh >>= 1) {
-#pragma unroll
-            for (int q = 0; q < 4; ++q) v[q] = __dadd_rn(v[q], __shfl_down_sync(0xffffffffu, v[q], sh));
-        }
-        // bits 1..0 in lane 0: q and q + 2, then q and q + 1
-        if (lane == 0) s = __dadd_rn(__dadd_rn(v[0], v[2]), __dadd_rn(v[1], v[3]));
+    if (t < 128) {
+        node[t] = tree8<128>(red + t);  // bits 9..7
+        asm volatile("bar.sync 1, 128;" ::: "memory");
+        if (t < 32) s = column_sum(node, lane);  // bits 6..0
     }
-    __syncthreads();  // red is reused by the next tile
     return s;
 }
 
 // Register-loaded path: four resident blocks (64 registers), measured 4-5 %
-// faster than three.  VEC: full tiles by 32-byte vectors (32-byte aligned
-// pointers), else element by element; the last, ragged tile always element by
-// element with FP64 products.  The product split applies to every full tile.
-template <int KIND, bool VEC, int SUML = 0>
+// faster than three.  DEAL is for the full tiles; the last, ragged tile is
+// always element by element with FP64 products.  The product split applies to
+// every full tile.
+//
+// What bounds it: the FP64 pipeline.  A tile's 8192 update sums and 8191 tree
+// sums are 512 warp instructions, at 1.7 lanes per clock per SM; the tree's
+// end adds as few as it can to them: bits 9..7 are seven sums of four full
+// warps, bits 6..0 eight instructions of one.  Summing bits 9..7 by halves of
+// the block and bits 6..0 on four values per lane took 51 warp instructions
+// and four block barriers more per tile, of which 36 and one are left:
+// norm2 at n = 2^26 (GB300) went from 309 to 289 us.
+template <int KIND, int DEAL, int SUML = 0>
 __global__ void __launch_bounds__(kThreads, 4) wxpy_reduce_kernel(const ReduceArgs a) {
-    __shared__ double red[kThreads][4];
-    __shared__ bool last;
+    __shared__ __align__(16) double red[2][1024];  // two tiles in turn: one block barrier per tile
+    __shared__ double node[128];
+    pdl_enter();
     const int64_t full = a.n / kTile;        // tiles with every element present
     unsigned slot = (blockIdx.x * 7u) & 15u;  // block-uniform rotation of the pipe choice
-    for (int64_t tile = blockIdx.x; tile < a.ntiles; tile += gridDim.x) {
+    int turn = 0;
+    for (int64_t tile = blockIdx.x; tile < a.ntiles; tile += gridDim.x, turn ^= 1) {
         double s;
-        if (tile >= full) s = tile_sum<KIND, false, false>(a, tile, red);
-        else if ((int)slot < a.mul_sixteenths) s = tile_sum<KIND, VEC, true, SUML>(a, tile, red);
-        else s = tile_sum<KIND, VEC, false, SUML>(a, tile, red);
+        if (tile >= full) s = tile_sum<KIND, kElements, false>(a, tile, red[turn], node);
+        else if ((int)slot < a.mul_sixteenths) s = tile_sum<KIND, DEAL, true, SUML>(a, tile, red[turn], node);
+        else s = tile_sum<KIND, DEAL, false, SUML>(a, tile, red[turn], node);
         if (threadIdx.x == 0) a.partial[tile] = s;
         slot = (slot + 1u) & 15u;
     }
-    finish_grid(a, last);
 }
 
 // ---- staged path ---------------------------------------------------------------
@@ -321,10 +403,7 @@ __device__ __forceinline__ void finish_tile(const ReduceArgs &a, const double *x
 #pragma unroll
         for (int q = 0; q < 2; ++q) p[q] = __dadd_rn(p[q], __shfl_down_sync(0xffffffffu, p[q], sh));
     }
-    if (lane == 0) {
-        a.partial[tile] = __dadd_rn(p[0], p[1]);  // bit 0
-        __threadfence();
-    }
+    if (lane == 0) a.partial[tile] = __dadd_rn(p[0], p[1]);  // bit 0
 }
 
 template <int KIND, int S, int MINB>
@@ -334,7 +413,6 @@ __global__ void __launch_bounds__(kStagedThreads, MINB) wxpy_reduce_staged_kerne
     extern __shared__ __align__(128) double ring[];  // [S][NIN][kChunk], then the exchange
     double *exch = ring + (size_t)S * RS::kStageElems;  // two slots of 8 x 128 doubles
     __shared__ __align__(8) uint64_t full[S], empty[S], xfull[2], xempty[2];
-    __shared__ bool last;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int64_t full_tiles = a.n / kTile;
     if (threadIdx.x == 0) {
@@ -419,7 +497,6 @@ __global__ void __launch_bounds__(kStagedThreads, MINB) wxpy_reduce_staged_kerne
             slot = (slot + 1u) & 15u;
         }
     }
-    finish_grid(a, last);
 }
 
 // Per staged shape and device: the dynamic shared-memory opt-in done and the
@@ -456,20 +533,21 @@ cudaError_t launch_staged(const ReduceArgs &a, const DeviceProps *dp, cudaStream
     return cudaGetLastError();
 }
 
-template <int KIND, bool VEC>
-int blocks_per_sm(int device) {
+template <int KIND, int DEAL, int SUML>
+cudaError_t launch_block(const ReduceArgs &a, const DeviceProps *dp, cudaStream_t s) {
     static std::atomic<int> cached[64];
-    if (device < 0 || device >= 64) return 1;
-    int v = cached[device].load(std::memory_order_relaxed);
-    if (v > 0) return v;
-    int nb = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, wxpy_reduce_kernel<KIND, VEC>, kThreads,
-                                                      0) != cudaSuccess || nb < 1) {
-        cudaGetLastError();
-        nb = 1;
+    const int dev = dp->device;
+    int nb = dev >= 0 && dev < 64 ? cached[dev].load(std::memory_order_relaxed) : 0;
+    if (nb <= 0) {
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, wxpy_reduce_kernel<KIND, DEAL, SUML>,
+                                                          kThreads, 0) != cudaSuccess || nb < 1) {
+            cudaGetLastError();
+            nb = 1;
+        }
+        if (dev >= 0 && dev < 64) cached[dev].store(nb, std::memory_order_relaxed);
     }
-    cached[device].store(nb, std::memory_order_relaxed);
-    return nb;
+    const int64_t grid = std::max<int64_t>(1, std::min<int64_t>((int64_t)dp->sm_count * nb, a.ntiles));
+    return launch_pdl(&wxpy_reduce_kernel<KIND, DEAL, SUML>, (unsigned)grid, kThreads, s, a);
 }
 
 std::atomic<int> g_reduce_mul{-1};
@@ -483,6 +561,13 @@ constexpr int kReduceVariants = 7;  // 0 register-loaded, 1..3 staged, 4..6 warp
 // (GB/s of algorithmic bytes, norm2 / dot): register-loaded 4482 / 5485;
 // staged (4, 2) 3771 / 4575, (3, 3) 3822 / 4252, (2, 3) 3904 / 4851.
 constexpr int kDefaultVariant[2] = {0, 0};  // norm2, dot
+// Tiles up to which a call takes the cluster form (reduce_split.cu).  Measured on
+// GB300, norm2 / dot, us, cluster against block form: 2^21 elements 16.7 / 18.2
+// against 17.8 / 19.5, 2^22 30.3 / 31.6 against 28.1 / 31.5.  With offsets that
+// differ the block form reads single elements too: 2^22 32.2 / 37.0 against
+// 34.2 / 37.2, 2^23 59.9 / 69.5 against 63.2 / 70.4, 2^24 107.6 / 121.7 against
+// 108.1 / 122.4.
+constexpr int64_t kSplitTiles = 256, kSplitTilesMixed = 1024;
 constexpr int kDefaultMulSixteenths = 16;  // measured fastest on GB300 (both operations)
 
 int64_t padded_tiles(int64_t n) {
@@ -551,7 +636,6 @@ int launch_reduce(int64_t n, double alpha, const double *x, const double *y, dou
     a.z = KIND == 1 ? z : nullptr;
     a.w = w;
     a.result = result;
-    a.ticket = (unsigned int *)workspace;
     a.partial = (double *)((char *)workspace + kHeaderBytes);
     a.n = n;
     a.ntiles = (n + kTile - 1) / kTile;
@@ -565,34 +649,32 @@ int launch_reduce(int64_t n, double alpha, const double *x, const double *y, dou
     a.drop_chunk = g_reduce_drop.load();
     uintptr_t any = (uintptr_t)x | (uintptr_t)y | (uintptr_t)w | (KIND == 1 ? (uintptr_t)z : 0);
     const bool vec = (any & 31u) == 0;
-    e = cudaMemsetAsync(a.ticket, 0, sizeof(unsigned int), s);
-    if (e != cudaSuccess) return fail_cuda(e, "reduce ticket");
+    const uintptr_t diff = ((uintptr_t)x ^ (uintptr_t)w) | ((uintptr_t)y ^ (uintptr_t)w) |
+                           (KIND == 1 ? (uintptr_t)z ^ (uintptr_t)w : 0);
+    const bool same = (diff & 31u) == 0;  // one offset modulo 32 bytes for all
+    a.shift = (int)(((uintptr_t)w >> 3) & 3u);
     const int variant = vec ? cfg.variant : 0;
-    if (variant == 0) {
-        const int nb = vec ? blocks_per_sm<KIND, true>(dp->device) : blocks_per_sm<KIND, false>(dp->device);
-        const int64_t grid = std::max<int64_t>(1, std::min<int64_t>((int64_t)dp->sm_count * nb, a.ntiles));
-        if (!vec) wxpy_reduce_kernel<KIND, false><<<(unsigned)grid, kThreads, 0, s>>>(a);
-        else if constexpr (KIND == 0) {
-            switch (std::min(cfg.suml, 3)) {  // the form's three in-thread levels
-                case 0: wxpy_reduce_kernel<0, true, 0><<<(unsigned)grid, kThreads, 0, s>>>(a); break;
-                case 1: wxpy_reduce_kernel<0, true, 1><<<(unsigned)grid, kThreads, 0, s>>>(a); break;
-                case 2: wxpy_reduce_kernel<0, true, 2><<<(unsigned)grid, kThreads, 0, s>>>(a); break;
-                default: wxpy_reduce_kernel<0, true, 3><<<(unsigned)grid, kThreads, 0, s>>>(a);
-            }
-        } else {
-            wxpy_reduce_kernel<KIND, true><<<(unsigned)grid, kThreads, 0, s>>>(a);
-        }
+    if (variant == 0 && cfg.suml == 0 && a.ntiles <= (vec || same ? kSplitTiles : kSplitTilesMixed)) {
+        e = launch_reduce_split(KIND, vec, a, s);
+        if (e == cudaSuccess && a.ntiles == 1) return WXPY_OK;
+    } else if (variant == 0) {
+        const int suml = KIND == 0 && vec ? std::min(cfg.suml, 3) : 0;  // the in-thread levels
+        if (!vec) e = same ? launch_block<KIND, kShifted, 0>(a, dp, s) : launch_block<KIND, kElements, 0>(a, dp, s);
+        else if constexpr (KIND == 0)
+            e = suml == 0   ? launch_block<0, kVectors, 0>(a, dp, s)
+                : suml == 1 ? launch_block<0, kVectors, 1>(a, dp, s)
+                : suml == 2 ? launch_block<0, kVectors, 2>(a, dp, s)
+                            : launch_block<0, kVectors, 3>(a, dp, s);
+        else e = launch_block<KIND, kVectors, 0>(a, dp, s);
     } else if (variant >= 4) {
-        const cudaError_t le = launch_reduce_warp(KIND, KIND == 0 ? cfg.suml : 0, variant - 4, a, dp, s);
-        if (le != cudaSuccess) return fail_cuda(le, "warp-tiled reduce launch");
+        e = launch_reduce_warp(KIND, KIND == 0 ? cfg.suml : 0, variant - 4, a, dp, s);
     } else {
         // staged shapes (ring stages, resident blocks): 1 (4, 2), 2 (3, 3), 3 (2, 3)
-        cudaError_t le = variant == 1   ? launch_staged<KIND, 4, 2>(a, dp, s)
-                         : variant == 2 ? launch_staged<KIND, 3, 3>(a, dp, s)
-                                        : launch_staged<KIND, 2, 3>(a, dp, s);
-        if (le != cudaSuccess) return fail_cuda(le, "staged reduce launch");
+        e = variant == 1   ? launch_staged<KIND, 4, 2>(a, dp, s)
+            : variant == 2 ? launch_staged<KIND, 3, 3>(a, dp, s)
+                           : launch_staged<KIND, 2, 3>(a, dp, s);
     }
-    e = cudaGetLastError();
+    if (e == cudaSuccess) e = launch_reduce_final(a, s);
     return e == cudaSuccess ? WXPY_OK : fail_cuda(e, "reduce launch");
 }
 

@@ -2,9 +2,10 @@
 // tile of the fixed summation tree, the argument block, the per-element
 // arithmetic (w = RN(RN(alpha*x) + y) of paper Sec. 3, Fig. 1, then the
 // term RN(w*w) or RN(w*z)), the integer-pipeline tree sum of non-negative
-// values, the 32-byte accesses, and the last block's sum of the tile sums.
-// Included by reduce.cu (register-loaded and staged forms) and
-// reduce_warp.cu (warp-tiled form); everything is internal to each.
+// values, the 32-byte accesses, and the end of a tile's tree.
+// Included by reduce.cu (register-loaded and staged forms), reduce_warp.cu
+// (warp-tiled form) and reduce_split.cu (a tile over a cluster of blocks, and
+// the tree over the tile sums); everything is internal to each.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -19,18 +20,18 @@
 namespace wx {
 
 constexpr int kTile = 8192;
-constexpr int64_t kHeaderBytes = 256;  // ticket counter, then the tile sums
+constexpr int64_t kHeaderBytes = 256;  // before the tile sums in the workspace
 
 struct ReduceArgs {
     const double *x, *y, *z;  // z: dot only
     double *w;
     double *result;
-    unsigned int *ticket;
-    double *partial;  // padded_tiles slots
+    double *partial;  // the tile sums: padded_tiles slots
     int64_t n, ntiles, padded_tiles;
     double alpha;
     MulCoef ca;
     int mul_sixteenths;
+    int shift;           // elements w starts past a 32-byte boundary (0..3)
     int64_t drop_chunk;  // staged path: the producer stops before this chunk (-1: never)
 };
 
@@ -144,34 +145,33 @@ __device__ __forceinline__ void vector_terms(const ReduceArgs &a, int64_t base, 
         }
     }
 }
-// The halving tree over partial[0 .. padded-1] (entries from ntiles on are +0),
-// by one block, in place.
-__device__ void final_tree(const ReduceArgs &a) {
-    const int t = threadIdx.x;
-    for (int64_t i = a.ntiles + t; i < a.padded_tiles; i += blockDim.x) a.partial[i] = 0.0;
-    __syncthreads();
-    for (int64_t s = a.padded_tiles / 2; s >= 1; s >>= 1) {
-        for (int64_t i = t; i < s; i += blockDim.x)
-            a.partial[i] = __dadd_rn(__ldcg(a.partial + i), __ldcg(a.partial + i + s));
-        __syncthreads();
-    }
-    if (t == 0) *a.result = __ldcg(a.partial);
+
+// Bits 6..0 of a tile's tree, by one warp, from the 128 node values that bits
+// 12..7 leave (node[j] at position j of a 128-element column, in shared
+// memory); valid in lane 0.  Lane l takes positions l + 32 r, so bits 6 and 5
+// are three sums in the lane and every further level is one instruction.
+__device__ __forceinline__ double column_sum(const double *node, int lane) {
+    double v = __dadd_rn(__dadd_rn(node[lane], node[lane + 64]),
+                         __dadd_rn(node[lane + 32], node[lane + 96]));
+#pragma unroll
+    for (int sh = 16; sh >= 1; sh >>= 1) v = __dadd_rn(v, __shfl_down_sync(0xffffffffu, v, sh));
+    return v;
 }
 
-// The last block to finish (after every tile sum of this grid is written)
-// sums the tile sums.  All threads of the block take part.
-__device__ __forceinline__ void finish_grid(const ReduceArgs &a, bool &last) {
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        __threadfence();
-        last = atomicAdd(a.ticket, 1u) == gridDim.x - 1;
-    }
-    __syncthreads();
-    if (last) {
-        __threadfence();
-        final_tree(a);
-    }
+// The halving tree over the eight values v[0], v[D], .., v[7 D] (three bits, the
+// top one first).
+template <int D>
+__device__ __forceinline__ double tree8(const double *v) {
+    return __dadd_rn(__dadd_rn(__dadd_rn(v[0], v[4 * D]), __dadd_rn(v[2 * D], v[6 * D])),
+                     __dadd_rn(__dadd_rn(v[D], v[5 * D]), __dadd_rn(v[3 * D], v[7 * D])));
 }
 
 }  // namespace
+
+// The cluster form (reduce_split.cu), for kind 0 (norm2) or 1 (dot); vec: every
+// pointer 32-byte aligned.  With one tile it writes the result itself.
+cudaError_t launch_reduce_split(int kind, bool vec, const ReduceArgs &a, cudaStream_t s);
+// The tree over the tile sums, after any form's kernel (reduce_split.cu).
+cudaError_t launch_reduce_final(const ReduceArgs &a, cudaStream_t s);
+
 }  // namespace wx

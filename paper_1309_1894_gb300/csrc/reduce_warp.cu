@@ -142,7 +142,6 @@ __device__ double warp_tile_sum(const ReduceArgs &a, int64_t tile, int lane) {
 
 template <int KIND, int SUML, int LR, int MINB>
 __global__ void __launch_bounds__(kWarpThreads, MINB) wxpy_reduce_warp_kernel(const ReduceArgs a) {
-    __shared__ bool last;
     const int lane = threadIdx.x & 31;
     const int64_t warps = (int64_t)gridDim.x * kWarpsPerBlock;
     const int64_t gw = (int64_t)blockIdx.x * kWarpsPerBlock + (threadIdx.x >> 5);
@@ -153,13 +152,9 @@ __global__ void __launch_bounds__(kWarpThreads, MINB) wxpy_reduce_warp_kernel(co
         if (tile >= full) s = warp_tile_sum<KIND, false, false, 0, LR>(a, tile, lane);
         else if ((int)slot < a.mul_sixteenths) s = warp_tile_sum<KIND, true, true, SUML, LR>(a, tile, lane);
         else s = warp_tile_sum<KIND, false, true, SUML, LR>(a, tile, lane);
-        if (lane == 0) {
-            a.partial[tile] = s;
-            __threadfence();
-        }
+        if (lane == 0) a.partial[tile] = s;
         slot = (slot + 1u) & 15u;
     }
-    finish_grid(a, last);
 }
 
 template <int KIND, int SUML, int LR, int MINB>
