@@ -229,11 +229,34 @@ Variant adjust_variant(const Variant &v, const CallClass &c) {
     return a;
 }
 
+// The variant of an untuned cell: 32-byte accesses, one pass per thread, and
+// (offload 3) every product in the integer pipelines, which leaves the FP64
+// pipeline one operation per element.  Measured on GB300, us per call back to
+// back with the inputs cold, against the single default {unroll 2, 256
+// threads, half the sums in the integer pipeline} that these lines replace:
 Variant default_variant(const CallClass &c, int64_t n) {
-    (void)n;
-    // 32-byte accesses, half the sums in the integer pipeline: the variant
-    // that streams at the HBM limit on GB300 when nothing is tuned.
-    Variant v{32, 2, 256, 0, 1, -1, 1, 1};
+    Variant v{32, 1, 128, 0, 1, -1, 1, 3};
+    const bool mixed = c.align < 32, xy = (c.alias & WXPY_ALIAS_XY) != 0;
+    if (n < ((int64_t)1 << 24)) {
+        // One vector per thread in small blocks: a short call has every load in
+        // flight at once, and a longer one ends on small blocks.  2^14 1.56
+        // against 2.09, 2^17 1.72 / 2.20, 2^22 15.3 / 16.0; offsets that differ
+        // 2^17 1.95 / 2.86, 2^22 15.1 / 16.4; x == y 2^22 10.5 / 13.9.
+        // Where the grid is between half a wave and one wave, 256 threads
+        // halve the blocks to start: 2^20 4.53 against 4.78 (and 6.05).
+        if (!mixed && n > ((int64_t)1 << 19) && n <= (int64_t)152 * 8 * 1024) v.threads = 256;
+    } else if (!mixed) {
+        // 2^24 56.4 / 57.1, 2^26 221.2 / 224.6, 2^28 878.8 / 885.9; x == y, where
+        // the sums' share weighs more, 38.8 / 49.6, 151.6 / 194.9, 599 / 772.
+        v.unroll = 2;
+        v.threads = 512;
+    } else if (xy) {
+        v.threads = 256;
+    } else {
+        // The old default holds: 2^24 56.8, 2^28 878.0 against 56.3, 883.8 with
+        // the products offloaded instead.
+        v = Variant{32, 2, 256, 0, 1, -1, 1, 1};
+    }
     return adjust_variant(v, c);
 }
 
