@@ -262,14 +262,14 @@ struct SingleEntry {
 // serialisation (api.cu; default on, WXPY_PDL=0 or wxpy_launch_pdl(0) off).
 bool pdl_enabled();
 
-// <<<grid, tpb, 0, s>>>, with the programmatic-serialisation attribute when on.
+// <<<grid, tpb, smem, s>>>, with the programmatic-serialisation attribute when on.
 template <typename... Args>
-cudaError_t launch_pdl(void (*kernel)(Args...), unsigned grid, unsigned tpb, cudaStream_t s,
-                       Args... args) {
+cudaError_t launch_pdl_smem(void (*kernel)(Args...), unsigned grid, unsigned tpb, size_t smem,
+                            cudaStream_t s, Args... args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);
     cfg.blockDim = dim3(tpb);
-    cfg.dynamicSmemBytes = 0;
+    cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -277,6 +277,12 @@ cudaError_t launch_pdl(void (*kernel)(Args...), unsigned grid, unsigned tpb, cud
     cfg.attrs = attr;
     cfg.numAttrs = pdl_enabled() ? 1 : 0;
     return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
+template <typename... Args>
+cudaError_t launch_pdl(void (*kernel)(Args...), unsigned grid, unsigned tpb, cudaStream_t s,
+                       Args... args) {
+    return launch_pdl_smem(kernel, grid, tpb, 0, s, args...);
 }
 
 template <int VW, int U, int GS, int CACHE, bool XY, int EMU>

@@ -223,6 +223,7 @@ __device__ __forceinline__ void elem_iter(const EwArgs<Op::kIn> &a, int64_t i0, 
 template <class Op>
 __global__ void __launch_bounds__(256) ew_elem_kernel(const EwArgs<Op::kIn> a) {
     constexpr int U = Op::kIn <= 3 ? 4 : (Op::kIn <= 5 ? 2 : 1);  // as elem_iter
+    pdl_enter();
     const int64_t tpb = blockDim.x;
     const int64_t stride = (int64_t)gridDim.x * tpb * U;
     // Warp-uniform rotation through 16 slots; slots below a.pm take the
@@ -270,6 +271,7 @@ __device__ __forceinline__ void direct_iter(const EwArgs<Op::kIn> &a, int64_t c0
 
 template <class Op>
 __global__ void __launch_bounds__(256) ew_direct_kernel(const EwArgs<Op::kIn> a) {
+    pdl_enter();
     const int64_t tpb = blockDim.x;
     const int64_t stride = (int64_t)gridDim.x * tpb * 2;
     unsigned slot = ((threadIdx.x >> 5) * 5u + blockIdx.x * 3u) & 15u;
@@ -417,6 +419,18 @@ __global__ void __launch_bounds__(kStagedThreads, StageShape<Op::kIn>::kMinBlock
         }
         mbar_init_fence();
     }
+    // The block's first tile on its way into the L2 while the launch before
+    // this one ends (a prefetch changes no value), then wait for that launch.
+    {
+        const int64_t e0 = (int64_t)blockIdx.x * TE;
+        const int64_t left = body - e0 < TE ? body - e0 : TE;
+        for (int64_t e = 16 * threadIdx.x; e < left; e += 16 * kStagedThreads) {
+#pragma unroll
+            for (int k = 0; k < NIN; ++k)
+                asm volatile("prefetch.global.L2 [%0];" ::"l"(a.in[k] + a.head + e0 + e));
+        }
+    }
+    pdl_enter();
     __syncthreads();
     if (warp == kConsumerWarps) {
         if (lane == 0) {
@@ -553,22 +567,21 @@ int launch_ew(const double *const *in, double *out, int64_t n, const double *coe
             const int64_t tiles = (a.nch * 4 + TE - 1) / TE;
             const int64_t grid =
                 std::max<int64_t>(1, std::min<int64_t>((int64_t)dp->sm_count * nb, tiles));
-            ew_staged_kernel<Op><<<(unsigned)grid, kStagedThreads, StageShape<NIN>::kSmem, s>>>(a);
+            e = launch_pdl_smem(&ew_staged_kernel<Op>, (unsigned)grid, kStagedThreads,
+                                StageShape<NIN>::kSmem, s, a);
         } else {
             const int64_t per_block = 256 * 2;
             const int64_t grid = std::max<int64_t>(
                 1, std::min<int64_t>((int64_t)dp->sm_count * 8, (a.nch + per_block - 1) / per_block));
-            ew_direct_kernel<Op><<<(unsigned)grid, 256, 0, s>>>(a);
+            e = launch_pdl(&ew_direct_kernel<Op>, (unsigned)grid, 256, s, a);
         }
-        e = cudaGetLastError();
     } else if (e == cudaSuccess) {
         a.head = 0;
         a.nch = n;
         const int64_t per_block = 256 * 4;
         const int64_t grid = std::max<int64_t>(
             1, std::min<int64_t>((int64_t)dp->sm_count * 8, (n + per_block - 1) / per_block));
-        ew_elem_kernel<Op><<<(unsigned)grid, 256, 0, s>>>(a);
-        e = cudaGetLastError();
+        e = launch_pdl(&ew_elem_kernel<Op>, (unsigned)grid, 256, s, a);
     }
     if (e != cudaSuccess) return fail_cuda(e, "vector kernel launch");
     return WXPY_OK;

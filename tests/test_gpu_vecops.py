@@ -311,3 +311,30 @@ def test_stream_and_graph_capture():
         torch.cuda.synchronize()
         assert same(z, z_want) and same(y, y_want)
     wx.wxpy_vecops_status()
+
+
+@pytest.mark.parametrize("off", [0, 8])
+@pytest.mark.parametrize("n", [67, 4099, 70001, 700001])
+def test_dependent_calls_back_to_back(n, off):
+    """A chain in which each call reads what the ones before wrote, through every
+    kernel of the family: a launch that overlaps the one before it must still
+    wait for its results."""
+    xh, yh, zh = (vals(3 * n + k, n, False) for k in range(3))
+    gx, gy, gz = (Guarded(n, off).set(v) for v in (xh, yh, zh))
+    gw = Guarded(n, 24 if off else 0)
+    for _ in range(4):
+        wx.wxpy_axpbypcz(0.5, -0.25, 0.75, gx.t, gy.t, gz.t)
+        wx.wxpy_pointwise_mult(gz.t, gx.t, gw.t)
+        wx.wxpy_axpby(0.5, 0.375, gw.t, gy.t)
+        wx.wxpy_maxpy([0.25, -0.5, 0.125], [gy.t, gw.t, gz.t], gx.t)
+        wx.wxpy_axpy(0.5, gx.t, gz.t)
+    torch.cuda.synchronize()
+    for _ in range(4):
+        zh = oracle.axpbypcz(0.5, -0.25, 0.75, xh, yh, zh)
+        wh = oracle.pmult(zh, xh)
+        yh = oracle.axpby(0.5, 0.375, wh, yh)
+        xh = oracle.maxpy([0.25, -0.5, 0.125], [yh, wh, zh], xh)
+        zh = oracle.axpy(0.5, xh, zh)
+    for g, h in ((gx, xh), (gy, yh), (gz, zh), (gw, wh)):
+        assert same(g.t, h)
+        g.check()
