@@ -451,7 +451,8 @@ typedef struct wxpy_batch_info {
  * independent: no two write overlapping ranges and none reads a range another
  * writes (WXPY_EOVERLAP).  Validation happens before any CUDA call.  The plan
  * cuts each problem into tiles whose length depends on its size bucket (tuned
- * by wxpy_batch_tune, else built in) and uploads the tile list to device
+ * by wxpy_batch_tune, else built in; shorter in a batch too small to give every
+ * SM work) and uploads the tile list to device
  * memory that the plan owns.  Synchronous.  *out is NULL on error. */
 int wxpy_batch_plan_create(const wxpy_desc *host_table, int64_t count,
                            wxpy_batch_plan **out);
@@ -482,8 +483,9 @@ int wxpy_batch_status(wxpy_batch_plan *plan, unsigned *status, int clear);
  * of it is still running).  NULL is a no-op. */
 int wxpy_batch_plan_destroy(wxpy_batch_plan *plan);
 
-/* One-shot form: validate, plan and launch in one call.  The tile list lives
- * in stream-ordered scratch (cudaMallocAsync / cudaFreeAsync on `stream`). */
+/* One-shot form: validate, plan and launch in one call.  Its plan, 24
+ * bytes per problem, lives in stream-ordered scratch (cudaMallocAsync /
+ * cudaFreeAsync on `stream`). */
 int wxpy_batch(const wxpy_desc *host_table, const wxpy_desc *dev_table, int64_t count,
                void *stream);
 
@@ -497,7 +499,7 @@ int wxpy_batch(const wxpy_desc *host_table, const wxpy_desc *dev_table, int64_t 
  * table of `count` descriptors, owned by the caller, as are all vectors).  It
  * calls no cudaMalloc, cudaFree or other allocating routine and takes no host
  * table: the tiles are planned on the device, in `stream`, into a fixed
- * scratch array of about 3 MiB that is a static device variable of the
+ * scratch array of about 1.5 MiB that is a static device variable of the
  * library, held by every GPU that loads the library until the process exits.
  * Limit: count <= 65536 (WXPY_EINVAL above it, before anything is launched).
  * The first call on a device looks up the scratch address

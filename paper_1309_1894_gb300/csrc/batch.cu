@@ -23,7 +23,7 @@
 
 #include "internal.h"
 #include "trace.h"
-#include "seg_tile.cuh"
+#include "seg_search.cuh"
 
 namespace wx {
 
@@ -38,9 +38,17 @@ struct SegParams {
 };
 
 // EMU: the integer-pipeline share (0 none, 1 half the sums, 3 every product),
-// chosen per launch.
-template <int EMU>
-__global__ void __launch_bounds__(256, 2) wxpy_seg_kernel(const SegParams p) {
+// chosen per launch.  Bound by HBM in large batches, by the three dependent
+// memory latencies of a tile (record, descriptor, vectors) in small ones, so
+// warps count for more than loads per warp: two vectors of x and of y per lane
+// and three resident blocks, against four and two, took 92.9 / 171 us against
+// 94.6 / 174 on 4096 / 2048 segments up to 2^16 / 2^18 elements and 44.6
+// against 51.9 on 40000 up to 1024 (GB300), and 1.5 % more on 4096 up to 2^20.
+// Reading the next tile's record and descriptor ahead gained nothing.
+// That batch, whose tiles are long, keeps the wide form (1075 us against 1090).
+template <int EMU, int MAXU>
+__global__ void __launch_bounds__(256, MAXU == kTileU ? 3 : 2) wxpy_seg_kernel(const SegParams p) {
+    pdl_enter();
     const int lane = threadIdx.x & 31;
     const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -52,23 +60,34 @@ __global__ void __launch_bounds__(256, 2) wxpy_seg_kernel(const SegParams p) {
             if (lane == 0) atomicOr(p.status, 1u);
             continue;
         }
-        tile_wxpy<EMU>(d.x + r.begin, d.y + r.begin, d.w + r.begin, d.alpha, len, lane,
-                       1 << (r.len_ul >> 30));
+        tile_wxpy<EMU, MAXU>(d.x + r.begin, d.y + r.begin, d.w + r.begin, d.alpha, len, lane,
+                             1 << (r.len_ul >> 30));
     }
 }
 
-static const void *seg_kernel_fn(int offload) {
-    return offload == 3   ? (const void *)&wxpy_seg_kernel<3>
-           : offload != 0 ? (const void *)&wxpy_seg_kernel<1>
-                          : (const void *)&wxpy_seg_kernel<0>;
+using SegKernelFn = void (*)(SegParams);
+
+// Long tiles: 2048 elements and more on average.
+static SegKernelFn seg_kernel_fn(int offload, int64_t ntiles, int64_t elems) {
+    const bool wide = elems >= 2048 * ntiles;
+    return offload == 3 ? (wide ? &wxpy_seg_kernel<3, kTileWideU> : &wxpy_seg_kernel<3, kTileU>)
+           : offload    ? (wide ? &wxpy_seg_kernel<1, kTileWideU> : &wxpy_seg_kernel<1, kTileU>)
+                        : (wide ? &wxpy_seg_kernel<0, kTileWideU> : &wxpy_seg_kernel<0, kTileU>);
 }
 
-static cudaError_t seg_launch(int offload, unsigned grid, int threads, const SegParams &sp,
-                              cudaStream_t s) {
-    if (offload == 3) wxpy_seg_kernel<3><<<grid, threads, 0, s>>>(sp);
-    else if (offload) wxpy_seg_kernel<1><<<grid, threads, 0, s>>>(sp);
-    else wxpy_seg_kernel<0><<<grid, threads, 0, s>>>(sp);
-    return cudaGetLastError();
+static cudaError_t seg_launch(int offload, unsigned grid, int threads, int64_t elems,
+                              const SegParams &sp, cudaStream_t s) {
+    return launch_pdl(seg_kernel_fn(offload, sp.ntiles, elems), grid, (unsigned)threads, s, sp);
+}
+
+// The same tiles without a list: the warp finds its tile's segment in the
+// per-segment plan (seg_search.cuh).  For one-shot calls, whose list would be
+// built and copied for a single launch.
+template <int EMU>
+__global__ void __launch_bounds__(256, 3)
+    wxpy_seg_search_kernel(const wxpy_desc *table, const SegPlan *plan, int64_t count) {
+    pdl_enter();
+    run_plan_tiles<EMU>(table, plan, count);
 }
 
 // ---------------------------------------------------------------- shapes
@@ -150,36 +169,100 @@ int validate_table(const wxpy_desc *t, int64_t count) {
     return WXPY_OK;
 }
 
-// Tile list of a validated table, largest tiles first (static round-robin
-// assignment then spreads the work evenly over the warps).
-int64_t build_tiles(const wxpy_desc *t, int64_t count, const BatchShape &shape,
-                    std::vector<TileRec> *out) {
-    out->clear();
+// Batches of kTargetTiles x 8192 elements and more keep the shape's tiles.
+// Smaller ones are cut into shorter tiles (down to 256 elements), so that their
+// warps still spread over every SM: with 8192-element tiles a lone problem of
+// 65536 elements would run on one block.
+constexpr int64_t kTargetTiles = 4864;  // 152 SMs x 4 blocks x 8 warps
+
+int64_t tile_cap(int64_t elems) {
+    int64_t t = 8192;
+    if (elems / t >= kTargetTiles) return kMaxTileElems;
+    while (t > 256 && elems / t < kTargetTiles) t >>= 1;
+    return t;
+}
+
+static int bucket_of(int64_t v) { return 63 - __builtin_clzll((unsigned long long)v); }
+
+static int64_t tile_len_of(const BatchShape &shape, int64_t n, int64_t t_cap) {
+    const int b = bucket_of(n);
+    const int64_t T = shape.tile_elems[b] > 0 ? shape.tile_elems[b] : n;
+    return std::min<int64_t>(std::min<int64_t>(T, t_cap), kMaxTileElems);
+}
+
+static int unroll_log2_of(const BatchShape &shape, int64_t n) {
+    return std::min<int>(2, std::max<int>(0, shape.unroll_log2[bucket_of(n)]));
+}
+
+// Blocks of a launch over `ntiles` tiles of `elems` elements in all.  Where the
+// tiles are short a block's start weighs as much as a tile, so blocks take
+// several: 40000 segments up to 1024 elements (147 each) 42.9 us with 6 blocks
+// per SM against 48.7 with 32, 20000 up to 4096 (490 each) 47.0 against 49.5;
+// from 4096 up to 65536 (1400 each) on there is no difference, or 32 is better.
+static unsigned batch_grid(const BatchShape &shape, int sm_count, int64_t ntiles, int64_t elems) {
+    const int64_t wpb = shape.threads / 32;
+    const int64_t bps = elems < 512 * ntiles ? std::min(shape.blocks_per_sm, 6) : shape.blocks_per_sm;
+    return (unsigned)std::max<int64_t>(1, std::min<int64_t>(bps * sm_count, (ntiles + wpb - 1) / wpb));
+}
+
+// Each problem cut into tiles of its size bucket's length (at most t_cap
+// elements), ordered longest first by eighths of an octave of the tile length --
+// a stable counting sort, linear in the tiles, so that a batch ends on short
+// tiles.  Returns the tile count; writes the tiles only when they fit in `cap`.
+int64_t fill_tiles(const wxpy_desc *t, int64_t count, const BatchShape &shape, int64_t t_cap,
+                   TileRec *out, int64_t cap) {
+    constexpr int kClasses = 64 * 8;
+    int64_t per_class[kClasses] = {0};
+    auto cls = [](int64_t len) {
+        const int b = bucket_of(len);
+        return b * 8 + (int)((b >= 3 ? len >> (b - 3) : len << (3 - b)) & 7);
+    };
     int64_t total = 0;
     for (int64_t s = 0; s < count; ++s) {
         const int64_t n = t[s].n;
-        if (n == 0) continue;
-        total += n;
-        const int b = 63 - __builtin_clzll((unsigned long long)n);
-        int64_t T = shape.tile_elems[b] > 0 ? shape.tile_elems[b] : n;
-        T = std::min<int64_t>(T, kMaxTileElems);
-        const uint32_t ul = (uint32_t)std::min<int>(2, std::max<int>(0, shape.unroll_log2[b])) << 30;
-        for (int64_t b0 = 0; b0 < n; b0 += T)
-            out->push_back(TileRec{b0, (int32_t)s, (uint32_t)std::min<int64_t>(T, n - b0) | ul});
+        if (n <= 0) continue;
+        const int64_t T = tile_len_of(shape, n, t_cap);
+        per_class[cls(T)] += n / T;
+        if (n % T) per_class[cls(n % T)] += 1;
+        total += (n + T - 1) / T;
     }
-    std::stable_sort(out->begin(), out->end(), [](const TileRec &a, const TileRec &b) {
-        return (a.len_ul & kLenMask) > (b.len_ul & kLenMask);
-    });
+    if (total > cap) return total;
+    int64_t start[kClasses];
+    int64_t pos = 0;
+    for (int c = kClasses - 1; c >= 0; --c) {
+        start[c] = pos;
+        pos += per_class[c];
+    }
+    for (int64_t s = 0; s < count; ++s) {
+        const int64_t n = t[s].n;
+        if (n <= 0) continue;
+        const int64_t T = tile_len_of(shape, n, t_cap);
+        const uint32_t ul = (uint32_t)unroll_log2_of(shape, n) << 30;
+        for (int64_t b0 = 0; b0 < n; b0 += T) {
+            const int64_t len = std::min<int64_t>(T, n - b0);
+            out[start[cls(len)]++] = TileRec{b0, (int32_t)s, (uint32_t)len | ul};
+        }
+    }
+    return total;
+}
+
+// Tile list of a validated table.  spread: shorter tiles for a small batch
+// (tile_cap); the search measures the shapes as they are.
+int64_t build_tiles(const wxpy_desc *t, int64_t count, const BatchShape &shape, bool spread,
+                    std::vector<TileRec> *out) {
+    int64_t total = 0;
+    for (int64_t s = 0; s < count; ++s) total += t[s].n;
+    const int64_t t_cap = spread ? tile_cap(total) : kMaxTileElems;
+    out->resize((size_t)fill_tiles(t, count, shape, t_cap, nullptr, -1));
+    fill_tiles(t, count, shape, t_cap, out->data(), (int64_t)out->size());
     return total;
 }
 
 cudaError_t launch_segmented(const wxpy_desc *dev_table, const TileRec *tiles, int64_t ntiles,
-                             unsigned *status, const BatchShape &shape, int sm_count,
+                             int64_t elems, unsigned *status, const BatchShape &shape, int sm_count,
                              cudaStream_t s) {
     if (ntiles == 0) return cudaSuccess;
-    const int64_t wpb = shape.threads / 32;
-    const unsigned grid = (unsigned)std::max<int64_t>(
-        1, std::min<int64_t>((int64_t)shape.blocks_per_sm * sm_count, (ntiles + wpb - 1) / wpb));
+    const unsigned grid = batch_grid(shape, sm_count, ntiles, elems);
     cudaError_t e = injected_launch_error();
     if (e != cudaSuccess) return e;
     SegParams sp;
@@ -187,7 +270,7 @@ cudaError_t launch_segmented(const wxpy_desc *dev_table, const TileRec *tiles, i
     sp.tiles = tiles;
     sp.ntiles = ntiles;
     sp.status = status;
-    return seg_launch(shape.offload, grid, shape.threads, sp, s);
+    return seg_launch(shape.offload, grid, shape.threads, elems, sp, s);
 }
 
 }  // namespace wx
@@ -246,12 +329,9 @@ int wxpy_batch_plan_create(const wxpy_desc *host_table, int64_t count, wxpy_batc
     p->count = count;
     p->shape = current_batch_shape();
     std::vector<TileRec> tiles;
-    p->total_elems = build_tiles(host_table, count, p->shape, &tiles);
+    p->total_elems = build_tiles(host_table, count, p->shape, true, &tiles);
     p->ntiles = (int64_t)tiles.size();
-    const int64_t warps_per_block = p->shape.threads / 32;
-    const int64_t max_grid = (int64_t)p->shape.blocks_per_sm * dp->sm_count;
-    p->grid = (unsigned)std::max<int64_t>(
-        1, std::min<int64_t>(max_grid, (p->ntiles + warps_per_block - 1) / warps_per_block));
+    p->grid = batch_grid(p->shape, dp->sm_count, p->ntiles, p->total_elems);
     cudaError_t e = cudaMalloc(&p->d_status, 256);
     if (e == cudaSuccess && p->ntiles > 0)
         e = cudaMalloc(&p->d_tiles, sizeof(TileRec) * (size_t)p->ntiles);
@@ -279,7 +359,7 @@ int wxpy_batch_launch(wxpy_batch_plan *plan, const wxpy_desc *dev_table, void *s
     if (!dev_table) return fail(WXPY_EINVAL, "null device table");
     cudaError_t e = injected_launch_error();
     if (e == cudaSuccess)
-        e = seg_launch(plan->shape.offload, plan->grid, plan->shape.threads,
+        e = seg_launch(plan->shape.offload, plan->grid, plan->shape.threads, plan->total_elems,
                        params_of(plan, dev_table), (cudaStream_t)stream);
     if (e != cudaSuccess) return fail_cuda(e, "batch kernel launch");
     return WXPY_OK;
@@ -294,7 +374,7 @@ int wxpy_batch_graph_launch(wxpy_batch_plan *plan, const wxpy_desc *dev_table, v
     SegParams sp = params_of(plan, dev_table);
     void *args[] = {&sp};
     cudaKernelNodeParams kp = {};
-    kp.func = const_cast<void *>(seg_kernel_fn(plan->shape.offload));
+    kp.func = (void *)seg_kernel_fn(plan->shape.offload, plan->ntiles, plan->total_elems);
     kp.gridDim = dim3(plan->grid);
     kp.blockDim = dim3(plan->shape.threads);
     kp.sharedMemBytes = 0;
@@ -350,35 +430,37 @@ int wxpy_batch(const wxpy_desc *host_table, const wxpy_desc *dev_table, int64_t 
     const DeviceProps *dp = current_device(&st);
     if (!dp) return st;
     const BatchShape shape = current_batch_shape();
-    std::vector<TileRec> tiles;
-    build_tiles(host_table, count, shape, &tiles);
-    if (tiles.empty()) return WXPY_OK;
+    // Per segment, not per tile: 24 bytes each whatever the tile length.
+    int64_t total = 0, ntiles = 0;
+    for (int64_t k = 0; k < count; ++k) total += host_table[k].n;
+    const int64_t t_cap = tile_cap(total);
+    std::vector<SegPlan> plan((size_t)count + 1);
+    for (int64_t k = 0; k < count; ++k) {
+        const int64_t n = host_table[k].n;
+        plan[k] = seg_plan_of(n, ntiles, n > 0 ? tile_len_of(shape, n, t_cap) : 1,
+                              n > 0 ? unroll_log2_of(shape, n) : 0);
+        ntiles += n > 0 ? (n + plan[k].tile_len() - 1) / plan[k].tile_len() : 0;
+    }
+    plan[count] = seg_plan_of(0, ntiles, 1, 0);
+    if (ntiles == 0) return WXPY_OK;
     cudaStream_t s = (cudaStream_t)stream;
-    // Stream-ordered scratch: tile list + status word, freed after the kernel.
-    const size_t bytes = sizeof(TileRec) * tiles.size() + 256;
+    // Stream-ordered scratch, freed after the kernel.
+    const size_t bytes = sizeof(SegPlan) * plan.size();
     void *buf = nullptr;
     cudaError_t e = cudaMallocAsync(&buf, bytes, s);
     if (e != cudaSuccess) {
         cudaGetLastError();
         return fail(WXPY_ENOMEM, "batch scratch allocation failed");
     }
-    auto *d_tiles = (TileRec *)((char *)buf + 256);
-    e = cudaMemsetAsync(buf, 0, 256, s);
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(d_tiles, tiles.data(), sizeof(TileRec) * tiles.size(),
-                            cudaMemcpyHostToDevice, s);
+    e = cudaMemcpyAsync(buf, plan.data(), bytes, cudaMemcpyHostToDevice, s);
+    if (e == cudaSuccess) e = injected_launch_error();
     if (e == cudaSuccess) {
-        SegParams sp;
-        sp.table = dev_table;
-        sp.tiles = d_tiles;
-        sp.ntiles = (int64_t)tiles.size();
-        sp.status = (unsigned *)buf;
-        const int64_t wpb = shape.threads / 32;
-        const unsigned grid = (unsigned)std::max<int64_t>(
-            1, std::min<int64_t>((int64_t)shape.blocks_per_sm * dp->sm_count,
-                                 ((int64_t)tiles.size() + wpb - 1) / wpb));
-        e = injected_launch_error();
-        if (e == cudaSuccess) e = seg_launch(shape.offload, grid, shape.threads, sp, s);
+        const unsigned grid = batch_grid(shape, dp->sm_count, ntiles, total);
+        const unsigned threads = (unsigned)shape.threads;
+        const SegPlan *d_plan = (const SegPlan *)buf;
+        e = shape.offload == 3 ? launch_pdl(&wxpy_seg_search_kernel<3>, grid, threads, s, dev_table, d_plan, count)
+            : shape.offload    ? launch_pdl(&wxpy_seg_search_kernel<1>, grid, threads, s, dev_table, d_plan, count)
+                               : launch_pdl(&wxpy_seg_search_kernel<0>, grid, threads, s, dev_table, d_plan, count);
     }
     cudaError_t e2 = cudaFreeAsync(buf, s);
     if (e != cudaSuccess) return fail_cuda(e, "batch launch");
@@ -487,7 +569,7 @@ int make_batch(int b, int bmin, int bmax, SynthBatch *sb, cudaStream_t s) {
 int upload_tiles(SynthBatch &sb, const BatchShape &shape, const DeviceProps &dp, int64_t *ntiles,
                  unsigned *grid, cudaStream_t s) {
     std::vector<TileRec> tiles;
-    build_tiles(sb.host.data(), (int64_t)sb.host.size(), shape, &tiles);
+    build_tiles(sb.host.data(), (int64_t)sb.host.size(), shape, false, &tiles);
     *ntiles = (int64_t)tiles.size();
     static thread_local size_t cap = 0;
     if (!sb.tiles.p || cap < tiles.size()) {
@@ -503,9 +585,7 @@ int upload_tiles(SynthBatch &sb, const BatchShape &shape, const DeviceProps &dp,
                                     cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) return fail_cuda(e, "batch search tile upload");
-    const int64_t wpb = shape.threads / 32;
-    *grid = (unsigned)std::max<int64_t>(
-        1, std::min<int64_t>((int64_t)shape.blocks_per_sm * dp.sm_count, (*ntiles + wpb - 1) / wpb));
+    *grid = batch_grid(shape, dp.sm_count, *ntiles, sb.elems);
     return WXPY_OK;
 }
 
@@ -524,7 +604,7 @@ int run_shape(SynthBatch &sb, const BatchShape &shape, const DeviceProps &dp, in
     // verification run on a poisoned output
     cudaError_t e = cudaMemsetAsync(sb.w.p, 0xff, (size_t)sb.slots * 8, s);
     if (e == cudaSuccess) e = cudaMemsetAsync(sb.count.p, 0, 8, s);
-    if (e == cudaSuccess) e = seg_launch(shape.offload, grid, shape.threads, sp, s);
+    if (e == cudaSuccess) e = seg_launch(shape.offload, grid, shape.threads, sb.elems, sp, s);
     if (e != cudaSuccess) return fail_cuda(e, "batch search launch");
     if ((st = launch_count_mismatch((const double *)sb.w.p, (const double *)sb.wref.p, sb.slots,
                                     (unsigned long long *)sb.count.p, s)))
@@ -535,7 +615,7 @@ int run_shape(SynthBatch &sb, const BatchShape &shape, const DeviceProps &dp, in
     std::vector<float> ms(reps);
     for (int r = 0; r < reps; ++r) {
         cudaEventRecord(e0, s);
-        seg_launch(shape.offload, grid, shape.threads, sp, s);
+        seg_launch(shape.offload, grid, shape.threads, sb.elems, sp, s);
         cudaEventRecord(e1, s);
         if ((e = cudaEventSynchronize(e1)) != cudaSuccess) return fail_cuda(e, "batch search timing");
         cudaEventElapsedTime(&ms[r], e0, e1);

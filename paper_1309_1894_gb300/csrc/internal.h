@@ -101,12 +101,15 @@ BatchShape default_batch_shape();
 BatchShape current_batch_shape();
 void set_batch_shape(const BatchShape &s);
 int validate_table(const wxpy_desc *t, int64_t count);
-// Tile list of a validated table (largest first); returns the element total.
-int64_t build_tiles(const wxpy_desc *t, int64_t count, const BatchShape &shape,
-                    std::vector<TileRec> *out);
-// One launch of the segmented kernel over `ntiles` device tile records.
+// batch.cu: longest tile of a batch of `elems` elements, so that a small batch
+// spreads over the GPU; a table's tile list (largest first), see there.
+int64_t tile_cap(int64_t elems);
+int64_t fill_tiles(const wxpy_desc *t, int64_t count, const BatchShape &shape, int64_t t_cap,
+                   TileRec *out, int64_t cap);
+// One launch of the segmented kernel over `ntiles` device tile records of `elems`
+// elements in all.
 cudaError_t launch_segmented(const wxpy_desc *dev_table, const TileRec *tiles, int64_t ntiles,
-                             unsigned *status, const BatchShape &shape, int sm_count,
+                             int64_t elems, unsigned *status, const BatchShape &shape, int sm_count,
                              cudaStream_t s);
 
 // api.cu: NVTX ranges on (WXPY_NVTX=1), read once; see trace.h.

@@ -303,61 +303,6 @@ __global__ void __launch_bounds__(256) serve_fill_kernel(const wxpy_desc *table,
     }
 }
 
-// Tile length cap for a batch of `elems` elements: small batches are cut into
-// shorter tiles (down to 256 elements), so that their warps still spread over
-// every SM -- with the batched shape's 8192-element tiles, a lone request of
-// 65k elements would run on one block.  Batches of kTargetTiles x 8192
-// elements and more keep the shape's tiles.
-constexpr int64_t kTargetTiles = 4864;  // 152 SMs x 4 blocks x 8 warps
-int64_t tile_cap(int64_t elems) {
-    int64_t t = 8192;
-    while (t > 256 && elems / t < kTargetTiles) t >>= 1;
-    return t;
-}
-
-// Tile list of a batch for the segmented kernel: each request cut into tiles
-// of its size bucket's length (the batch shape, as in wxpy_batch; at most
-// t_cap elements), ordered
-// longest first by power-of-two class of the tile length -- a stable counting
-// sort, linear in the tiles, so that the static round-robin over warps ends
-// on short tiles.  Returns the tile count; writes the tiles only when they
-// fit in `cap`.
-int64_t serve_tiles(const wxpy_desc *t, int64_t count, const BatchShape &shape, int64_t t_cap,
-                     TileRec *out, int64_t cap) {
-    int64_t per_class[64] = {0};
-    auto tile_len = [&](int64_t n) {
-        const int b = 63 - __builtin_clzll((unsigned long long)n);
-        const int64_t T = shape.tile_elems[b] > 0 ? shape.tile_elems[b] : n;
-        return std::min<int64_t>(std::min<int64_t>(T, t_cap), kMaxTileElems);
-    };
-    auto cls = [](int64_t len) { return 63 - __builtin_clzll((unsigned long long)len); };
-    int64_t total = 0;
-    for (int64_t s = 0; s < count; ++s) {
-        const int64_t n = t[s].n, T = tile_len(n);
-        per_class[cls(T)] += n / T;
-        if (n % T) per_class[cls(n % T)] += 1;
-        total += (n + T - 1) / T;
-    }
-    if (total > cap) return total;
-    int64_t start[64];
-    int64_t pos = 0;
-    for (int c = 63; c >= 0; --c) {
-        start[c] = pos;
-        pos += per_class[c];
-    }
-    for (int64_t s = 0; s < count; ++s) {
-        const int64_t n = t[s].n, T = tile_len(n);
-        const int b = 63 - __builtin_clzll((unsigned long long)n);
-        const uint32_t ul =
-            (uint32_t)std::min<int>(2, std::max<int>(0, shape.unroll_log2[b])) << 30;
-        for (int64_t b0 = 0; b0 < n; b0 += T) {
-            const int64_t len = std::min<int64_t>(T, n - b0);
-            out[start[cls(len)]++] = TileRec{b0, (int32_t)s, (uint32_t)len | ul};
-        }
-    }
-    return total;
-}
-
 // Saturated Poisson load on GB300 (n log-uniform in [2^8, 2^24]): 2.09e11
 // elements/s with every product in FP64, 1.82e11 with half, 1.59e11 with all
 // in the integer pipelines -- the generator keeps the ALU pipe busy and
@@ -581,7 +526,7 @@ cudaError_t launch_batch(wxpy_server *sv, Slot &s, const std::vector<Request *> 
         // The tile list of step (b), before anything of this batch is queued:
         // the slot is idle (its last batch completed), so a region too short
         // for this batch can be reallocated here (the tables are rewritten).
-        ntiles = serve_tiles(h_table, count, shape, tile_cap(elems), s.host<TileRec>(s.off_tiles),
+        ntiles = fill_tiles(h_table, count, shape, tile_cap(elems), s.host<TileRec>(s.off_tiles),
                              s.cap_tiles);
         if (ntiles > s.cap_tiles) {
             std::vector<wxpy_desc> t(h_table, h_table + count);
@@ -594,7 +539,7 @@ cudaError_t launch_batch(wxpy_server *sv, Slot &s, const std::vector<Request *> 
             std::copy(t.begin(), t.end(), h_table);
             std::copy(sd.begin(), sd.end(), h_seeds);
             std::copy(pl.begin(), pl.end(), h_plan);
-            ntiles = serve_tiles(h_table, count, shape, tile_cap(elems),
+            ntiles = fill_tiles(h_table, count, shape, tile_cap(elems),
                                  s.host<TileRec>(s.off_tiles), s.cap_tiles);
         }
     }
@@ -633,7 +578,7 @@ cudaError_t launch_batch(wxpy_server *sv, Slot &s, const std::vector<Request *> 
     // (b) one segmented launch over the batch: reads x, y, writes w; its
     // status word (uploaded as zero) comes back with the batch
     unsigned *d_status = s.dev<unsigned>(0);
-    e = launch_segmented(d_table, s.dev<TileRec>(s.off_tiles), ntiles, d_status, shape,
+    e = launch_segmented(d_table, s.dev<TileRec>(s.off_tiles), ntiles, elems, d_status, shape,
                          sv->sm_count, s.stream);
     if (e != cudaSuccess) return e;
     sv->launches += 1;
