@@ -13,8 +13,9 @@
 //   2. coalesces every admitted, not yet launched request (up to max_batch)
 //      into one batch and runs it on the next free stream in two steps:
 //      (a) the inputs are put into the requests' resident buffers -- one
-//      segmented fill launch generates x and y of every seeded request, and
-//      the caller-data requests are copied in;
+//      segmented launch generates x and y of the seeded requests, one copies
+//      those of the requests on the caller's device data; host data is copied
+//      request by request;
 //      (b) one launch of the batched segmented kernel (wxpy_seg_kernel, the
 //      same kernel and tile body as wxpy_batch) reads x and y from those
 //      buffers and writes w -- 24 bytes per element, one launch per batch
@@ -124,6 +125,7 @@ struct Request {
     // Caller data: source pointers and kind (WXPY_SERVE_DATA_*), or -1 for a
     // seeded request whose inputs the server generates.
     int src_kind = -1;
+    bool by_kernel = false;  // caller data in this device's memory: the inputs launch copies it
     const double *src_x = nullptr, *src_y = nullptr;
     int state = kQueued;
     bool auto_release = false;
@@ -146,8 +148,8 @@ struct ServePlan {
 
 // A batch in flight on one stream.  Its tables live in one staging region,
 // pinned on the host and mirrored on the device, so that a batch's tables go
-// up in ONE copy: [status word | descriptors | seeds | fill plan | tiles of
-// the segmented kernel], each part 256-byte aligned.  The status word is
+// up in ONE copy: [status word | descriptors | seeds | fill plan | sources |
+// copy plan | tiles of the segmented kernel], each part 256-byte aligned.  The status word is
 // uploaded as zero with the tables and comes back, after the kernels, into a
 // separate pinned word.
 struct Slot {
@@ -160,7 +162,8 @@ struct Slot {
     std::vector<uint64_t> tickets;
     int64_t cap_segs = 0, cap_tiles = 0;
     char *h_stage = nullptr, *d_stage = nullptr;
-    size_t off_table = 0, off_seeds = 0, off_plan = 0, off_tiles = 0, stage_bytes = 0;
+    size_t off_table = 0, off_seeds = 0, off_plan = 0, off_src = 0, off_cplan = 0, off_tiles = 0;
+    size_t stage_bytes = 0;
     unsigned *h_status = nullptr;  // the status word of the last batch, copied back
     template <class T>
     T *host(size_t off) const { return (T *)(h_stage + off); }
@@ -259,6 +262,41 @@ __global__ void __launch_bounds__(256) serve_fused_kernel(const wxpy_desc *table
     }
 }
 
+// Where the inputs of a request on the caller's device data are.
+struct ServeSrc {
+    const double *x, *y;
+};
+
+// Copies elements [begin, end) of one vector, by a warp; dst + begin is 32-byte
+// aligned (begin is a multiple of 4).  Four 32-byte vectors per lane in flight
+// where the source is aligned like the destination, else eight elements.
+__device__ __forceinline__ void copy_tile(const double *src, double *dst, int64_t begin,
+                                          int64_t end, int lane) {
+    int64_t i = begin;
+    if (((uintptr_t)src & 31u) == 0) {
+        const int64_t nvec = (end - begin) >> 2;
+        for (int64_t c = lane; c < nvec; c += 128) {
+            double v[4][4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                if (c + 32 * u < nvec) ld_vec<4, 2>(src + begin + 4 * (c + 32 * u), v[u]);
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                if (c + 32 * u < nvec) st_vec<4, 2>(dst + begin + 4 * (c + 32 * u), v[u]);
+        }
+        i = begin + 4 * nvec;
+    }
+    for (i += lane; i < end; i += 256) {
+        double v[8][1];
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+            if (i + 32 * u < end) ld_vec<1, 2>(src + i + 32 * u, v[u]);
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+            if (i + 32 * u < end) st_vec<1, 2>(dst + i + 32 * u, v[u]);
+    }
+}
+
 // The inputs step of a batch: for every seeded request, x and y from the
 // request's seed (streams (seed, 1) and (seed, 2), the values
 // wxpy_fill_uniform writes) stored into its resident buffers.  A warp takes a
@@ -300,6 +338,31 @@ __global__ void __launch_bounds__(256) serve_fill_kernel(const wxpy_desc *table,
             x[i] = uniform_pm1(kx, i);
             y[i] = uniform_pm1(ky, i);
         }
+    }
+}
+
+// The same for the requests on the caller's device data, in one launch: x and
+// y from there into the resident buffers.  32 bytes per element; bound by HBM
+// in large batches, by latency in small ones.  Two cudaMemcpyAsync per request
+// in its place cost the stream about 2.5 us each: a burst of 48 requests of
+// 2^8 to 2^20 elements waited 399 us for its results on GB300, 150 with this
+// launch.
+__global__ void __launch_bounds__(256) serve_copy_kernel(const wxpy_desc *table,
+                                                         const ServeSrc *src,
+                                                         const ServePlan *plan, int64_t count,
+                                                         int64_t ntiles) {
+    const int lane = threadIdx.x & 31;
+    const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    int64_t s = 0;
+    for (int64_t t = warp; t < ntiles; t += nwarps) {
+        s = find_request(plan, count, t, s);
+        const wxpy_desc d = table[s];
+        const ServePlan sp = plan[s];
+        const int64_t begin = (t - sp.first_tile) * sp.tile_len;
+        const int64_t end = min(d.n, begin + sp.tile_len);
+        copy_tile(src[s].x, const_cast<double *>(d.x), begin, end, lane);
+        copy_tile(src[s].y, const_cast<double *>(d.y), begin, end, lane);
     }
 }
 
@@ -371,7 +434,9 @@ cudaError_t alloc_stage(Slot &s, int64_t segs, int64_t tiles) {
     s.off_table = 256;
     s.off_seeds = s.off_table + align256(sizeof(wxpy_desc) * segs);
     s.off_plan = s.off_seeds + align256(sizeof(uint64_t) * segs);
-    s.off_tiles = s.off_plan + align256(sizeof(ServePlan) * segs);
+    s.off_src = s.off_plan + align256(sizeof(ServePlan) * segs);
+    s.off_cplan = s.off_src + align256(sizeof(ServeSrc) * segs);
+    s.off_tiles = s.off_cplan + align256(sizeof(ServePlan) * segs);
     const size_t bytes = s.off_tiles + sizeof(TileRec) * (size_t)tiles;
     cudaError_t e = cudaMalloc(&s.d_stage, bytes);
     if (e == cudaSuccess) e = cudaMallocHost(&s.h_stage, bytes);
@@ -499,17 +564,22 @@ cudaError_t launch_batch(wxpy_server *sv, Slot &s, const std::vector<Request *> 
     // fused mode; caller-data requests get none.
     wxpy_desc *h_table = s.host<wxpy_desc>(s.off_table);
     uint64_t *h_seeds = s.host<uint64_t>(s.off_seeds);
+    ServeSrc *h_src = s.host<ServeSrc>(s.off_src);
     ServePlan *h_plan = s.host<ServePlan>(s.off_plan);
-    int64_t nplan = 0, elems = 0, seeded = 0;
+    ServePlan *h_cplan = s.host<ServePlan>(s.off_cplan);
+    int64_t nplan = 0, ncopy = 0, elems = 0, seeded = 0, copied = 0;
     for (const Request *r : batch) {
         elems += r->n;
         if (r->src_kind < 0) seeded += r->n;
+        if (r->by_kernel) copied += r->n;
     }
     const int64_t fill_tile = std::min<int64_t>(kFillTile, tile_cap(seeded));
+    const int64_t copy_tile = std::min<int64_t>(kFillTile, tile_cap(copied));
     for (int64_t i = 0; i < count; ++i) {
         const Request *r = batch[i];
         h_table[i] = wxpy_desc{r->n, r->alpha, r->x, r->y, r->w};
         h_seeds[i] = r->seed;
+        h_src[i] = r->by_kernel ? ServeSrc{r->src_x, r->src_y} : ServeSrc{nullptr, nullptr};
         int64_t T = fill_tile;
         int ulog = 0;
         if (fused) {
@@ -520,6 +590,8 @@ cudaError_t launch_batch(wxpy_server *sv, Slot &s, const std::vector<Request *> 
         }
         h_plan[i] = ServePlan{nplan, T, ulog, 0};
         if (r->src_kind < 0) nplan += (r->n + T - 1) / T;
+        h_cplan[i] = ServePlan{ncopy, copy_tile, 0, 0};
+        if (r->by_kernel) ncopy += (r->n + copy_tile - 1) / copy_tile;
     }
     int64_t ntiles = 0;
     if (!fused) {
@@ -531,11 +603,16 @@ cudaError_t launch_batch(wxpy_server *sv, Slot &s, const std::vector<Request *> 
         if (ntiles > s.cap_tiles) {
             std::vector<wxpy_desc> t(h_table, h_table + count);
             std::vector<uint64_t> sd(h_seeds, h_seeds + count);
-            std::vector<ServePlan> pl(h_plan, h_plan + count);
+            std::vector<ServeSrc> sr(h_src, h_src + count);
+            std::vector<ServePlan> pl(h_plan, h_plan + count), cp(h_cplan, h_cplan + count);
             if ((e = alloc_stage(s, s.cap_segs, ntiles + ntiles / 4)) != cudaSuccess) return e;
             h_table = s.host<wxpy_desc>(s.off_table);
             h_seeds = s.host<uint64_t>(s.off_seeds);
+            h_src = s.host<ServeSrc>(s.off_src);
             h_plan = s.host<ServePlan>(s.off_plan);
+            h_cplan = s.host<ServePlan>(s.off_cplan);
+            std::copy(sr.begin(), sr.end(), h_src);
+            std::copy(cp.begin(), cp.end(), h_cplan);
             std::copy(t.begin(), t.end(), h_table);
             std::copy(sd.begin(), sd.end(), h_seeds);
             std::copy(pl.begin(), pl.end(), h_plan);
@@ -563,15 +640,31 @@ cudaError_t launch_batch(wxpy_server *sv, Slot &s, const std::vector<Request *> 
         sv->launches += 1;
         return cudaEventRecord(s.done, s.stream);
     }
-    // (a) inputs into the resident buffers
+    // (a) inputs into the resident buffers.  These kernels do not let the
+    // segmented one start early: its blocks would hold registers, waiting, that
+    // batches on the other streams could use (p50 at 3.2e4 requests/s 0.141 ms
+    // against 0.133).
     for (const Request *r : batch)
-        if (r->src_kind >= 0 && (e = copy_in(r, s.stream)) != cudaSuccess) return e;
+        if (r->src_kind >= 0 && !r->by_kernel && (e = copy_in(r, s.stream)) != cudaSuccess) return e;
+    auto input_grid = [&](int64_t tiles) {
+        return (unsigned)std::max<int64_t>(
+            1, std::min<int64_t>((int64_t)8 * sv->sm_count, (tiles + wpb - 1) / wpb));
+    };
     if (nplan > 0) {
-        const unsigned grid = (unsigned)std::max<int64_t>(
-            1, std::min<int64_t>((int64_t)8 * sv->sm_count, (nplan + wpb - 1) / wpb));
         e = injected_launch_error();
         if (e != cudaSuccess) return e;
-        serve_fill_kernel<<<grid, 256, 0, s.stream>>>(d_table, d_seeds, d_plan, count, nplan);
+        serve_fill_kernel<<<input_grid(nplan), 256, 0, s.stream>>>(d_table, d_seeds, d_plan, count,
+                                                                   nplan);
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        sv->launches += 1;
+    }
+    if (ncopy > 0) {
+        const ServeSrc *d_src = s.dev<ServeSrc>(s.off_src);
+        const ServePlan *d_cplan = s.dev<ServePlan>(s.off_cplan);
+        e = injected_launch_error();
+        if (e != cudaSuccess) return e;
+        serve_copy_kernel<<<input_grid(ncopy), 256, 0, s.stream>>>(d_table, d_src, d_cplan, count,
+                                                                   ncopy);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
         sv->launches += 1;
     }
@@ -745,7 +838,7 @@ void scheduler(wxpy_server *sv) {
 
 int submit_locked(wxpy_server *sv, int64_t n, double alpha, uint64_t seed, bool auto_release,
                   uint64_t *ticket, int src_kind = -1, const double *src_x = nullptr,
-                  const double *src_y = nullptr) {
+                  const double *src_y = nullptr, bool by_kernel = false) {
     if (n <= 0) return fail(WXPY_EINVAL, "request needs n > 0");
     const int64_t bytes = 3 * round_up(n * 8, kBlock);
     if (n > (int64_t)1 << 40 || bytes > sv->arena.size())
@@ -761,6 +854,7 @@ int submit_locked(wxpy_server *sv, int64_t n, double alpha, uint64_t seed, bool 
     r.alpha = alpha;
     r.seed = seed;
     r.src_kind = src_kind;
+    r.by_kernel = by_kernel;
     r.src_x = src_x;
     r.src_y = src_y;
     r.auto_release = auto_release;
@@ -770,6 +864,16 @@ int submit_locked(wxpy_server *sv, int64_t n, double alpha, uint64_t seed, bool 
     ++sv->submitted;
     *ticket = t;
     return WXPY_OK;
+}
+
+// Whether p is memory of device `dev`.
+bool on_device(const void *p, int dev) {
+    cudaPointerAttributes a;
+    if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return a.type == cudaMemoryTypeDevice && a.device == dev;
 }
 
 double percentile(std::vector<double> v, double q) {
@@ -848,8 +952,12 @@ int wxpy_server_submit_data(wxpy_server *sv, int64_t n, double alpha, const doub
     if (sv->cfg.mode == WXPY_SERVE_FUSED)
         return fail(WXPY_EINVAL, "the fused mode generates its inputs: caller data needs the "
                                  "batched or serial mode");
+    // Plain memory of the server's device is read by the inputs launch; any
+    // other source (another device's, say) keeps its own copy.
+    const bool by_kernel = kind == WXPY_SERVE_DATA_DEVICE && sv->cfg.mode == WXPY_SERVE_BATCHED &&
+                           n > 0 && on_device(x, sv->device) && on_device(y, sv->device);
     std::lock_guard<std::mutex> lk(sv->mu);
-    const int st = submit_locked(sv, n, alpha, 0, false, ticket, kind, x, y);
+    const int st = submit_locked(sv, n, alpha, 0, false, ticket, kind, x, y, by_kernel);
     if (st == WXPY_OK) sv->cv_submit.notify_one();
     return st;
 }

@@ -323,3 +323,31 @@ def test_tile_list_grows_for_a_batch_of_short_tiles():
             assert torch.equal(out[s].view(torch.int64), alone(n, a, s).view(torch.int64)), n
     finally:
         wx.wxpy_batch_shape_reset()
+
+
+@pytest.mark.parametrize("shift", [0, 1, 2, 3])
+def test_device_data_at_every_offset_and_length(shift):
+    """Device-data requests copied by the batch's launch: sources at any element
+    offset, lengths around the copy's vectors, passes and tiles, and two
+    requests on one source; resident x and y hold the caller's bits."""
+    lens = [1, 3, 4, 5, 31, 33, 127, 128, 129, 255, 256, 257, 1023, 1025, 8191, 8193, 100003]
+    src = synth.uniform_pm1(77 + shift, synth.TAG_X, sum(lens) + 8)
+    src[3::97] = np.nan
+    src[5::101] = -0.0
+    dev = torch.from_numpy(src).cuda()
+    with Server(budget_bytes=64 << 20, n_streams=2, max_batch=8) as sv:
+        reqs, at = [], 0
+        for n in lens + lens[-2:]:
+            x, y = dev[at + shift: at + shift + n], dev[at: at + n]
+            reqs.append((n, at, sv.submit_data(-1.25, x, y)))
+            at = (at + n) % (len(src) - 100020)
+        for n, at, t in reqs:
+            sv.wait(t, 60.0)
+            _, px, py, pw = sv.result(t)
+            xh, yh = src[at + shift: at + shift + n], src[at: at + n]
+            got = [_from_ptr(p, n).cpu().numpy().view(np.uint64) for p in (px, py, pw)]
+            want = oracle.wxpy(-1.25, np.ascontiguousarray(xh), np.ascontiguousarray(yh))
+            assert np.array_equal(got[0], xh.view(np.uint64))
+            assert np.array_equal(got[1], yh.view(np.uint64))
+            ok = (got[2] == want.view(np.uint64)) | (np.isnan(want) & np.isnan(got[2].view(np.float64)))
+            assert ok.all()
