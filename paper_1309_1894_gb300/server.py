@@ -73,7 +73,8 @@ class Server:
         """Queue a request on the caller's data: float64 1-D contiguous tensors
         x and y (same length), both on the GPU or both in host memory.  They
         must stay alive and unchanged until the request is done or failed."""
-        if x.dtype != y.dtype or str(x.dtype) != "torch.float64":
+        import torch
+        if x.dtype is not torch.float64 or y.dtype is not torch.float64:
             raise TypeError("x and y must be float64 tensors")
         if x.dim() != 1 or y.dim() != 1 or not x.is_contiguous() or not y.is_contiguous():
             raise ValueError("x and y must be contiguous 1-D tensors")
