@@ -168,10 +168,18 @@ __device__ __forceinline__ void wxpy_vec_emu(double alpha, const MulCoef &ca, co
         for (int k = 0; k < VW; ++k)
             p[k] = mul_rn_quick(ca, (uint64_t)__double_as_longlong(x[k]), away);
         if ((int32_t)away < 0) {
+            const uint64_t ab = (uint64_t)__double_as_longlong(alpha);
 #pragma unroll
-            for (int k = 0; k < VW; ++k)  // out of line
-                p[k] = mul_rn_hw_bits((uint64_t)__double_as_longlong(alpha),
-                                      (uint64_t)__double_as_longlong(x[k]));
+            for (int k = 0; k < VW; k += 2) {  // out of line
+                if constexpr (VW == 1) {
+                    p[k] = mul_rn_hw_bits(ab, (uint64_t)__double_as_longlong(x[k]));
+                } else {
+                    const ulonglong2 r = mul2_rn_hw_bits(ab, (uint64_t)__double_as_longlong(x[k]),
+                                                         (uint64_t)__double_as_longlong(x[k + 1]));
+                    p[k] = r.x;
+                    p[k + 1] = r.y;
+                }
+            }
         }
 #pragma unroll
         for (int k = 0; k < VW; ++k) w[k] = __dadd_rn(__longlong_as_double((long long)p[k]), y[k]);

@@ -20,6 +20,14 @@ static __device__ __noinline__ uint64_t mul_rn_hw_bits(uint64_t ua, uint64_t ub)
     return (uint64_t)__double_as_longlong(
         __dmul_rn(__longlong_as_double((long long)ua), __longlong_as_double((long long)ub)));
 }
+
+// RN(a * b) and RN(a * c), one call for the two.
+static __device__ __noinline__ ulonglong2 mul2_rn_hw_bits(uint64_t ua, uint64_t ub, uint64_t uc) {
+    const double a = __longlong_as_double((long long)ua);
+    return make_ulonglong2(
+        (uint64_t)__double_as_longlong(__dmul_rn(a, __longlong_as_double((long long)ub))),
+        (uint64_t)__double_as_longlong(__dmul_rn(a, __longlong_as_double((long long)uc))));
+}
 #endif
 
 // Bits sh .. sh + 31 of the 64-bit word hi:lo, 0 <= sh < 32.

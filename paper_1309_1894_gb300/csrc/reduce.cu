@@ -88,9 +88,10 @@ enum Deal {
 //   kElements  positions 128 warp + lane + 32 q, so that the 8-byte accesses of
 //              a warp are contiguous
 template <int KIND, bool EMU, int DEAL>
-__device__ __forceinline__ void row_terms(const ReduceArgs &a, int64_t row, double (&t)[4]) {
+__device__ __forceinline__ void row_terms(const ReduceArgs &a, int64_t row, double (&t)[4],
+                                          bool &left) {
     if constexpr (DEAL == kVectors) {
-        vector_terms<KIND, EMU, true>(a, row + 4 * threadIdx.x, t);
+        vector_terms<KIND, EMU, true>(a, row + 4 * threadIdx.x, t, left);
     } else if constexpr (DEAL == kShifted) {
         const int64_t i = row + 4 * (int)threadIdx.x - a.shift;
         double x[4], y[4], z[4], w[4];
@@ -108,7 +109,8 @@ __device__ __forceinline__ void row_terms(const ReduceArgs &a, int64_t row, doub
             }
         }
 #pragma unroll
-        for (int q = 0; q < 4; ++q) element<KIND, EMU>(a, x[q], y[q], KIND == 1 ? z[q] : 0.0, w[q], t[q]);
+        for (int q = 0; q < 4; ++q)
+            element<KIND, EMU>(a, x[q], y[q], KIND == 1 ? z[q] : 0.0, w[q], t[q], left);
         if (threadIdx.x != 0) {
             st4(a.w + i, w);
         } else {
@@ -136,7 +138,7 @@ __device__ __forceinline__ void row_terms(const ReduceArgs &a, int64_t row, doub
                 t[g + q] = 0.0;
                 if (i < a.n) {
                     double w;
-                    element<KIND, EMU>(a, x[q], y[q], KIND == 1 ? z[q] : 0.0, w, t[g + q]);
+                    element<KIND, EMU>(a, x[q], y[q], KIND == 1 ? z[q] : 0.0, w, t[g + q], left);
                     a.w[i] = w;
                 }
             }
@@ -147,12 +149,14 @@ __device__ __forceinline__ void row_terms(const ReduceArgs &a, int64_t row, doub
 // The sum of tile `tile`; valid in thread 0.  red: 1024 doubles of shared memory,
 // the node of position p of the rows at red[p]; node: 128 doubles.
 // SUML (norm2 only): the first SUML of the three in-thread tree levels run as
-// integer-pipeline sums of non-negative values.
+// integer-pipeline sums of non-negative values.  *left: the threads with an
+// element off the integer products' fast path.
 template <int KIND, int DEAL, bool EMU, int SUML = 0>
-__device__ double tile_sum(const ReduceArgs &a, int64_t tile, double *red, double *node) {
+__device__ double tile_sum(const ReduceArgs &a, int64_t tile, double *red, double *node, int *left) {
     static_assert(SUML == 0 || KIND == 0, "integer tree sums need non-negative terms");
     const int t = threadIdx.x, lane = t & 31;
     const int64_t t0 = tile * kTile;
+    bool mine = false;
     // bits 12..10: rows j and j + 4 (bit 12), then j and j + 2 (bit 11), then bit 10,
     // with j in the order 0, 2, 1, 3: each pair (0, 2), (1, 3) is summed as soon as
     // both are formed, so at most two level-1 vectors are live
@@ -165,8 +169,8 @@ __device__ double tile_sum(const ReduceArgs &a, int64_t tile, double *red, doubl
         for (int m = 0; m < 2; ++m) {
             const int j = h + 2 * m;
             double lo[4], hi[4];
-            row_terms<KIND, EMU, DEAL>(a, t0 + 1024 * j, lo);
-            row_terms<KIND, EMU, DEAL>(a, t0 + 1024 * (j + 4), hi);
+            row_terms<KIND, EMU, DEAL>(a, t0 + 1024 * j, lo, mine);
+            row_terms<KIND, EMU, DEAL>(a, t0 + 1024 * (j + 4), hi, mine);
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
                 rp[q] = rc[q];
@@ -193,7 +197,7 @@ __device__ double tile_sum(const ReduceArgs &a, int64_t tile, double *red, doubl
 #pragma unroll
         for (int q = 0; q < 4; ++q) red[128 * (t >> 5) + lane + 32 * q] = v[q];
     }
-    __syncthreads();
+    *left = __syncthreads_count(mine);
     double s = 0.0;
     if (t < 128) {
         node[t] = tree8<128>(red + t);  // bits 9..7
@@ -222,12 +226,19 @@ __global__ void __launch_bounds__(kThreads, 4) wxpy_reduce_kernel(const ReduceAr
     pdl_enter();
     const int64_t full = a.n / kTile;        // tiles with every element present
     unsigned slot = (blockIdx.x * 7u) & 15u;  // block-uniform rotation of the pipe choice
-    int turn = 0;
+    int turn = 0, fp64 = 0;
     for (int64_t tile = blockIdx.x; tile < a.ntiles; tile += gridDim.x, turn ^= 1) {
         double s;
-        if (tile >= full) s = tile_sum<KIND, kElements, false>(a, tile, red[turn], node);
-        else if ((int)slot < a.mul_sixteenths) s = tile_sum<KIND, DEAL, true, SUML>(a, tile, red[turn], node);
-        else s = tile_sum<KIND, DEAL, false, SUML>(a, tile, red[turn], node);
+        int left = 0;
+        if (tile >= full) s = tile_sum<KIND, kElements, false>(a, tile, red[turn], node, &left);
+        else if ((int)slot < a.mul_sixteenths && fp64 == 0)
+            s = tile_sum<KIND, DEAL, true, SUML>(a, tile, red[turn], node, &left);
+        else s = tile_sum<KIND, DEAL, false, SUML>(a, tile, red[turn], node, &left);
+        // Data that keeps leaving the fast path (zeros, say) pays for both kinds of
+        // product: after a tile where a quarter of the threads did, the block takes
+        // FP64 products for sixteen tiles.  Every seventh element zero, n = 2^26:
+        // 552 us against 683 without, and 576 before with a test per product.
+        fp64 = left > kThreads / 4 ? 16 : fp64 > 0 ? fp64 - 1 : 0;
         if (threadIdx.x == 0) a.partial[tile] = s;
         slot = (slot + 1u) & 15u;
     }

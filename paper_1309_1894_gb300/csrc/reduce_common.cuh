@@ -83,9 +83,10 @@ static __device__ __noinline__ ulonglong2 element_hw_bits(uint64_t alpha, uint64
 // with one fallback test for the element.  At n = 2^26 (GB300) the windowed
 // products with one test run norm2 / dot at 0.75 / 0.89 of the measured peak,
 // against 0.72 / 0.84 with the fully checked products and a test for each.
+// `left` is set when the element left the fast path.
 template <int KIND, bool EMU>
 __device__ __forceinline__ void element(const ReduceArgs &a, double x, double y, double z,
-                                        double &w, double &t) {
+                                        double &w, double &t, bool &left) {
     if constexpr (EMU) {
         uint32_t away = 0;
         bool slow = false;
@@ -97,11 +98,19 @@ __device__ __forceinline__ void element(const ReduceArgs &a, double x, double y,
                 element_hw_bits<KIND>(bits_of(a.alpha), bits_of(x), bits_of(y), bits_of(z));
             w = double_of(r.x);
             t = double_of(r.y);
+            left = true;
         }
     } else {
         w = __dadd_rn(__dmul_rn(a.alpha, x), y);
         t = __dmul_rn(w, KIND == 0 ? w : z);
     }
+}
+
+template <int KIND, bool EMU>
+__device__ __forceinline__ void element(const ReduceArgs &a, double x, double y, double z,
+                                        double &w, double &t) {
+    bool left;
+    element<KIND, EMU>(a, x, y, z, w, t, left);
 }
 
 // Coherent evict-first 32-byte accesses: w may be one of the inputs.
@@ -121,14 +130,16 @@ __device__ __forceinline__ void st4(double *p, const double (&v)[4]) {
 // co-aligned vector of every operand; else element by element with bounds,
 // +0 terms past n.
 template <int KIND, bool EMU, bool VEC>
-__device__ __forceinline__ void vector_terms(const ReduceArgs &a, int64_t base, double (&t)[4]) {
+__device__ __forceinline__ void vector_terms(const ReduceArgs &a, int64_t base, double (&t)[4],
+                                             bool &left) {
     if constexpr (VEC) {
         double x[4], y[4], z[4], w[4];
         ld4(a.x + base, x);
         ld4(a.y + base, y);
         if constexpr (KIND == 1) ld4(a.z + base, z);
 #pragma unroll
-        for (int q = 0; q < 4; ++q) element<KIND, EMU>(a, x[q], y[q], KIND == 1 ? z[q] : 0.0, w[q], t[q]);
+        for (int q = 0; q < 4; ++q)
+            element<KIND, EMU>(a, x[q], y[q], KIND == 1 ? z[q] : 0.0, w[q], t[q], left);
         st4(a.w + base, w);
     } else {
 #pragma unroll
@@ -144,6 +155,12 @@ __device__ __forceinline__ void vector_terms(const ReduceArgs &a, int64_t base, 
             }
         }
     }
+}
+
+template <int KIND, bool EMU, bool VEC>
+__device__ __forceinline__ void vector_terms(const ReduceArgs &a, int64_t base, double (&t)[4]) {
+    bool left;
+    vector_terms<KIND, EMU, VEC>(a, base, t, left);
 }
 
 // Bits 6..0 of a tile's tree, by one warp, from the 128 node values that bits

@@ -369,9 +369,10 @@ __device__ __noinline__ void staged_tile_fp64(double d0, double d1, double d2, d
 // that the compiler can interleave (one element's FP64 sums with another's
 // integer products); if any product left the fast path, the thread's
 // elements are recomputed in FP64 and written again (nothing reads them
-// before the kernel ends, and the stage still holds the inputs).
+// before the kernel ends, and the stage still holds the inputs).  Returns
+// whether that happened.
 template <class Op, int PM, int TE>
-__device__ __forceinline__ void staged_tile(const Coefs &cf, const double *sb, double *out, int len,
+__device__ __forceinline__ bool staged_tile(const Coefs &cf, const double *sb, double *out, int len,
                                             int c) {
     constexpr int NIN = Op::kIn;
     uint32_t away = 0;
@@ -399,6 +400,7 @@ __device__ __forceinline__ void staged_tile(const Coefs &cf, const double *sb, d
             staged_tile_fp64<Op, TE>(cf.d[0], cf.d[1], cf.d[2], cf.d[3], cf.d[4], cf.d[5], cf.d[6],
                                      cf.d[7], sb, out, len, c);
     }
+    return (int32_t)away < 0;
 }
 
 template <class Op>
@@ -461,7 +463,7 @@ __global__ void __launch_bounds__(kStagedThreads, StageShape<Op::kIn>::kMinBlock
         }
     } else {
         unsigned slot = (warp * 5u + blockIdx.x * 3u) & 15u;
-        int i = 0;
+        int i = 0, fp64 = 0;
         for (int64_t t = blockIdx.x; t < ntiles; t += gridDim.x, ++i) {
             const int s = i % S;
             if (!mbar_wait(smem_addr(&full[s]), (i / S) & 1)) {
@@ -472,9 +474,15 @@ __global__ void __launch_bounds__(kStagedThreads, StageShape<Op::kIn>::kMinBlock
             const int len = (int)(body - e0 < TE ? body - e0 : TE);
             const double *sb = ring + (size_t)s * NIN * TE;
             double *out = a.out + a.head + e0;
-            if ((int)slot < a.pm) staged_tile<Op, 1, TE>(a.cf, sb, out, len, threadIdx.x);
+            // Data that keeps leaving the fast path (zeros, say) pays for both
+            // kinds of product: after a tile where a quarter of the lanes did,
+            // the warp takes FP64 products for sixteen tiles.  Every seventh
+            // element zero, maxpy with 4 terms, n = 2^26 (GB300): 1065 us
+            // against 1557.
+            bool left = false;
+            if ((int)slot < a.pm && fp64 == 0) left = staged_tile<Op, 1, TE>(a.cf, sb, out, len, threadIdx.x);
             else staged_tile<Op, 0, TE>(a.cf, sb, out, len, threadIdx.x);
-            __syncwarp();
+            fp64 = __popc(__ballot_sync(0xffffffffu, left)) > 8 ? 16 : fp64 > 0 ? fp64 - 1 : 0;
             if (lane == 0) mbar_arrive(smem_addr(&empty[s]));
             slot = (slot + 1u) & 15u;
         }
