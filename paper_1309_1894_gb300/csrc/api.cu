@@ -337,7 +337,7 @@ int launch_piece(const Variant &v, const DeviceProps &dp, int xy, int64_t n, dou
     const int64_t head = std::min<int64_t>((vw - off) % vw, n);
     uint64_t ab;
     std::memcpy(&ab, &alpha, 8);
-    SingleArgs a{x, y, w, alpha, n, head, (n - head) / vw, mul_coef_of(ab)};
+    SingleArgs a{x, y, w, alpha, n, head, (n - head) / vw, mul_coef_of(ab), false};
     const int u_idx = v.unroll == 1 ? 0 : v.unroll == 2 ? 1 : v.unroll == 4 ? 2 : 3;
     const int rx = rel32(x, w), ry = rel32(y, w);
     // 32-byte variants on pointers whose offsets disagree modulo 32 bytes run
@@ -355,6 +355,12 @@ int launch_piece(const Variant &v, const DeviceProps &dp, int xy, int64_t n, dou
     int64_t grid = need;
     if (v.blocks_per_sm > 0) grid = std::min<int64_t>(need, (int64_t)v.blocks_per_sm * dp.sm_count);
     if (grid > 0x7fffffff) return fail(WXPY_EINVAL, "grid too large for n = %lld", (long long)n);
+    // A grid that fills at most a quarter of the GPU's threads ends at once: the
+    // next launch gains nothing by starting with it, and loses if its blocks are
+    // few and long and spread unevenly over the SMs that are still taken (wxpy,
+    // axpbypcz, norm2 and dot in turn on 131072 elements: 16.5 us a round when it
+    // starts early, 15.0 late; larger grids hide its launch, 2^20 4.5 against 5.1).
+    a.late = grid * threads <= (int64_t)dp.sm_count * 512;
     cudaError_t e = set_carveout(ent.func, dp.device, v.carveout);
     if (e != cudaSuccess) return fail_cuda(e, "cudaFuncSetAttribute(carveout)");
     e = injected_launch_error();
@@ -605,7 +611,7 @@ int wxpy_reference(int64_t n, double alpha, const double *x, const double *y, do
     if (st != WXPY_OK || n == 0) return st;
     const int64_t grid = (n + 255) / 256;
     if (grid > 0x7fffffff) return fail(WXPY_EINVAL, "n too large for the reference variant");
-    SingleArgs a{x, y, w, alpha, n, 0, 0, MulCoef{}};
+    SingleArgs a{x, y, w, alpha, n, 0, 0, MulCoef{}, false};
     cudaError_t e = injected_launch_error();
     if (e == cudaSuccess) e = launch_reference((unsigned)grid, 256u, a, (cudaStream_t)stream);
     if (e != cudaSuccess) return fail_cuda(e, "reference kernel launch");

@@ -41,6 +41,7 @@ struct SingleArgs {
     int64_t head;      // scalar elements before the vector body (< VW)
     int64_t nchunks;   // vector body: chunks of VW elements starting at `head`
     MulCoef ca;        // alpha split for the integer-pipeline product (EMU == 3)
+    bool late;         // let the next launch start after this grid's passes, not before
 };
 
 template <int VW, int CACHE>
@@ -206,9 +207,15 @@ constexpr int max_threads() {
 // Nothing is read or written before the wait, so any dependence between calls
 // (w of one call is x of the next) is kept; only L2 prefetches are issued
 // ahead of it (prefetch_first_pass).
-__device__ __forceinline__ void pdl_enter() {
-    asm volatile("griddepcontrol.wait;" ::: "memory");
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+__device__ __forceinline__ void pdl_trigger() {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+__device__ __forceinline__ void pdl_enter() {
+    pdl_wait();
+    pdl_trigger();
 }
 
 // Before the wait: the L2 lines of this thread's first pass of x and y are
@@ -232,7 +239,8 @@ template <int VW, int U, int GS, int CACHE, bool XY, int EMU>
 __global__ void __launch_bounds__(max_threads<VW, U, GS, XY, EMU>())
     wxpy_single_kernel(const SingleArgs a) {
     prefetch_first_pass<VW, U, XY>(a, (int64_t)blockIdx.x * blockDim.x * U + threadIdx.x, blockDim.x);
-    pdl_enter();
+    pdl_wait();
+    if (!a.late) pdl_trigger();
     const int64_t tpb = blockDim.x;
     if constexpr (GS == 0) {
         const int64_t c0 = (int64_t)blockIdx.x * tpb * U + threadIdx.x;
@@ -243,6 +251,7 @@ __global__ void __launch_bounds__(max_threads<VW, U, GS, XY, EMU>())
              c0 += stride)
             wxpy_pass<VW, U, CACHE, XY, EMU>(a, c0, tpb);
     }
+    if (a.late) pdl_trigger();
     wxpy_edges<CACHE, XY>(a, VW);
 }
 
