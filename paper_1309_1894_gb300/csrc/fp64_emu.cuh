@@ -102,6 +102,78 @@ WX_EMU_FN uint64_t add_rn_with(uint64_t ua, uint64_t ub, Hw hw) {
     return bits;
 }
 
+// RN(a + b) with the cheapest checks, for kernels that move a few of many sums:
+// ORs into `away` a word whose top bit is set when the operands leave the fast
+// path (the bits are then meaningless): the larger magnitude's exponent field
+// outside [512, 1535], a gap of more than 30 between the two (zeros always),
+// or a difference that cancels 20 bits or more.
+//
+// Method, in 32-bit words.  The larger operand's significand, hidden bit at bit
+// 19 of the top word, and the smaller one's shifted right by the gap are held
+// exactly in 96 bits; they are added, or subtracted as a two's complement when
+// the signs differ.  The sum's leading bit is at bit 20 or below, so one left
+// shift puts it there.  The lowest word is then all that is rounded away, and
+// adding one half to it carries into the significand exactly when it is at
+// least one half; it becomes 0 exactly on a tie, which clears the lowest bit.
+WX_EMU_FN uint64_t add_rn_quick(uint64_t ua, uint64_t ub, uint32_t &away) {
+    const uint32_t ah = (uint32_t)(ua >> 32), al = (uint32_t)ua;
+    const uint32_t bh = (uint32_t)(ub >> 32), bl = (uint32_t)ub;
+    const uint32_t A = ah & 0x7FFFFFFFu, B = bh & 0x7FFFFFFFu;
+    const bool b_big = A < B;
+    const uint32_t H = b_big ? B : A, L = b_big ? A : B;
+    const uint32_t hl = b_big ? bl : al, ll = b_big ? al : bl, hh = b_big ? bh : ah;
+    const uint32_t x = H - (L & 0x7FF00000u);  // gap << 20, and fraction bits below
+    const uint32_t d = (x + 0x100000u) >> 20;  // gap + 1
+    const uint32_t hm = (H & 0xFFFFFu) | 0x100000u, lm = (L & 0xFFFFFu) | 0x100000u;
+    const uint32_t m = (uint32_t)((int32_t)(ah ^ bh) >> 31);
+    const uint32_t t2 = lm >> (d & 31u), t1 = funnel_r(ll, lm, d & 31u), t0 = funnel_r(0u, ll, d & 31u);
+    uint32_t s2, s1, s0;
+#ifdef __CUDA_ARCH__
+    uint32_t drop;
+    asm("add.cc.u32 %3, %4, 1;\n\t"  // carry in: 1 to subtract
+        "addc.cc.u32 %0, %5, %6;\n\t"
+        "addc.cc.u32 %1, %7, %8;\n\t"
+        "addc.u32 %2, %9, %10;"
+        : "=r"(s0), "=r"(s1), "=r"(s2), "=r"(drop)
+        : "r"(m), "r"(hl << 31), "r"(t0 ^ m), "r"(funnel_r(hl, hm, 1u)), "r"(t1 ^ m), "r"(hm >> 1),
+          "r"(t2 ^ m));
+    const int lz = __clz((int)s2);
+#else
+    const uint64_t w0 = (uint64_t)(hl << 31) + (t0 ^ m) + (m & 1u);
+    const uint64_t w1 = (uint64_t)funnel_r(hl, hm, 1u) + (t1 ^ m) + (w0 >> 32);
+    s0 = (uint32_t)w0, s1 = (uint32_t)w1, s2 = (hm >> 1) + (t2 ^ m) + (uint32_t)(w1 >> 32);
+    const int lz = s2 ? __builtin_clz(s2) : 32;
+#endif
+    away |= ((H << 1) - (512u << 21)) | ((31u << 20) - 1u - x) | (s2 - 1u);
+    const uint32_t n = (uint32_t)lz - 11u;  // left shift: leading bit to bit 20
+    const uint32_t r = 32u - n;
+    // left funnels as right ones of the neighbouring words (n in 0..20)
+#ifdef __CUDA_ARCH__
+    const uint32_t o2 = __funnelshift_l(s1, s2, n), o1 = __funnelshift_l(s0, s1, n);
+    const uint32_t g = s0 << (n & 31u);
+    (void)r;
+#else
+    const uint32_t o2 = n ? (s2 << n) | (uint32_t)((uint64_t)s1 >> (r & 63u)) : s2;
+    const uint32_t o1 = n ? (s1 << n) | (uint32_t)((uint64_t)s0 >> (r & 63u)) : s1;
+    const uint32_t g = s0 << (n & 31u);
+#endif
+    const uint32_t hw = (hh & 0xFFF00000u) + (o2 - (n << 20));
+    uint32_t gs, lo, hi;
+#ifdef __CUDA_ARCH__
+    asm("add.cc.u32 %0, %3, 0x80000000;\n\t"
+        "addc.cc.u32 %1, %4, 0;\n\t"
+        "addc.u32 %2, %5, 0;"
+        : "=r"(gs), "=r"(lo), "=r"(hi)
+        : "r"(g), "r"(o1), "r"(hw));
+#else
+    gs = g + 0x80000000u;
+    lo = o1 + (g >> 31);
+    hi = hw + (uint32_t)(lo < o1);
+#endif
+    lo = gs == 0u ? lo & ~1u : lo;
+    return ((uint64_t)hi << 32) | lo;
+}
+
 #ifdef __CUDACC__
 
 // The hardware sum for the rare operands the integer path leaves out, on bit

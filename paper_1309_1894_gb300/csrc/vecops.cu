@@ -28,7 +28,8 @@
 // computes all of its products in the integer pipeline, the rest in FP64;
 // the choice is uniform across the warp (no divergence) and rotates with the
 // iteration, so every SM sub-partition sees the same mix.  Sums can move too
-// (add offload 1: every other one, 2: all).  Every split gives the same bits.
+// (add offload 1: every other one, 2: all; 0: none, but for one or two of a wide
+// maxpy group's, see integer_sums).  Every split gives the same bits.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -117,7 +118,7 @@ struct AxpbyOp {
         products<PM>(c, e, p);
         return add_sel<OFF>(p[0], p[1], 1);
     }
-    __device__ __forceinline__ static double apply_fast(const Coefs &c, const double (&e)[kIn],
+    __device__ __forceinline__ static double apply_fast(const Coefs &c, const double (&e)[kIn], int,
                                                         uint32_t &away) {
         double p[2];
         products_fast(c, e, p, away);
@@ -136,7 +137,7 @@ struct AxpbypczOp {
         const double s1 = add_sel<OFF>(p[0], p[1], 1);
         return add_sel<OFF>(s1, p[2], OFF == 1 ? 0 : 1);
     }
-    __device__ __forceinline__ static double apply_fast(const Coefs &c, const double (&e)[kIn],
+    __device__ __forceinline__ static double apply_fast(const Coefs &c, const double (&e)[kIn], int,
                                                         uint32_t &away) {
         double p[3];
         products_fast(c, e, p, away);
@@ -144,6 +145,21 @@ struct AxpbypczOp {
         return add_sel<OFF>(s1, p[2], OFF == 1 ? 0 : 1);
     }
 };
+
+// Which of a maxpy group's sums (bit j: the one that adds term j) run in the
+// integer pipeline on the staged kernel's fast path, for the two elements of a
+// pair.  The FP64 pipeline does 1.7 sums per clock and SM whatever the code
+// (5.0e11/s), so m sums per 8(m + 2) bytes hold these kernels to 0.92 of the HBM
+// peak with 4 terms and 0.76 with 8; an integer sum is about 45 ALU operations,
+// and there is ALU time left for one or two in sixteen.  n = 2^26 (GB300), us
+// with none / these: 4 terms 532 / 502, 5 660 / 611, 6 802 / 751, 7 929 / 856,
+// 8 1056 / 973; with 3 terms one of six is slower, 408 / 414.
+template <int M>
+__device__ constexpr unsigned integer_sums(int q) {
+    constexpr unsigned k[7][2] = {{0, 0}, {0, 0}, {0, 1u << 2}, {0, 1u << 3},
+                                  {0, 1u << 2}, {1u << 0, 1u << 3}, {1u << 3, 1u << 3}};
+    return k[M - 2][q];
+}
 
 template <int M, int OFF>
 struct MaxpyOp {
@@ -158,13 +174,18 @@ struct MaxpyOp {
         for (int j = 0; j < M; ++j) acc = add_sel<OFF>(acc, p[j], j + 1);
         return acc;
     }
-    __device__ __forceinline__ static double apply_fast(const Coefs &c, const double (&e)[kIn],
+    __device__ __forceinline__ static double apply_fast(const Coefs &c, const double (&e)[kIn], int q,
                                                         uint32_t &away) {
         double p[M];
         products_fast(c, e, p, away);
         double acc = e[0];
 #pragma unroll
-        for (int j = 0; j < M; ++j) acc = add_sel<OFF>(acc, p[j], j + 1);
+        for (int j = 0; j < M; ++j) {
+            if (OFF == 0 && (integer_sums<M>(q) >> j & 1u))
+                acc = double_of(add_rn_quick(j ? opaque_bits(acc) : bits_of(acc), bits_of(p[j]), away));
+            else
+                acc = add_sel<OFF>(acc, p[j], j + 1);
+        }
         return acc;
     }
 };
@@ -389,7 +410,7 @@ __device__ __forceinline__ bool staged_tile(const Coefs &cf, const double *sb, d
                 double e[NIN];
 #pragma unroll
                 for (int k = 0; k < NIN; ++k) e[k] = v[k][q];
-                if constexpr (PM == 1) r[q] = Op::apply_fast(cf, e, away);
+                if constexpr (PM == 1) r[q] = Op::apply_fast(cf, e, q, away);
                 else r[q] = Op::template apply<0>(cf, e);
             }
             st_global_v2_cs(out + p, r[0], r[1]);

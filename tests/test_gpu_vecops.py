@@ -338,3 +338,27 @@ def test_dependent_calls_back_to_back(n, off):
     for g, h in ((gx, xh), (gy, yh), (gz, zh), (gw, wh)):
         assert same(g.t, h)
         g.check()
+
+
+@pytest.mark.parametrize("special", [False, True])
+@pytest.mark.parametrize("m", [2, 4, 5, 6, 7, 8])
+def test_maxpy_integer_sums(m, special):
+    """Groups whose sums partly run in the integer pipeline: sums of every
+    exponent gap and sign, ties and deep cancellations (terms that undo each
+    other), through the whole range of a tile."""
+    n = 70001
+    rng = np.random.default_rng(60 + m)
+    yh = vals(5 * m, n, special)
+    xsh = [vals(6 * m + j, n, special) for j in range(m)]
+    if not special:
+        for j in range(m):
+            xsh[j] *= np.ldexp(1.0, rng.integers(-40, 3, n))
+        xsh[1] = np.where(rng.random(n) < 0.3, -xsh[0], xsh[1])
+        xsh[m - 1][::5] = np.round(xsh[m - 1][::5] * 64) / 64 * 2.0 ** -45
+    al = [1.0, 1.0] + list(synth.uniform_pm2(9 + m, synth.TAG_ALPHA, m)[2:])
+    gy, gxs = Guarded(n, 8).set(yh), [Guarded(n, 8).set(x) for x in xsh]
+    wx.wxpy_maxpy(al, [g.t for g in gxs], gy.t)
+    torch.cuda.synchronize()
+    assert same(gy.t, oracle.maxpy(al, xsh, yh))
+    for g in [gy] + gxs:
+        g.check()
