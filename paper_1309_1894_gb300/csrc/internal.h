@@ -142,7 +142,7 @@ struct VecPipes {
 int vecops_inputs(int cls);
 int vecops_run(int cls, int64_t n, const double *coef, const double *const *in, double *out,
                VecPipes p, cudaStream_t s);
-VecPipes vecops_default(int cls);
+VecPipes vecops_default(int cls, int64_t n);
 bool vecops_tuned_load(int cls, VecPipes *p);
 void vecops_tuned_store(int cls, const VecPipes *p);  // nullptr clears
 

@@ -161,10 +161,12 @@ __device__ __forceinline__ void wxpy_pass(const SingleArgs &a, int64_t c0, int64
 }
 
 // Head (elements [0, head)) and tail (elements after the vector body), at most
-// VW-1 each, done with scalar accesses by threads 0..7 of block 0.
+// VW-1 each, done with scalar accesses by threads 0..7 of the last block -- in a
+// one-shot grid a block of its own, so that no other block has a second memory
+// latency to wait for.
 template <int CACHE, bool XY>
 __device__ __forceinline__ void wxpy_edges(const SingleArgs &a, int64_t vw) {
-    if (blockIdx.x != 0 || threadIdx.x >= 8) return;
+    if (blockIdx.x != gridDim.x - 1 || threadIdx.x >= 8) return;
     const int t = threadIdx.x;
     const int64_t body_end = a.head + a.nchunks * vw;
     int64_t e = -1;

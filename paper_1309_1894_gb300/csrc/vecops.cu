@@ -56,6 +56,7 @@ struct EwArgs {
     double *out;
     int64_t n, head, nch;  // nch: 4-element chunks (32-byte path) or elements after `head`
     int pm;                // sixteenths of warp iterations whose products run in the integer pipeline
+    unsigned odd;          // staged path: inputs an odd number of elements off the output's 16 bytes
     int64_t drop_tile;     // debug: the producer stops before this tile (-1: never)
     Coefs cf;
 };
@@ -111,7 +112,7 @@ __device__ __forceinline__ void products_fast(const Coefs &c, const double (&e)[
 template <int OFF>
 struct AxpbyOp {
     static constexpr int kIn = 2;  // x, y
-    static constexpr bool kStaged = true;
+    static constexpr bool kStaged = true, kDefaultSums = OFF == 0;
     template <int PM>
     __device__ __forceinline__ static double apply(const Coefs &c, const double (&e)[kIn]) {
         double p[2];
@@ -129,7 +130,7 @@ struct AxpbyOp {
 template <int OFF>
 struct AxpbypczOp {
     static constexpr int kIn = 3;  // x, y, z
-    static constexpr bool kStaged = true;
+    static constexpr bool kStaged = true, kDefaultSums = OFF == 0;
     template <int PM>
     __device__ __forceinline__ static double apply(const Coefs &c, const double (&e)[kIn]) {
         double p[3];
@@ -164,7 +165,7 @@ __device__ constexpr unsigned integer_sums(int q) {
 template <int M, int OFF>
 struct MaxpyOp {
     static constexpr int kIn = M + 1;  // y, x0 .. x_{M-1}
-    static constexpr bool kStaged = true;
+    static constexpr bool kStaged = true, kDefaultSums = OFF == 0;
     template <int PM>
     __device__ __forceinline__ static double apply(const Coefs &c, const double (&e)[kIn]) {
         double p[M];
@@ -192,7 +193,7 @@ struct MaxpyOp {
 
 struct PmultOp {
     static constexpr int kIn = 2;
-    static constexpr bool kStaged = false;
+    static constexpr bool kStaged = false, kDefaultSums = false;
     template <int PM>
     __device__ __forceinline__ static double apply(const Coefs &, const double (&e)[kIn]) {
         if constexpr (PM == 1) return double_of(mul_rn_bits(bits_of(e[0]), bits_of(e[1])));
@@ -301,7 +302,8 @@ __global__ void __launch_bounds__(256) ew_direct_kernel(const EwArgs<Op::kIn> a)
         else direct_iter<Op, 0>(a, c0, tpb);
         slot = (slot + 1u) & 15u;
     }
-    if (blockIdx.x == 0 && threadIdx.x < 8) {
+    // head and tail by the last block (one of its own in a short call)
+    if (blockIdx.x == gridDim.x - 1 && threadIdx.x < 8) {
         const int t = threadIdx.x;
         const int64_t body_end = a.head + a.nch * 4;
         if (t < 4 && t < a.head) ew_scalar<Op>(a, t);
@@ -334,17 +336,26 @@ constexpr int kStagedThreads = 32 * (kConsumerWarps + 1);
 // 2: consumer); read and cleared by wxpy_vecops_status().
 __device__ unsigned int g_vec_fault;
 
-template <int NIN>
+// EPT: elements per consumer thread per tile.  MIXED: inputs whose offset from
+// the output is odd in elements (see staged_pair), with room for the element
+// before and after a tile.
+template <int NIN, int EPT, bool MIXED>
 struct StageShape {
-    static constexpr int kEpt = NIN <= 3 ? 4 : 2;  // elements per consumer thread per tile
-    static constexpr int kTile = 256 * kEpt;
-    static constexpr int kTileBytes = NIN * kTile * 8;
+    static constexpr int kTile = 256 * EPT;
+    static constexpr int kStride = kTile + (MIXED ? 2 : 0);  // of an input in a stage
+    static constexpr int kTileBytes = NIN * kStride * 8;
     static constexpr int kStages = std::max(2, std::min(4, (72 * 1024) / kTileBytes));
     static constexpr int kSmem = kStages * kTileBytes;
     // three resident blocks for the widest maxpy groups (a register cap of 75
     // measured 6 % faster there; narrower operations gain nothing from it)
     static constexpr int kMinBlocks = NIN >= 7 ? 3 : 2;
 };
+
+// The usual tile; calls whose tiles of this length would not give every SM one
+// take half of it where there is the choice (65536 elements, GB300: axpbypcz
+// 2.25 -> 1.84 us, axpby 1.94 -> 1.69; 262144 and more gain nothing).
+template <int NIN>
+constexpr int kEpt = NIN <= 3 ? 4 : 2;
 
 __device__ __forceinline__ void ld_shared_v2(const double *p, double &a, double &b) {
     asm volatile("ld.shared.v2.f64 {%0,%1}, [%2];" : "=d"(a), "=d"(b) : "r"(smem_addr(p)));
@@ -354,35 +365,71 @@ __device__ __forceinline__ void st_global_v2_cs(double *p, double a, double b) {
     asm volatile("st.global.cs.v2.f64 [%0], {%1,%2};" ::"l"(p), "d"(a), "d"(b) : "memory");
 }
 
+__device__ __forceinline__ double ld_shared_1(const double *p) {
+    double v;
+    asm volatile("ld.shared.f64 %0, [%1];" : "=d"(v) : "r"(smem_addr(p)));
+    return v;
+}
+
+// The j-th two elements of consumer thread c in a tile of `len`: elements 2c + 512 j
+// and the next one, in 16-byte accesses; or, MIXED, elements c + 512 j and 256
+// further, in single ones.  A bulk copy must start on a 16-byte boundary, so an
+// input whose offset from the output is an odd number of elements is copied from
+// one element earlier (bit k of `odd`), and its 16-byte pairs would straddle the
+// output's; single accesses, 256 contiguous bytes a warp, are free of bank
+// conflicts at either offset.  Returns whether the first of the two is there;
+// the second is too, but for MIXED where it says so.
+template <class Op, int PM, int EPT, bool MIXED>
+__device__ __forceinline__ void staged_pair(const Coefs &cf, const double *sb, double *out, int len,
+                                            int c, int j, unsigned odd, uint32_t &away) {
+    constexpr int NIN = Op::kIn;
+    using SS = StageShape<NIN, EPT, MIXED>;
+    const int p = (MIXED ? c : 2 * c) + 512 * j;
+    if (p >= len) return;
+    double v[NIN][2];
+#pragma unroll
+    for (int k = 0; k < NIN; ++k) {
+        if constexpr (MIXED) {
+            const double *in = sb + k * SS::kStride + (odd >> k & 1u) + p;
+            v[k][0] = ld_shared_1(in);
+            v[k][1] = p + 256 < len ? ld_shared_1(in + 256) : 1.0;
+        } else {
+            ld_shared_v2(sb + k * SS::kStride + p, v[k][0], v[k][1]);
+        }
+    }
+    double r[2];
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+        double e[NIN];
+#pragma unroll
+        for (int k = 0; k < NIN; ++k) e[k] = v[k][q];
+        if constexpr (PM == 1) r[q] = Op::apply_fast(cf, e, q, away);
+        else r[q] = Op::template apply<0>(cf, e);
+    }
+    if constexpr (MIXED) {
+        const double r0[1] = {r[0]}, r1[1] = {r[1]};
+        st_vec<1, 2>(out + p, r0);
+        if (p + 256 < len) st_vec<1, 2>(out + p + 256, r1);
+    } else {
+        st_global_v2_cs(out + p, r[0], r[1]);
+    }
+}
+
 // This thread's elements of a tile, every product in FP64 (PM 0), from the
 // stage, which is still held; d: the launch's coefficients.  Out of line: it
 // runs only when an integer-pipeline product left its fast path, and inlined
 // it would be issued, predicated off, on the FP64 pipeline for every tile.
-template <class Op, int TE>
+template <class Op, int EPT, bool MIXED>
 __device__ __noinline__ void staged_tile_fp64(double d0, double d1, double d2, double d3,
                                               double d4, double d5, double d6, double d7,
-                                              const double *sb, double *out, int len, int c) {
-    constexpr int NIN = Op::kIn;
+                                              const double *sb, double *out, int len, int c,
+                                              unsigned odd) {
     Coefs cf;  // the FP64 products read only the doubles
     cf.d[0] = d0, cf.d[1] = d1, cf.d[2] = d2, cf.d[3] = d3;
     cf.d[4] = d4, cf.d[5] = d5, cf.d[6] = d6, cf.d[7] = d7;
-    for (int j = 0; j < TE / 512; ++j) {
-        const int p = 2 * c + 512 * j;
-        if (p < len) {
-            double v[NIN][2];
-#pragma unroll
-            for (int k = 0; k < NIN; ++k) ld_shared_v2(sb + k * TE + p, v[k][0], v[k][1]);
-            double r[2];
-#pragma unroll
-            for (int q = 0; q < 2; ++q) {
-                double e[NIN];
-#pragma unroll
-                for (int k = 0; k < NIN; ++k) e[k] = v[k][q];
-                r[q] = Op::template apply<0>(cf, e);
-            }
-            st_global_v2_cs(out + p, r[0], r[1]);
-        }
-    }
+    uint32_t none = 0;
+    for (int j = 0; j < EPT / 2; ++j)
+        staged_pair<Op, 0, EPT, MIXED>(cf, sb, out, len, c, j, odd, none);
 }
 
 // PM = 1: the integer-pipeline products take their fast path with no test
@@ -392,45 +439,28 @@ __device__ __noinline__ void staged_tile_fp64(double d0, double d1, double d2, d
 // elements are recomputed in FP64 and written again (nothing reads them
 // before the kernel ends, and the stage still holds the inputs).  Returns
 // whether that happened.
-template <class Op, int PM, int TE>
+template <class Op, int PM, int EPT, bool MIXED>
 __device__ __forceinline__ bool staged_tile(const Coefs &cf, const double *sb, double *out, int len,
-                                            int c) {
-    constexpr int NIN = Op::kIn;
+                                            int c, unsigned odd) {
     uint32_t away = 0;
 #pragma unroll
-    for (int j = 0; j < TE / 512; ++j) {
-        const int p = 2 * c + 512 * j;
-        if (p < len) {
-            double v[NIN][2];
-#pragma unroll
-            for (int k = 0; k < NIN; ++k) ld_shared_v2(sb + k * TE + p, v[k][0], v[k][1]);
-            double r[2];
-#pragma unroll
-            for (int q = 0; q < 2; ++q) {
-                double e[NIN];
-#pragma unroll
-                for (int k = 0; k < NIN; ++k) e[k] = v[k][q];
-                if constexpr (PM == 1) r[q] = Op::apply_fast(cf, e, q, away);
-                else r[q] = Op::template apply<0>(cf, e);
-            }
-            st_global_v2_cs(out + p, r[0], r[1]);
-        }
-    }
+    for (int j = 0; j < EPT / 2; ++j)
+        staged_pair<Op, PM, EPT, MIXED>(cf, sb, out, len, c, j, odd, away);
     if constexpr (PM == 1) {
         if ((int32_t)away < 0)
-            staged_tile_fp64<Op, TE>(cf.d[0], cf.d[1], cf.d[2], cf.d[3], cf.d[4], cf.d[5], cf.d[6],
-                                     cf.d[7], sb, out, len, c);
+            staged_tile_fp64<Op, EPT, MIXED>(cf.d[0], cf.d[1], cf.d[2], cf.d[3], cf.d[4], cf.d[5],
+                                             cf.d[6], cf.d[7], sb, out, len, c, odd);
     }
     return (int32_t)away < 0;
 }
 
-template <class Op>
-__global__ void __launch_bounds__(kStagedThreads, StageShape<Op::kIn>::kMinBlocks)
+template <class Op, int EPT, bool MIXED>
+__global__ void __launch_bounds__(kStagedThreads, (StageShape<Op::kIn, EPT, MIXED>::kMinBlocks))
     ew_staged_kernel(const EwArgs<Op::kIn> a) {
     constexpr int NIN = Op::kIn;
-    using SS = StageShape<NIN>;
+    using SS = StageShape<NIN, EPT, MIXED>;
     constexpr int TE = SS::kTile, S = SS::kStages;
-    extern __shared__ __align__(128) double ring[];  // [S][NIN][TE]
+    extern __shared__ __align__(128) double ring[];  // [S][NIN][SS::kStride]
     __shared__ __align__(8) uint64_t full[S], empty[S];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int64_t body = a.nch * 4;  // elements from a.head, a multiple of 4
@@ -470,11 +500,13 @@ __global__ void __launch_bounds__(kStagedThreads, StageShape<Op::kIn>::kMinBlock
                 const int64_t e0 = t * TE;
                 const uint32_t len = (uint32_t)(body - e0 < TE ? body - e0 : TE);
                 const uint32_t bar = smem_addr(&full[s]);
-                mbar_arrive_expect_tx(bar, len * 8u * NIN);
+                mbar_arrive_expect_tx(bar, len * 8u * NIN + (MIXED ? 16u * __popc(a.odd) : 0u));
 #pragma unroll
-                for (int k = 0; k < NIN; ++k)
-                    bulk_load(smem_addr(ring + ((size_t)s * NIN + k) * TE), a.in[k] + a.head + e0,
-                              len * 8u, bar, policy);
+                for (int k = 0; k < NIN; ++k) {
+                    const unsigned o = MIXED ? a.odd >> k & 1u : 0u;
+                    bulk_load(smem_addr(ring + ((size_t)s * NIN + k) * SS::kStride),
+                              a.in[k] + a.head + e0 - o, (len + 2u * o) * 8u, bar, policy);
+                }
             }
             // Every issued copy lands before the block exits (the earlier
             // ones were consumed before their stage was reused).
@@ -483,6 +515,14 @@ __global__ void __launch_bounds__(kStagedThreads, StageShape<Op::kIn>::kMinBlock
             if (!ok) atomicOr(&g_vec_fault, 1u);
         }
     } else {
+        // Head and tail elements (four each at most) by eight lanes of the last
+        // block, while its first tile is on its way: at the end they were a
+        // memory latency of their own (65536 elements, 8 bytes off, GB300:
+        // axpbypcz 2.7 us, 1.95 here).
+        if (blockIdx.x == gridDim.x - 1 && warp == kConsumerWarps - 1 && lane < 8) {
+            const int64_t e = lane < 4 ? lane : a.head + body + (lane - 4);
+            if (lane < 4 ? e < a.head : e < a.n) ew_scalar<Op>(a, e);
+        }
         unsigned slot = (warp * 5u + blockIdx.x * 3u) & 15u;
         int i = 0, fp64 = 0;
         for (int64_t t = blockIdx.x; t < ntiles; t += gridDim.x, ++i) {
@@ -493,7 +533,7 @@ __global__ void __launch_bounds__(kStagedThreads, StageShape<Op::kIn>::kMinBlock
             }
             const int64_t e0 = t * TE;
             const int len = (int)(body - e0 < TE ? body - e0 : TE);
-            const double *sb = ring + (size_t)s * NIN * TE;
+            const double *sb = ring + (size_t)s * NIN * SS::kStride;
             double *out = a.out + a.head + e0;
             // Data that keeps leaving the fast path (zeros, say) pays for both
             // kinds of product: after a tile where a quarter of the lanes did,
@@ -501,8 +541,9 @@ __global__ void __launch_bounds__(kStagedThreads, StageShape<Op::kIn>::kMinBlock
             // element zero, maxpy with 4 terms, n = 2^26 (GB300): 1065 us
             // against 1557.
             bool left = false;
-            if ((int)slot < a.pm && fp64 == 0) left = staged_tile<Op, 1, TE>(a.cf, sb, out, len, threadIdx.x);
-            else staged_tile<Op, 0, TE>(a.cf, sb, out, len, threadIdx.x);
+            if ((int)slot < a.pm && fp64 == 0) 
+                left = staged_tile<Op, 1, EPT, MIXED>(a.cf, sb, out, len, threadIdx.x, a.odd);
+            else staged_tile<Op, 0, EPT, MIXED>(a.cf, sb, out, len, threadIdx.x, a.odd);
             fp64 = __popc(__ballot_sync(0xffffffffu, left)) > 8 ? 16 : fp64 > 0 ? fp64 - 1 : 0;
             if (lane == 0) mbar_arrive(smem_addr(&empty[s]));
             slot = (slot + 1u) & 15u;
@@ -513,34 +554,41 @@ __global__ void __launch_bounds__(kStagedThreads, StageShape<Op::kIn>::kMinBlock
         // they come at the start, 3.45 here; maxpy with 8 terms on 131075, 5.7
         // and 4.9).
         pdl_trigger();
-        // head (< 4) and tail (< 4) elements by threads 0..7 of block 0
-        if (blockIdx.x == 0 && threadIdx.x < 8) {
-            const int t = threadIdx.x;
-            const int64_t body_end = a.head + body;
-            if (t < 4 && t < a.head) ew_scalar<Op>(a, t);
-            if (t >= 4 && body_end + (t - 4) < a.n) ew_scalar<Op>(a, body_end + (t - 4));
-        }
     }
 }
 
 // Per device: the dynamic shared-memory opt-in done and the resident blocks
 // per SM of one staged kernel.
-template <class Op>
+template <class Op, int EPT, bool MIXED>
 int staged_blocks_per_sm(int device) {
     static std::atomic<int> cached[64];
     if (device < 0 || device >= 64) return 0;
     int v = cached[device].load(std::memory_order_relaxed);
     if (v > 0) return v;
-    constexpr int smem = StageShape<Op::kIn>::kSmem;
-    if (cudaFuncSetAttribute(ew_staged_kernel<Op>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             smem) != cudaSuccess)
+    constexpr int smem = StageShape<Op::kIn, EPT, MIXED>::kSmem;
+    if (cudaFuncSetAttribute(ew_staged_kernel<Op, EPT, MIXED>,
+                             cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess)
         return 0;
     int nb = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, ew_staged_kernel<Op>, kStagedThreads,
-                                                      smem) != cudaSuccess || nb < 1)
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, ew_staged_kernel<Op, EPT, MIXED>,
+                                                      kStagedThreads, smem) != cudaSuccess || nb < 1)
         return 0;
     cached[device].store(nb, std::memory_order_relaxed);
     return nb;
+}
+
+template <class Op, int EPT, bool MIXED>
+cudaError_t launch_staged(const EwArgs<Op::kIn> &a, const DeviceProps *dp, cudaStream_t s) {
+    using SS = StageShape<Op::kIn, EPT, MIXED>;
+    const int nb = staged_blocks_per_sm<Op, EPT, MIXED>(dp->device);
+    if (nb == 0) {
+        const cudaError_t e = cudaGetLastError();
+        return e == cudaSuccess ? cudaErrorInvalidConfiguration : e;
+    }
+    const int64_t tiles = (a.nch * 4 + SS::kTile - 1) / SS::kTile;
+    const int64_t grid = std::max<int64_t>(1, std::min<int64_t>((int64_t)dp->sm_count * nb, tiles));
+    return launch_pdl_smem(&ew_staged_kernel<Op, EPT, MIXED>, (unsigned)grid, kStagedThreads,
+                           SS::kSmem, s, a);
 }
 
 std::atomic<long long> g_drop_tile{-1};
@@ -591,26 +639,42 @@ int launch_ew(const double *const *in, double *out, int64_t n, const double *coe
         if (k < ncoef && a.cf.m[k].win == 0) a.pm = 0;
     }
     cudaError_t e = injected_launch_error();
-    if (e == cudaSuccess && (diff & 31u) == 0) {
-        // 32-byte co-aligned: peel the head to the boundary, stage the body
+    if (e != cudaSuccess) return fail_cuda(e, "vector kernel launch");
+    a.odd = 0;
+    for (int k = 0; k < NIN; ++k)
+        if (((uintptr_t)in[k] ^ (uintptr_t)out) & 8u) a.odd |= 1u << k;
+    // The staged body wants its inputs at the output's place in 16 bytes, the
+    // direct one in 32; with the default sums the staged one takes any offset.
+    // Single elements from registers, the path they replace, ran axpbypcz and
+    // maxpy with 5 / 8 terms at 0.81 and 0.78 / 0.68 of the measured peak with
+    // differing offsets (n = 2^26, GB300), against 0.97 and 0.81 / 0.76 staged.
+    if (Op::kStaged ? a.odd == 0 || Op::kDefaultSums : (diff & 31u) == 0) {
+        // peel the head to the output's 32-byte boundary
         a.head = std::min<int64_t>((4 - (int64_t)(((uintptr_t)out >> 3) & 3)) & 3, n);
         a.nch = (n - a.head) / 4;
+        if (a.odd) {
+            // the copies reach one element before the body and one past it
+            if (a.head == 0) a.head = std::min<int64_t>(4, n);
+            a.nch = std::max<int64_t>(0, n - a.head - 1) / 4;
+        }
         if constexpr (Op::kStaged) {
-            const int nb = staged_blocks_per_sm<Op>(dp->device);
-            if (nb == 0) return fail_cuda(cudaGetLastError(), "staged kernel set-up");
-            constexpr int TE = StageShape<NIN>::kTile;
-            const int64_t tiles = (a.nch * 4 + TE - 1) / TE;
-            const int64_t grid =
-                std::max<int64_t>(1, std::min<int64_t>((int64_t)dp->sm_count * nb, tiles));
-            e = launch_pdl_smem(&ew_staged_kernel<Op>, (unsigned)grid, kStagedThreads,
-                                StageShape<NIN>::kSmem, s, a);
+            constexpr int EPT = kEpt<NIN>;
+            if constexpr (Op::kDefaultSums) {
+                const bool small = EPT > 2 && a.nch * 4 < (int64_t)dp->sm_count * 256 * EPT;
+                if (a.odd) e = small ? launch_staged<Op, 2, true>(a, dp, s) : launch_staged<Op, EPT, true>(a, dp, s);
+                else e = small ? launch_staged<Op, 2, false>(a, dp, s) : launch_staged<Op, EPT, false>(a, dp, s);
+            } else {
+                e = launch_staged<Op, EPT, false>(a, dp, s);
+            }
         } else {
             const int64_t per_block = 256 * 2;
+            const int64_t edges = a.head + 4 * a.nch != a.n || a.head != 0;
             const int64_t grid = std::max<int64_t>(
-                1, std::min<int64_t>((int64_t)dp->sm_count * 8, (a.nch + per_block - 1) / per_block));
+                1, std::min<int64_t>((int64_t)dp->sm_count * 8,
+                                     (a.nch + per_block - 1) / per_block + edges));
             e = launch_pdl(&ew_direct_kernel<Op>, (unsigned)grid, 256, s, a);
         }
-    } else if (e == cudaSuccess) {
+    } else {
         a.head = 0;
         a.nch = n;
         const int64_t per_block = 256 * 4;
@@ -630,8 +694,8 @@ std::atomic<int> g_vec_tuned[WXPY_VEC_CLASSES] = {-1, -1, -1, -1, -1, -1, -1, -1
 
 using Pipes = VecPipes;
 
-Pipes pipes_for(int cls) {
-    Pipes p = vecops_default(cls);
+Pipes pipes_for(int cls, int64_t n) {
+    Pipes p = vecops_default(cls, n);
     vecops_tuned_load(cls, &p);
     const int add = g_vec_add.load(), mul = g_vec_mul.load();
     if (add >= 0) p.add = add;
@@ -650,13 +714,19 @@ int maxpy_group(int64_t n, const double *alpha, const double *const *in, Pipes p
 
 }  // namespace
 
-// Defaults, measured on GB300 at n = 2^26 (sums in FP64, the cheaper pipe for
-// them; the product share that balanced the FP64 and ALU pipelines best).
-VecPipes vecops_default(int cls) {
-    if (cls == WXPY_VEC_AXPBYPCZ) return {0, 14};
-    if (cls == WXPY_VEC_AXPBY) return {0, 10};
+// Defaults, measured on GB300 (the product share that balanced the FP64 and ALU
+// pipelines best).  In calls that the L2 serves the fewer FP64 instructions the
+// better; where HBM sets the pace a few FP64 products are free and shorter.
+// us at 10^6 / 4x10^6 / 2^24 / 2^26 elements: axpby with all products integer
+// 4.8 / 14.2 / 68.0 / 263, with 10/16 6.2 / 17.7 / 66.1 / 245; axpbypcz 6.6 /
+// 20.1 / 82.5 / 320, 15/16 7.1 / 21.3 / 82.5 / 315; maxpy with two terms 6.6 /
+// 19.1 / 84.5 / 332, 14/16 7.3 / 21.6 / 82.1 / 313.
+VecPipes vecops_default(int cls, int64_t n) {
     if (cls == WXPY_VEC_PMULT) return {0, 4};
-    return {0, cls + 1 == 2 ? 14 : 16};  // maxpy with cls + 1 terms
+    const bool short_call = n < ((int64_t)1 << 23);
+    if (cls == WXPY_VEC_AXPBYPCZ) return {0, short_call ? 16 : 15};
+    if (cls == WXPY_VEC_AXPBY) return {0, short_call ? 16 : 10};
+    return {0, cls + 1 == 2 && !short_call ? 14 : 16};  // maxpy with cls + 1 terms
 }
 
 int vecops_inputs(int cls) {
@@ -722,7 +792,7 @@ int wxpy_aypx(int64_t n, double alpha, const double *x, double *y, void *stream)
 int wxpy_axpby(int64_t n, double alpha, double beta, const double *x, double *y, void *stream) {
     const double *in[2] = {x, y};
     const double coef[2] = {alpha, beta};
-    return vecops_run(WXPY_VEC_AXPBY, n, coef, in, y, pipes_for(WXPY_VEC_AXPBY),
+    return vecops_run(WXPY_VEC_AXPBY, n, coef, in, y, pipes_for(WXPY_VEC_AXPBY, n),
                       (cudaStream_t)stream);
 }
 
@@ -730,7 +800,7 @@ int wxpy_axpbypcz(int64_t n, double alpha, double beta, double gamma, const doub
                   const double *y, double *z, void *stream) {
     const double *in[3] = {x, y, z};
     const double coef[3] = {alpha, beta, gamma};
-    return vecops_run(WXPY_VEC_AXPBYPCZ, n, coef, in, z, pipes_for(WXPY_VEC_AXPBYPCZ),
+    return vecops_run(WXPY_VEC_AXPBYPCZ, n, coef, in, z, pipes_for(WXPY_VEC_AXPBYPCZ, n),
                       (cudaStream_t)stream);
 }
 
@@ -755,7 +825,7 @@ int wxpy_maxpy(int64_t n, int m, const double *alpha, const double *const *x, do
             const double *in[9];
             in[0] = y;
             for (int j = 0; j < g; ++j) in[j + 1] = x[j0 + j];
-            st = vecops_run(g - 1, n, alpha + j0, in, y, pipes_for(g - 1), s);
+            st = vecops_run(g - 1, n, alpha + j0, in, y, pipes_for(g - 1, n), s);
         }
         if (st != WXPY_OK) return st;
     }
@@ -764,7 +834,7 @@ int wxpy_maxpy(int64_t n, int m, const double *alpha, const double *const *x, do
 
 int wxpy_pointwise_mult(int64_t n, const double *x, const double *y, double *w, void *stream) {
     const double *in[2] = {x, y};
-    return vecops_run(WXPY_VEC_PMULT, n, nullptr, in, w, pipes_for(WXPY_VEC_PMULT),
+    return vecops_run(WXPY_VEC_PMULT, n, nullptr, in, w, pipes_for(WXPY_VEC_PMULT, n),
                       (cudaStream_t)stream);
 }
 

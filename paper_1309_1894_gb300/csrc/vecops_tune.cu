@@ -193,7 +193,7 @@ int tune_class(int cls, int64_t n, VScratch &sc, wxpy_vecops_tune_result *res) {
     }
     if (!have) return fail(WXPY_EMISMATCH, "every split of vector class %d differed", cls);
     double def_us = 0.0;
-    if ((st = time_split(c, n, vecops_default(cls), sc, &def_us)) != WXPY_OK) return st;
+    if ((st = time_split(c, n, vecops_default(cls, n), sc, &def_us)) != WXPY_OK) return st;
     vecops_tuned_store(cls, &best);
     if (res) {
         res->op_class = cls;

@@ -362,3 +362,34 @@ def test_maxpy_integer_sums(m, special):
     assert same(gy.t, oracle.maxpy(al, xsh, yh))
     for g in [gy] + gxs:
         g.check()
+
+
+@pytest.mark.parametrize("offs", [(8, 0, 16, 24), (0, 8, 8, 8), (16, 8, 0, 8), (24, 24, 24, 16),
+                                  (0, 16, 0, 16)])
+@pytest.mark.parametrize("n", [1, 2, 3, 4, 5, 8, 9, 12, 13, 511, 512, 517, 1029, 2053, 155700,
+                               700001])
+def test_staged_inputs_at_any_offset(n, offs):
+    """Inputs whose offsets from the output differ: copies that start one element
+    early and end one late stay inside the vectors (the guards hold signalling
+    NaN patterns, which an element used from outside would carry into a result),
+    heads, tails, both tile lengths, in place, with fallbacks in some tiles."""
+    rng = np.random.default_rng(n + sum(offs))
+    hs = [vals(n + 31 * k, n, False) for k in range(4)]
+    if n > 1000:
+        hs[0][n // 3: n // 3 + 700] = 0.0  # FP64 fallback in a few tiles
+    gs = [Guarded(n, o).set(h) for o, h in zip(offs, hs)]
+    x, y, z, u = (g.t for g in gs)
+    wx.wxpy_axpbypcz(0.75, -1.25, 0.5, x, y, z)
+    hs[2] = oracle.axpbypcz(0.75, -1.25, 0.5, hs[0], hs[1], hs[2])
+    wx.wxpy_axpby(-0.625, 0.375, z, u)
+    hs[3] = oracle.axpby(-0.625, 0.375, hs[2], hs[3])
+    wx.wxpy_maxpy([0.5, -0.25, 0.125], [y, z, u], x)
+    hs[0] = oracle.maxpy([0.5, -0.25, 0.125], [hs[1], hs[2], hs[3]], hs[0])
+    five = list(rng.uniform(-1, 1, 8))
+    wx.wxpy_maxpy(five, [x, z, u, x, z, u, x, z], y)
+    hs[1] = oracle.maxpy(five, [hs[0], hs[2], hs[3], hs[0], hs[2], hs[3], hs[0], hs[2]], hs[1])
+    torch.cuda.synchronize()
+    wx.wxpy_vecops_status()
+    for g, h in zip(gs, hs):
+        assert same(g.t, h)
+        g.check()
