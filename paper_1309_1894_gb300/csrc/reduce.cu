@@ -87,11 +87,11 @@ enum Deal {
 //              to the end of the row, and only its accesses are single ones
 //   kElements  positions 128 warp + lane + 32 q, so that the 8-byte accesses of
 //              a warp are contiguous
-template <int KIND, bool EMU, int DEAL>
+template <int KIND, bool EMU, int DEAL, bool EARLY>
 __device__ __forceinline__ void row_terms(const ReduceArgs &a, int64_t row, double (&t)[4],
                                           bool &left) {
     if constexpr (DEAL == kVectors) {
-        vector_terms<KIND, EMU, true>(a, row + 4 * threadIdx.x, t, left);
+        vector_terms<KIND, EMU, true, EARLY>(a, row + 4 * threadIdx.x, t, left);
     } else if constexpr (DEAL == kShifted) {
         const int64_t i = row + 4 * (int)threadIdx.x - a.shift;
         double x[4], y[4], z[4], w[4];
@@ -108,9 +108,7 @@ __device__ __forceinline__ void row_terms(const ReduceArgs &a, int64_t row, doub
                 if constexpr (KIND == 1) z[q] = a.z[e];
             }
         }
-#pragma unroll
-        for (int q = 0; q < 4; ++q)
-            element<KIND, EMU>(a, x[q], y[q], KIND == 1 ? z[q] : 0.0, w[q], t[q], left);
+        elements4<KIND, EMU, EARLY>(a, x, y, z, w, t, left);
         if (threadIdx.x != 0) {
             st4(a.w + i, w);
         } else {
@@ -151,7 +149,7 @@ __device__ __forceinline__ void row_terms(const ReduceArgs &a, int64_t row, doub
 // SUML (norm2 only): the first SUML of the three in-thread tree levels run as
 // integer-pipeline sums of non-negative values.  *left: the threads with an
 // element off the integer products' fast path.
-template <int KIND, int DEAL, bool EMU, int SUML = 0>
+template <int KIND, int DEAL, bool EMU, int SUML = 0, bool EARLY = false>
 __device__ double tile_sum(const ReduceArgs &a, int64_t tile, double *red, double *node, int *left) {
     static_assert(SUML == 0 || KIND == 0, "integer tree sums need non-negative terms");
     const int t = threadIdx.x, lane = t & 31;
@@ -169,8 +167,8 @@ __device__ double tile_sum(const ReduceArgs &a, int64_t tile, double *red, doubl
         for (int m = 0; m < 2; ++m) {
             const int j = h + 2 * m;
             double lo[4], hi[4];
-            row_terms<KIND, EMU, DEAL>(a, t0 + 1024 * j, lo, mine);
-            row_terms<KIND, EMU, DEAL>(a, t0 + 1024 * (j + 4), hi, mine);
+            row_terms<KIND, EMU, DEAL, EARLY>(a, t0 + 1024 * j, lo, mine);
+            row_terms<KIND, EMU, DEAL, EARLY>(a, t0 + 1024 * (j + 4), hi, mine);
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
                 rp[q] = rc[q];
@@ -219,7 +217,7 @@ __device__ double tile_sum(const ReduceArgs &a, int64_t tile, double *red, doubl
 // the block and bits 6..0 on four values per lane took 51 warp instructions
 // and four block barriers more per tile, of which 36 and one are left:
 // norm2 at n = 2^26 (GB300) went from 309 to 289 us.
-template <int KIND, int DEAL, int SUML = 0>
+template <int KIND, int DEAL, int SUML, bool EARLY>
 __global__ void __launch_bounds__(kThreads, 4) wxpy_reduce_kernel(const ReduceArgs a) {
     __shared__ __align__(16) double red[2][1024];  // two tiles in turn: one block barrier per tile
     __shared__ double node[128];
@@ -232,7 +230,7 @@ __global__ void __launch_bounds__(kThreads, 4) wxpy_reduce_kernel(const ReduceAr
         int left = 0;
         if (tile >= full) s = tile_sum<KIND, kElements, false>(a, tile, red[turn], node, &left);
         else if ((int)slot < a.mul_sixteenths && fp64 == 0)
-            s = tile_sum<KIND, DEAL, true, SUML>(a, tile, red[turn], node, &left);
+            s = tile_sum<KIND, DEAL, true, SUML, EARLY>(a, tile, red[turn], node, &left);
         else s = tile_sum<KIND, DEAL, false, SUML>(a, tile, red[turn], node, &left);
         // Data that keeps leaving the fast path (zeros, say) pays for both kinds of
         // product: after a tile where a quarter of the threads did, the block takes
@@ -544,21 +542,22 @@ cudaError_t launch_staged(const ReduceArgs &a, const DeviceProps *dp, cudaStream
     return cudaGetLastError();
 }
 
-template <int KIND, int DEAL, int SUML>
+template <int KIND, int DEAL, int SUML, bool EARLY>
 cudaError_t launch_block(const ReduceArgs &a, const DeviceProps *dp, cudaStream_t s) {
     static std::atomic<int> cached[64];
+    auto kernel = &wxpy_reduce_kernel<KIND, DEAL, SUML, EARLY>;
     const int dev = dp->device;
     int nb = dev >= 0 && dev < 64 ? cached[dev].load(std::memory_order_relaxed) : 0;
     if (nb <= 0) {
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, wxpy_reduce_kernel<KIND, DEAL, SUML>,
-                                                          kThreads, 0) != cudaSuccess || nb < 1) {
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kernel, kThreads, 0) != cudaSuccess ||
+            nb < 1) {
             cudaGetLastError();
             nb = 1;
         }
         if (dev >= 0 && dev < 64) cached[dev].store(nb, std::memory_order_relaxed);
     }
     const int64_t grid = std::max<int64_t>(1, std::min<int64_t>((int64_t)dp->sm_count * nb, a.ntiles));
-    return launch_pdl(&wxpy_reduce_kernel<KIND, DEAL, SUML>, (unsigned)grid, kThreads, s, a);
+    return launch_pdl(kernel, (unsigned)grid, kThreads, s, a);
 }
 
 std::atomic<int> g_reduce_mul{-1};
@@ -670,13 +669,21 @@ int launch_reduce(int64_t n, double alpha, const double *x, const double *y, dou
         if (e == cudaSuccess && a.ntiles == 1) return WXPY_OK;
     } else if (variant == 0) {
         const int suml = KIND == 0 && vec ? std::min(cfg.suml, 3) : 0;  // the in-thread levels
-        if (!vec) e = same ? launch_block<KIND, kShifted, 0>(a, dp, s) : launch_block<KIND, kElements, 0>(a, dp, s);
-        else if constexpr (KIND == 0)
-            e = suml == 0   ? launch_block<0, kVectors, 0>(a, dp, s)
-                : suml == 1 ? launch_block<0, kVectors, 1>(a, dp, s)
-                : suml == 2 ? launch_block<0, kVectors, 2>(a, dp, s)
-                            : launch_block<0, kVectors, 3>(a, dp, s);
-        else e = launch_block<KIND, kVectors, 0>(a, dp, s);
+        // blocks of a tile or two: the early test (elements4)
+        const bool brief = a.ntiles <= 8 * (int64_t)dp->sm_count;
+        if (!vec) {
+            e = !same   ? launch_block<KIND, kElements, 0, false>(a, dp, s)
+                : brief ? launch_block<KIND, kShifted, 0, true>(a, dp, s)
+                        : launch_block<KIND, kShifted, 0, false>(a, dp, s);
+        } else if constexpr (KIND == 0) {
+            e = suml == 0   ? (brief ? launch_block<0, kVectors, 0, true>(a, dp, s)
+                                     : launch_block<0, kVectors, 0, false>(a, dp, s))
+                : suml == 1 ? launch_block<0, kVectors, 1, false>(a, dp, s)
+                : suml == 2 ? launch_block<0, kVectors, 2, false>(a, dp, s)
+                            : launch_block<0, kVectors, 3, false>(a, dp, s);
+        } else {
+            e = launch_block<KIND, kVectors, 0, true>(a, dp, s);
+        }
     } else if (variant >= 4) {
         e = launch_reduce_warp(KIND, KIND == 0 ? cfg.suml : 0, variant - 4, a, dp, s);
     } else {

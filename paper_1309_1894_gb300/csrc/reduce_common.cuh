@@ -113,6 +113,52 @@ __device__ __forceinline__ void element(const ReduceArgs &a, double x, double y,
     element<KIND, EMU>(a, x, y, z, w, t, left);
 }
 
+static __device__ __noinline__ uint64_t mul_hw_bits(uint64_t ua, uint64_t ub) {
+    return bits_of(__dmul_rn(double_of(ua), double_of(ub)));
+}
+
+// w and the terms of four elements.  EARLY: the window of the four x is tested
+// before their products, so that data outside it (zeros, say) pays for no second
+// update sum; it costs norm2 4 % on data inside (n = 2^26, 291 against 303 us),
+// dot nothing (both 3-4 % on vectors past the boundary).  Without it, element() by element, a grid of a tile or two per
+// block has no next tile to take with FP64 products: every seventh element zero,
+// 2^22 elements, norm2 / dot 56 / 57 us, with it 47 / 48.
+template <int KIND, bool EMU, bool EARLY>
+__device__ __forceinline__ void elements4(const ReduceArgs &a, const double (&x)[4],
+                                          const double (&y)[4], const double (&z)[4],
+                                          double (&w)[4], double (&t)[4], bool &left) {
+    if constexpr (EMU && EARLY) {
+        uint32_t away = 0;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) away |= ((uint32_t)(bits_of(x[q]) >> 32) << 1) - a.ca.win;
+        uint64_t pb[4];
+        if ((int32_t)away < 0) {
+#pragma unroll
+            for (int q = 0; q < 4; ++q) pb[q] = mul_hw_bits(bits_of(a.alpha), bits_of(x[q]));
+            left = true;
+        } else {
+#pragma unroll
+            for (int q = 0; q < 4; ++q) pb[q] = mul_rn_quick(a.ca, bits_of(x[q]), away);
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            w[q] = __dadd_rn(double_of(pb[q]), y[q]);
+            const uint64_t wb = opaque_bits(w[q]);
+            bool slow = false;
+            uint64_t tb = KIND == 0 ? sqr_rn_core(wb, slow) : mul_rn_quick2(wb, bits_of(z[q]), slow);
+            if (slow) {
+                tb = mul_hw_bits(wb, KIND == 0 ? wb : bits_of(z[q]));
+                left = true;
+            }
+            t[q] = double_of(tb);
+        }
+    } else {
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+            element<KIND, EMU>(a, x[q], y[q], KIND == 1 ? z[q] : 0.0, w[q], t[q], left);
+    }
+}
+
 // Coherent evict-first 32-byte accesses: w may be one of the inputs.
 __device__ __forceinline__ void ld4(const double *p, double (&v)[4]) {
     asm volatile("ld.global.cs.v4.f64 {%0,%1,%2,%3}, [%4];"
@@ -129,7 +175,7 @@ __device__ __forceinline__ void st4(double *p, const double (&v)[4]) {
 // Terms of the four elements base .. base + 3; w stored.  VEC: one 32-byte
 // co-aligned vector of every operand; else element by element with bounds,
 // +0 terms past n.
-template <int KIND, bool EMU, bool VEC>
+template <int KIND, bool EMU, bool VEC, bool EARLY = false>
 __device__ __forceinline__ void vector_terms(const ReduceArgs &a, int64_t base, double (&t)[4],
                                              bool &left) {
     if constexpr (VEC) {
@@ -137,9 +183,7 @@ __device__ __forceinline__ void vector_terms(const ReduceArgs &a, int64_t base, 
         ld4(a.x + base, x);
         ld4(a.y + base, y);
         if constexpr (KIND == 1) ld4(a.z + base, z);
-#pragma unroll
-        for (int q = 0; q < 4; ++q)
-            element<KIND, EMU>(a, x[q], y[q], KIND == 1 ? z[q] : 0.0, w[q], t[q], left);
+        elements4<KIND, EMU, EARLY>(a, x, y, z, w, t, left);
         st4(a.w + base, w);
     } else {
 #pragma unroll
