@@ -229,33 +229,48 @@ Variant adjust_variant(const Variant &v, const CallClass &c) {
     return a;
 }
 
-// The variant of an untuned cell: 32-byte accesses, one pass per thread, and
-// (offload 3) every product in the integer pipelines, which leaves the FP64
-// pipeline one operation per element.  Measured on GB300, us per call back to
-// back with the inputs cold, against the single default {unroll 2, 256
-// threads, half the sums in the integer pipeline} that these lines replace:
+// The variant of an untuned cell: one pass per thread, and (offload 3) every
+// product in the integer pipelines, which leaves the FP64 pipeline one operation
+// per element.  Measured on GB300, us per call back to back with the inputs cold;
+// "before": the single default {32 bytes, unroll 2, 256 threads, half the sums in
+// the integer pipeline} that these lines replace.
 Variant default_variant(const CallClass &c, int64_t n) {
-    Variant v{32, 1, 128, 0, 1, -1, 1, 3};
-    const bool mixed = c.align < 32, xy = (c.alias & WXPY_ALIAS_XY) != 0;
-    if (n < ((int64_t)1 << 24)) {
-        // One vector per thread in small blocks: a short call has every load in
-        // flight at once, and a longer one ends on small blocks.  2^14 1.56
-        // against 2.09, 2^17 1.72 / 2.20, 2^22 15.3 / 16.0; offsets that differ
-        // 2^17 1.95 / 2.86, 2^22 15.1 / 16.4; x == y 2^22 10.5 / 13.9.
-        // Where the grid is between half a wave and one wave, 256 threads
-        // halve the blocks to start: 2^20 4.53 against 4.78 (and 6.05).
-        if (!mixed && n > ((int64_t)1 << 19) && n <= (int64_t)152 * 8 * 1024) v.threads = 256;
-    } else if (!mixed) {
-        // 2^24 56.4 / 57.1, 2^26 221.2 / 224.6, 2^28 878.8 / 885.9; x == y, where
-        // the sums' share weighs more, 38.8 / 49.6, 151.6 / 194.9, 599 / 772.
-        v.unroll = 2;
-        v.threads = 512;
-    } else if (xy) {
-        v.threads = 256;
-    } else {
-        // The old default holds: 2^24 56.8, 2^28 878.0 against 56.3, 883.8 with
-        // the products offloaded instead.
-        v = Variant{32, 2, 256, 0, 1, -1, 1, 1};
+    // 16-byte accesses: two elements per thread, so a short call has most threads
+    // to hide latency with and a long one ends on small blocks.  2^17 1.56, 2^19
+    // 2.74, 2^22 14.9, 2^24 56.5, 2^26 221.9, 2^28 881.0, against 1.72, 3.01, 15.4,
+    // 57.0, 222.6, 880.6 for the best 32-byte shape and 2.20, 3.38, 16.0, 57.1,
+    // 224.6, 885.9 before.
+    Variant v{16, 1, 256, 0, 0, -1, 1, 3};
+    const bool xy = (c.alias & WXPY_ALIAS_XY) != 0;
+    const bool one_wave = n > ((int64_t)3 << 18) && n <= (int64_t)152 * 8 * 1024;
+    if (n <= 4096 && c.align >= 16) {
+        // The smallest calls are launches: 1.31 to 1.43 against 1.69 before.
+        // Narrower accesses are faster (one element per thread 0.94 to 1.18); they
+        // are left to forced variants and to the search, because with one as the
+        // default no cell would count as launch-bound any more: the search marks a
+        // cell where the plain reference kernel is within its tie band of the best
+        // shape, and its choice and the saved one follow that mark.
+        v = Variant{32, 1, 128, 0, 1, -1, 1, 3};
+    } else if (c.align < 16) {
+        // Offsets that differ by an odd number of elements: the mixed-alignment
+        // kernel, which 32-byte variants run.  2^17 1.95, 2^22 15.1 against 2.86,
+        // 16.4 before; from 2^24 on the old default is the better one (2^28 878.0
+        // against 883.8), but for x == y.
+        v = Variant{32, 1, 128, 0, 1, -1, 1, 3};
+        if (n >= ((int64_t)1 << 24)) v = xy ? Variant{32, 1, 256, 0, 1, -1, 1, 3} : Variant{32, 2, 256, 0, 1, -1, 1, 1};
+        else if (one_wave) v.threads = 256;
+    } else if (n <= ((int64_t)1 << 15)) {
+        // 8192 1.20, 2^14 1.18, 2^15 1.20 against 1.30 with 256 threads (before:
+        // 2.09); 2^16 1.31 with either
+        v.threads = 128;
+    } else if (one_wave) {
+        // one wave of 32-byte accesses: 2^20 4.56 against 4.73 (before: 6.05)
+        v = Variant{32, 1, 256, 0, 1, -1, 1, 3};
+    } else if (xy && n > ((int64_t)1 << 20)) {
+        // x == y has one load per element in flight, and wants 32 bytes of it:
+        // 2^22 10.5, 2^26 149.1, 2^28 590 against 11.6, 165.9, 656 (before: 13.9,
+        // 194.9, 772).
+        v = Variant{32, 1, n < ((int64_t)1 << 23) ? 256 : 512, 0, 1, -1, 1, 3};
     }
     return adjust_variant(v, c);
 }
@@ -359,12 +374,13 @@ int launch_piece(const Variant &v, const DeviceProps &dp, int xy, int64_t n, dou
     int64_t grid = need + (edges && a.nchunks > 0 ? 1 : 0);
     if (v.blocks_per_sm > 0) grid = std::min<int64_t>(need, (int64_t)v.blocks_per_sm * dp.sm_count);
     if (grid > 0x7fffffff) return fail(WXPY_EINVAL, "grid too large for n = %lld", (long long)n);
-    // A grid that fills at most a quarter of the GPU's threads ends at once: the
+    // A grid that fills at most an eighth of the GPU's threads ends at once: the
     // next launch gains nothing by starting with it, and loses if its blocks are
     // few and long and spread unevenly over the SMs that are still taken (wxpy,
     // axpbypcz, norm2 and dot in turn on 131072 elements: 16.5 us a round when it
-    // starts early, 15.0 late; larger grids hide its launch, 2^20 4.5 against 5.1).
-    a.late = grid * threads <= (int64_t)dp.sm_count * 512;
+    // starts early, 15.0 late; larger grids hide its launch: two calls each on 2^18
+    // and 2^19 15.3 us early, 17.4 late, 2^20 4.5 against 5.1).
+    a.late = grid * threads <= (int64_t)dp.sm_count * 256;
     cudaError_t e = set_carveout(ent.func, dp.device, v.carveout);
     if (e != cudaSuccess) return fail_cuda(e, "cudaFuncSetAttribute(carveout)");
     e = injected_launch_error();
