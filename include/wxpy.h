@@ -241,12 +241,12 @@ int wxpy_reference(int64_t n, double alpha, const double *x, const double *y,
  *   wxpy_maxpy:          y[i] = RN(..RN(RN(y[i] + RN(a[0]*x[0][i])) + RN(a[1]*x[1][i])).. + RN(a[m-1]*x[m-1][i]))
  *   wxpy_pointwise_mult: w[i] = RN(x[i]*y[i])                     (VecPointwiseMult)
  *
- * axpy and aypx run the tuned wxpy() variants.  When all pointers share their
- * offset mod 32 bytes, axpby, axpbypcz and maxpy stream their inputs through a
- * shared-memory ring filled by bulk asynchronous copies (one producer warp,
- * eight consumer warps per block, persistent grid; see wxpy_vecops_status)
- * and pointwise_mult loads 32 bytes per thread into registers; otherwise all
- * three take one element per thread.  maxpy takes `alpha` (m values) and `x`
+ * axpy and aypx run the tuned wxpy() variants.  axpby, axpbypcz and maxpy
+ * stream their inputs, at any 8-byte offsets, through a shared-memory ring
+ * filled by bulk asynchronous copies (one producer warp, eight consumer warps
+ * per block, persistent grid; see wxpy_vecops_status).  pointwise_mult loads
+ * 32 bytes per thread into registers where all pointers share their offset
+ * mod 32 bytes, and one element per thread otherwise.  maxpy takes `alpha` (m values) and `x`
  * (m device pointers) as HOST arrays and makes one launch per group of 8
  * terms, in order. */
 int wxpy_axpy(int64_t n, double alpha, const double *x, double *y, void *stream);
@@ -267,9 +267,10 @@ int wxpy_pointwise_mult(int64_t n, const double *x, const double *y, double *w, 
  * the fraction, in sixteenths, of each warp's loop iterations whose products
  * run there (0..16).  -1 in either leaves that part to the operation's
  * searched split (wxpy_vecops_tune) or, when it has none, its default (sums
- * in FP64; products 12/16 for axpby, 14/16 for axpbypcz and for maxpy groups of 2 terms,
- * 16/16 for groups of 3..8, 4/16 for pointwise_mult; a maxpy group of one
- * term runs as wxpy() and its tuned variant).  The bits of every result are
+ * in FP64; products 16/16 below 2^23 elements, and from there 10/16 for axpby,
+ * 15/16 for axpbypcz, 14/16 for maxpy groups of 2 terms and 16/16 for groups of
+ * 3..8; 4/16 for pointwise_mult at every size; a maxpy group of one term runs
+ * as wxpy() and its tuned variant).  The bits of every result are
  * the same under every split; only the speed differs.  Process-wide, read at
  * each call.  Errors: WXPY_EINVAL out of range. */
 int wxpy_vecops_pipes(int add_offload, int mul_sixteenths);
@@ -314,7 +315,7 @@ int wxpy_vecops_tune(int64_t n, wxpy_vecops_tune_result *results);
 int wxpy_vecops_tuned_get(int op_class, int *add_offload, int *mul_sixteenths);
 int wxpy_vecops_tuned_set(int op_class, int add_offload, int mul_sixteenths);
 
-/* axpbypcz, maxpy and pointwise_mult on 32-byte co-aligned pointers stream
+/* axpby, axpbypcz and maxpy stream
  * their inputs into shared memory with bulk asynchronous copies, completed on
  * mbarriers; every wait on those barriers gives up after one second.  This
  * synchronises the current device, then returns WXPY_ETIMEOUT (and clears
@@ -619,8 +620,9 @@ typedef struct wxpy_batch_tune_result {
  * by running the plain reference variant on every segment, then runs the
  * batched launch with every (tile length, unroll) candidate, rejects any
  * whose output differs by a bit, and keeps the fastest (median time) for b.
- * Finally picks blocks per SM and fp64_offload (0, 1 or 3) on a mixed batch.
- * The results replace the
+ * Finally picks blocks per SM and fp64_offload (0, 1 or 3) on a mixed batch of
+ * all the buckets, with the tiles found above and with the built-in ones, and
+ * keeps (and reports) the faster set.  The results replace the
  * process's batch shape table, used by later plans.  Synchronous; allocates
  * and frees its own scratch.  flags: WXPY_TUNE_QUICK narrows the search. */
 int wxpy_batch_tune(int bucket_min, int bucket_max, unsigned flags,

@@ -252,13 +252,19 @@ Variant default_variant(const CallClass &c, int64_t n) {
         // shape, and its choice and the saved one follow that mark.
         v = Variant{32, 1, 128, 0, 1, -1, 1, 3};
     } else if (c.align < 16) {
-        // Offsets that differ by an odd number of elements: the mixed-alignment
-        // kernel, which 32-byte variants run.  2^17 1.95, 2^22 15.1 against 2.86,
-        // 16.4 before; from 2^24 on the old default is the better one (2^28 878.0
-        // against 883.8), but for x == y.
-        v = Variant{32, 1, 128, 0, 1, -1, 1, 3};
-        if (n >= ((int64_t)1 << 24)) v = xy ? Variant{32, 1, 256, 0, 1, -1, 1, 3} : Variant{32, 2, 256, 0, 1, -1, 1, 1};
-        else if (one_wave) v.threads = 256;
+        // Offsets that differ by an odd number of elements.  The worst of the
+        // offsets {0, 8, 24}, {8, 24, 0} and {16, 0, 8} bytes (x, y, w) decides, as
+        // the shapes differ by up to 9 % between them.  Short calls take scalar
+        // accesses: 2^14 1.19, 2^17 1.56 against 1.59, 1.83 for the 32-byte
+        // mixed-alignment kernel, which the longer ones run: with half the sums in
+        // the integer pipeline 2^20 5.59, 2^22 15.3, 2^24 57.2, 2^28 880 against
+        // 5.86, 15.7, 58.6, 952 with every product there (before: 6.3, 16.8, 58.8,
+        // 880).  x == y keeps the products there: 2^20 3.78, 2^28 604 against 4.01,
+        // 619 with 256 threads.
+        v = Variant{32, 1, 128, 0, 1, -1, 1, xy ? 3 : 1};
+        if (n > 4096 && n <= ((int64_t)1 << 17)) v = Variant{8, 1, 256, 0, 0, -1, 1, 3};
+        if (n >= ((int64_t)1 << 23) && !xy) v.threads = 256;
+        if (n >= ((int64_t)1 << 25) && !xy) v.unroll = 2;
     } else if (n <= ((int64_t)1 << 15)) {
         // 8192 1.20, 2^14 1.18, 2^15 1.20 against 1.30 with 256 threads (before:
         // 2.09); 2^16 1.31 with either
@@ -269,8 +275,10 @@ Variant default_variant(const CallClass &c, int64_t n) {
     } else if (xy && n > ((int64_t)1 << 20)) {
         // x == y has one load per element in flight, and wants 32 bytes of it:
         // 2^22 10.5, 2^26 149.1, 2^28 590 against 11.6, 165.9, 656 (before: 13.9,
-        // 194.9, 772).
-        v = Variant{32, 1, n < ((int64_t)1 << 23) ? 256 : 512, 0, 1, -1, 1, 3};
+        // 194.9, 772).  Where offsets mod 32 differ and it runs 16-byte accesses, small
+        // blocks: 2^22 11.2, 2^24 40.2, 2^28 605 against 11.4, 43.4, 650.
+        const int wide = n < ((int64_t)1 << 23) ? 256 : 512;
+        v = Variant{32, 1, c.align < 32 ? 128 : wide, 0, 1, -1, 1, 3};
     }
     return adjust_variant(v, c);
 }

@@ -652,6 +652,9 @@ int batch_tune_impl(int bmin, int bmax, unsigned flags, wxpy_batch_tune_result *
         }
     } cleanup{s, e0, e1};
     BatchShape shape = current_batch_shape();
+    BatchShape plain = shape;  // the same with the built-in tiles in the searched buckets
+    const BatchShape builtin = default_batch_shape();
+    double plain_us[kBuckets] = {};
     if (out) std::memset(out, 0, sizeof *out);
     int rejected = 0, candidates = 0;
     static const int32_t kTiles[] = {0, 1024, 2048, 4096, 8192, 16384, 32768, 65536};
@@ -659,6 +662,9 @@ int batch_tune_impl(int bmin, int bmax, unsigned flags, wxpy_batch_tune_result *
         SynthBatch sb;
         if ((st = make_batch(b, 0, 0, &sb, s))) return st;
         double best_us = 1e30;
+        plain.tile_elems[b] = builtin.tile_elems[b];
+        plain.unroll_log2[b] = builtin.unroll_log2[b];
+        plain_us[b] = 0;
         int32_t best_tile = shape.tile_elems[b];
         int8_t best_u = shape.unroll_log2[b];
         for (int32_t T : kTiles) {
@@ -676,6 +682,7 @@ int batch_tune_impl(int bmin, int bmax, unsigned flags, wxpy_batch_tune_result *
                     ++rejected;
                     continue;
                 }
+                if (T == builtin.tile_elems[b] && ul == builtin.unroll_log2[b]) plain_us[b] = us;
                 if (us < best_us) {
                     best_us = us;
                     best_tile = T;
@@ -693,36 +700,48 @@ int batch_tune_impl(int bmin, int bmax, unsigned flags, wxpy_batch_tune_result *
             out->gbs[b] = 24.0 * (double)sb.elems / (best_us * 1e-6) / 1e9;
         }
     }
-    // grid size on a mixed batch
+    // Grid size on a mixed batch, with the tiles found above and with the built-in
+    // ones: the buckets were searched one by one on batches of one size, which favour
+    // shorter tiles than a batch of many sizes does (4096 segments: 1114 us with the
+    // tiles that won there, 1078 us with the built-in ones).
     {
         SynthBatch sb;
         if ((st = make_batch(-1, bmin, bmax, &sb, s))) return st;
+        bool plain_ok = true;
+        for (int b = bmin; b <= bmax; ++b) plain_ok = plain_ok && plain_us[b] > 0;
         double best_us = 1e30;
-        int best_bps = shape.blocks_per_sm, best_of = shape.offload;
-        for (int of : {0, 1, 3})
-            for (int bps : {2, 4, 8, 32}) {
-                BatchShape cand = shape;
-                cand.blocks_per_sm = bps;
-                cand.offload = of;
-                double us = 0;
-                unsigned long long bad = 0;
-                if ((st = run_shape(sb, cand, *dp, reps, s, e0, e1, &us, &bad))) return st;
-                ++candidates;
-                if (bad) {
-                    ++rejected;
-                    continue;
+        BatchShape best = shape;
+        bool best_plain = false;
+        for (int tiles = 0; tiles < (plain_ok ? 2 : 1); ++tiles)
+            for (int of : {0, 1, 3})
+                for (int bps : {2, 4, 8, 32}) {
+                    BatchShape cand = tiles ? plain : shape;
+                    cand.blocks_per_sm = bps;
+                    cand.offload = of;
+                    double us = 0;
+                    unsigned long long bad = 0;
+                    if ((st = run_shape(sb, cand, *dp, reps, s, e0, e1, &us, &bad))) return st;
+                    ++candidates;
+                    if (bad) {
+                        ++rejected;
+                        continue;
+                    }
+                    if (us < best_us) {
+                        best_us = us;
+                        best = cand;
+                        best_plain = tiles != 0;
+                    }
                 }
-                if (us < best_us) {
-                    best_us = us;
-                    best_bps = bps;
-                    best_of = of;
-                }
-            }
-        shape.blocks_per_sm = best_bps;
-        shape.offload = best_of;
+        shape = best;
         if (out) {
-            out->blocks_per_sm = best_bps;
-            out->fp64_offload = best_of;
+            for (int b = bmin; b <= bmax && best_plain; ++b) {
+                out->tile_elems[b] = shape.tile_elems[b];
+                out->unroll[b] = 1 << shape.unroll_log2[b];
+                out->gbs[b] *= out->us[b] / plain_us[b];
+                out->us[b] = plain_us[b];
+            }
+            out->blocks_per_sm = shape.blocks_per_sm;
+            out->fp64_offload = shape.offload;
             out->mixed_us = best_us;
             out->mixed_gbs = 24.0 * (double)sb.elems / (best_us * 1e-6) / 1e9;
         }

@@ -320,10 +320,14 @@ int tune_impl(int64_t n, unsigned flags, wxpy_tune_result *out) {
         return le == cudaSuccess ? WXPY_OK : fail_cuda(le, "tuner reference timing");
     }, &ref_us);
     if (st != WXPY_OK) return st;
-    // Keep whichever of the winner and the default is faster on the re-timing.
+    // Keep whichever of the winner and the default is faster on the re-timing; within
+    // the timing's noise the default, whose shape was chosen over all offsets of the
+    // class where the search sees one set of them (mixed offsets at 2^28: a shape
+    // 0.3 % faster than the default on one set is 8 % slower on two others).
+    constexpr double kNoise = 1.005;
     Variant chosen = best.v;
     double chosen_us = best_us;
-    if (def_us < best_us) {
+    if (def_us < best_us * kNoise) {
         chosen = dv;
         chosen_us = def_us;
     }
