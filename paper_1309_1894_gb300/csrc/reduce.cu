@@ -568,8 +568,9 @@ std::atomic<int> g_reduce_tuned[2] = {-1, -1};  // (variant << 10) | (suml << 5)
 constexpr int kDefaultSumLevels = 0;
 constexpr int kReduceVariants = 7;  // 0 register-loaded, 1..3 staged, 4..6 warp-tiled
 // Measured on GB300 at n = 2^26 with every product in the integer pipelines
-// (GB/s of algorithmic bytes, norm2 / dot): register-loaded 4482 / 5485;
-// staged (4, 2) 3771 / 4575, (3, 3) 3822 / 4252, (2, 3) 3904 / 4851.
+// (GB/s of algorithmic bytes, norm2 / dot): register-loaded 5500 / 6115; staged
+// 4700 / 5136, 4604 / 4784, 4637 / 5194; warp-tiled 4599 / 5526, 5029 / 5286,
+// 4697 / 5838.
 constexpr int kDefaultVariant[2] = {0, 0};  // norm2, dot
 // Tiles up to which a call takes the cluster form (reduce_split.cu).  Measured on
 // GB300, norm2 / dot, us, cluster against block form: 2^21 elements 16.7 / 18.2
