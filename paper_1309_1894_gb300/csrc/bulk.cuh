@@ -38,6 +38,16 @@ __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
 }
 
+// One arrival for the calling warp, after every lane's accesses to the memory
+// that the barrier hands over.  The arrival is a release, but of lane 0's accesses
+// only: __syncwarp() orders the other lanes' before it, where a vote or a shuffle
+// would bring the lanes together without ordering memory, and a copy into the
+// memory could then pass reads that are still under way.
+__device__ __forceinline__ void mbar_arrive_warp(uint32_t bar, int lane) {
+    __syncwarp();
+    if (lane == 0) mbar_arrive(bar);
+}
+
 __device__ __forceinline__ bool mbar_test(uint32_t bar, uint32_t parity) {
     uint32_t done;
     asm volatile(

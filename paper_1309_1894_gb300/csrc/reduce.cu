@@ -314,8 +314,7 @@ __device__ __forceinline__ bool staged_chunk(const ReduceArgs &a, const double *
         ld_shared_v2(sb + kChunk + 64 * h, y[2 * h], y[2 * h + 1]);
         if constexpr (KIND == 1) ld_shared_v2(sb + 2 * kChunk + 64 * h, z[2 * h], z[2 * h + 1]);
     }
-    __syncwarp();
-    if (lane == 0) mbar_arrive(smem_addr(&empty[s]));  // the stage is in registers
+    mbar_arrive_warp(smem_addr(&empty[s]), lane);  // the stage is in registers
 #pragma unroll
     for (int q = 0; q < 4; ++q) element<KIND, EMU>(a, x[q], y[q], KIND == 1 ? z[q] : 0.0, w[q], e[q]);
     st_global_v2_cs(wp, w[0], w[1]);
@@ -492,16 +491,14 @@ __global__ void __launch_bounds__(kStagedThreads, MINB) wxpy_reduce_staged_kerne
             double *slotp = exch + (size_t)xs * kConsumerWarps * 128;
             st_shared_v2(slotp + exch_index(warp, 0, lane), v[0], v[1]);
             st_shared_v2(slotp + exch_index(warp, 1, lane), v[2], v[3]);
-            __syncwarp();
-            if (lane == 0) mbar_arrive(smem_addr(&xfull[xs]));
+            mbar_arrive_warp(smem_addr(&xfull[xs]), lane);
             if (warp == (k & 7)) {
                 if (!mbar_wait(smem_addr(&xfull[xs]), (k >> 1) & 1)) {
                     if (lane == 0) atomicOr(&g_reduce_fault, 4u);
                     break;
                 }
                 finish_tile(a, slotp, t, lane);
-                __syncwarp();
-                if (lane == 0) mbar_arrive(smem_addr(&xempty[xs]));
+                mbar_arrive_warp(smem_addr(&xempty[xs]), lane);
             }
             slot = (slot + 1u) & 15u;
         }

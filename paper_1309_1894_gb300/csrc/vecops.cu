@@ -545,7 +545,7 @@ __global__ void __launch_bounds__(kStagedThreads, (StageShape<Op::kIn, EPT, MIXE
                 left = staged_tile<Op, 1, EPT, MIXED>(a.cf, sb, out, len, threadIdx.x, a.odd);
             else staged_tile<Op, 0, EPT, MIXED>(a.cf, sb, out, len, threadIdx.x, a.odd);
             fp64 = __popc(__ballot_sync(0xffffffffu, left)) > 8 ? 16 : fp64 > 0 ? fp64 - 1 : 0;
-            if (lane == 0) mbar_arrive(smem_addr(&empty[s]));
+            mbar_arrive_warp(smem_addr(&empty[s]), lane);
             slot = (slot + 1u) & 15u;
         }
         // The next launch may start now, not before: blocks that come while these
