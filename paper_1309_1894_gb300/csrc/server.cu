@@ -34,6 +34,7 @@
 // Each request's result is element-wise w = RN(RN(alpha*x) + y) on its own
 // inputs (paper Sec. 3, Fig. 1 vecwxpy), so it is the same bits alone and in
 // any mix.
+#include <cuda.h>
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -54,6 +55,7 @@
 #include "fp64_mul.cuh"
 #include "gen.cuh"
 #include "internal.h"
+#include "ptr_range.h"
 #include "trace.h"
 
 namespace wx {
@@ -125,7 +127,7 @@ struct Request {
     // Caller data: source pointers and kind (WXPY_SERVE_DATA_*), or -1 for a
     // seeded request whose inputs the server generates.
     int src_kind = -1;
-    bool by_kernel = false;  // caller data in this device's memory: the inputs launch copies it
+    bool by_kernel = false;  // caller data that the inputs launch copies; set when the batch is built
     const double *src_x = nullptr, *src_y = nullptr;
     int state = kQueued;
     bool auto_release = false;
@@ -531,6 +533,43 @@ cudaError_t copy_in(const Request *r, cudaStream_t st) {
     return e;
 }
 
+// The driver's knowledge of an address (ptr_range.h); no context is needed.
+bool address_info(uint64_t p, AddressInfo *info) {
+    using Fn = CUresult (*)(unsigned, CUpointer_attribute *, void **, CUdeviceptr);
+    static const Fn get = [] {
+        void *f = nullptr;
+        cudaDriverEntryPointQueryResult found;
+        const cudaError_t e = cudaGetDriverEntryPointByVersion("cuPointerGetAttributes", &f, 12000,
+                                                               cudaEnableDefault, &found);
+        if (e != cudaSuccess) cudaGetLastError();
+        return e == cudaSuccess && found == cudaDriverEntryPointSuccess ? (Fn)f : nullptr;
+    }();
+    if (!get) return false;
+    CUmemorytype type = (CUmemorytype)0;
+    unsigned managed = 1;
+    int mapped = 0, device = -1;
+    CUdeviceptr start = 0;
+    size_t size = 0;
+    CUpointer_attribute what[] = {CU_POINTER_ATTRIBUTE_MEMORY_TYPE, CU_POINTER_ATTRIBUTE_IS_MANAGED,
+                                  CU_POINTER_ATTRIBUTE_MAPPED, CU_POINTER_ATTRIBUTE_DEVICE_ORDINAL,
+                                  CU_POINTER_ATTRIBUTE_RANGE_START_ADDR,
+                                  CU_POINTER_ATTRIBUTE_RANGE_SIZE};
+    void *to[] = {&type, &managed, &mapped, &device, &start, &size};
+    if (get(6, what, to, (CUdeviceptr)p) != CUDA_SUCCESS) return false;
+    *info = AddressInfo{type == CU_MEMORYTYPE_DEVICE && !managed && mapped, device, start, size};
+    return true;
+}
+
+// Whether the inputs launch may read the request's x and y.  Asked when the
+// batch is built, as the copy calls in its place would ask: a buffer may have
+// been freed since the request was submitted.
+bool readable_by_kernel(const Request *r, int device) {
+    const uint64_t bytes = (uint64_t)r->n * 8;
+    return r->src_kind == WXPY_SERVE_DATA_DEVICE &&
+           range_on_device((uint64_t)(uintptr_t)r->src_x, bytes, device, address_info) &&
+           range_on_device((uint64_t)(uintptr_t)r->src_y, bytes, device, address_info);
+}
+
 // Launches the requests in `batch` on slot s.  Caller does NOT hold the lock;
 // the requests are already marked running.  Returns a cudaError_t.
 cudaError_t launch_batch(wxpy_server *sv, Slot &s, const std::vector<Request *> &batch) {
@@ -568,9 +607,10 @@ cudaError_t launch_batch(wxpy_server *sv, Slot &s, const std::vector<Request *> 
     ServePlan *h_plan = s.host<ServePlan>(s.off_plan);
     ServePlan *h_cplan = s.host<ServePlan>(s.off_cplan);
     int64_t nplan = 0, ncopy = 0, elems = 0, seeded = 0, copied = 0;
-    for (const Request *r : batch) {
+    for (Request *r : batch) {
         elems += r->n;
         if (r->src_kind < 0) seeded += r->n;
+        r->by_kernel = readable_by_kernel(r, sv->device);
         if (r->by_kernel) copied += r->n;
     }
     const int64_t fill_tile = std::min<int64_t>(kFillTile, tile_cap(seeded));
@@ -838,7 +878,7 @@ void scheduler(wxpy_server *sv) {
 
 int submit_locked(wxpy_server *sv, int64_t n, double alpha, uint64_t seed, bool auto_release,
                   uint64_t *ticket, int src_kind = -1, const double *src_x = nullptr,
-                  const double *src_y = nullptr, bool by_kernel = false) {
+                  const double *src_y = nullptr) {
     if (n <= 0) return fail(WXPY_EINVAL, "request needs n > 0");
     const int64_t bytes = 3 * round_up(n * 8, kBlock);
     if (n > (int64_t)1 << 40 || bytes > sv->arena.size())
@@ -854,7 +894,6 @@ int submit_locked(wxpy_server *sv, int64_t n, double alpha, uint64_t seed, bool 
     r.alpha = alpha;
     r.seed = seed;
     r.src_kind = src_kind;
-    r.by_kernel = by_kernel;
     r.src_x = src_x;
     r.src_y = src_y;
     r.auto_release = auto_release;
@@ -864,16 +903,6 @@ int submit_locked(wxpy_server *sv, int64_t n, double alpha, uint64_t seed, bool 
     ++sv->submitted;
     *ticket = t;
     return WXPY_OK;
-}
-
-// Whether p is memory of device `dev`.
-bool on_device(const void *p, int dev) {
-    cudaPointerAttributes a;
-    if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
-        cudaGetLastError();
-        return false;
-    }
-    return a.type == cudaMemoryTypeDevice && a.device == dev;
 }
 
 double percentile(std::vector<double> v, double q) {
@@ -952,12 +981,8 @@ int wxpy_server_submit_data(wxpy_server *sv, int64_t n, double alpha, const doub
     if (sv->cfg.mode == WXPY_SERVE_FUSED)
         return fail(WXPY_EINVAL, "the fused mode generates its inputs: caller data needs the "
                                  "batched or serial mode");
-    // Plain memory of the server's device is read by the inputs launch; any
-    // other source (another device's, say) keeps its own copy.
-    const bool by_kernel = kind == WXPY_SERVE_DATA_DEVICE && sv->cfg.mode == WXPY_SERVE_BATCHED &&
-                           n > 0 && on_device(x, sv->device) && on_device(y, sv->device);
     std::lock_guard<std::mutex> lk(sv->mu);
-    const int st = submit_locked(sv, n, alpha, 0, false, ticket, kind, x, y, by_kernel);
+    const int st = submit_locked(sv, n, alpha, 0, false, ticket, kind, x, y);
     if (st == WXPY_OK) sv->cv_submit.notify_one();
     return st;
 }

@@ -351,3 +351,22 @@ def test_device_data_at_every_offset_and_length(shift):
             assert np.array_equal(got[1], yh.view(np.uint64))
             ok = (got[2] == want.view(np.uint64)) | (np.isnan(want) & np.isnan(got[2].view(np.float64)))
             assert ok.all()
+
+
+@pytest.mark.parametrize("kind", ["allocation", "part of one", "host"])
+def test_which_sources_the_inputs_launch_reads(kind):
+    """Ranges inside one device allocation are copied by the batch's own launch
+    (one more than the segmented one); host memory by copy calls."""
+    n = 40000
+    x = torch.rand(3 * n, dtype=torch.float64)
+    x = x if kind == "host" else x.cuda()
+    x, y = (x[:n], x[n:2 * n]) if kind != "part of one" else (x[n:2 * n], x[2 * n:])
+    with Server(budget_bytes=8 << 20, n_streams=1, max_batch=4) as sv:
+        for t in [sv.submit_data(0.5, x, y) for _ in range(6)]:
+            sv.wait(t, 60.0)
+            _, px, _, pw = sv.result(t)
+            assert torch.equal(_from_ptr(px, n).cpu(), x.cpu())
+            assert torch.equal(_from_ptr(pw, n).cpu(), (0.5 * x + y).cpu())
+            sv.release(t)
+        st = sv.stats()
+        assert st["launches"] == (1 if kind == "host" else 2) * st["batches"]
