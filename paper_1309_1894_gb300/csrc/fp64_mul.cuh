@@ -64,6 +64,8 @@ struct MulCoef {
     int32_t e;     // biased exponent - 1024; 2^20 when the operand is not normal
     uint32_t k;    // sign << 31 plus (biased exponent - 1024) << 20, modulo 2^32
     uint32_t win;  // mul_rn_quick: first exponent field of the other operand's window, << 21
+    uint32_t from, span;  // mul_rn_range: first exponent field of the other operand's
+                          // range, << 21, and the range's length, << 21 (0: none)
 };
 
 // The exponent window of mul_rn_quick: the 1024 exponent fields from first on,
@@ -90,6 +92,10 @@ WX_MUL_FN MulCoef mul_coef_of(uint64_t ua) {
     c.e = ea - 1u >= 0x7FEu ? (1 << 20) : (int32_t)ea - 1024;
     c.k = (ah & 0x80000000u) + ((uint32_t)((int32_t)ea - 1024) << 20);
     c.win = (uint32_t)mul_window_first(ua) << 21;
+    // result exponent fields 1 .. 0x7FD, t = 1 included, of normal operands
+    const int32_t first = c.e < 0 ? -c.e : 1, last = c.e > -3 ? 0x7FB - c.e : 0x7FE;
+    c.from = (uint32_t)first << 21;
+    c.span = last >= first ? (uint32_t)(last + 1 - first) << 21 : 0u;
     return c;
 }
 
@@ -150,6 +156,23 @@ WX_MUL_FN uint64_t mul_rn_quick(const MulCoef &c, uint64_t ub, uint32_t &away) {
     const uint32_t bh = (uint32_t)(ub >> 32), bl = (uint32_t)ub;
     const uint32_t b1 = (bh & 0xFFFFFu) | 0x100000u;
     away |= (bh << 1) - c.win;
+    const uint64_t p00 = (uint64_t)c.lo * bl;
+    const uint64_t x = (uint64_t)c.hi * bl + (uint64_t)c.lo * b1 + (p00 >> 32);
+    const uint64_t top = (uint64_t)c.hi * b1 + (x >> 32);
+    uint32_t t;
+    return round_product(top, (uint32_t)x, (uint32_t)p00, c.k + (bh & 0xFFF00000u), &t);
+}
+
+// The same over the whole range of operands whose product is in the normal range
+// whatever t and the rounding: `far` becomes the largest distance of their
+// exponent fields above the range's first (modulo 2^32, so a field below it is
+// far as well), and the products made so far are meaningless once it is
+// c.span or more.  One coefficient for all of them.
+WX_MUL_FN uint64_t mul_rn_range(const MulCoef &c, uint64_t ub, uint32_t &far) {
+    const uint32_t bh = (uint32_t)(ub >> 32), bl = (uint32_t)ub;
+    const uint32_t b1 = (bh & 0xFFFFFu) | 0x100000u;
+    const uint32_t d = (bh << 1) - c.from;
+    far = d > far ? d : far;
     const uint64_t p00 = (uint64_t)c.lo * bl;
     const uint64_t x = (uint64_t)c.hi * bl + (uint64_t)c.lo * b1 + (p00 >> 32);
     const uint64_t top = (uint64_t)c.hi * b1 + (x >> 32);

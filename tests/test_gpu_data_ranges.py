@@ -1,0 +1,91 @@
+"""GPU parity on data that leaves the integer products' fast path: zeros,
+infinities, NaNs and subnormals among ordinary values, magnitudes over the whole
+exponent range, and coefficients at its ends -- every element bit for bit (a NaN
+for a NaN)."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import paper_1309_1894_gb300 as wx
+from paper_1309_1894_gb300 import binding, synth
+
+pytestmark = pytest.mark.gpu
+
+KINDS = ["zeros", "sevenths", "infinite", "mixed", "huge", "tiny", "spread"]
+
+
+def data(kind, n, seed):
+    """Values of one kind; the rest U(-1, 1)."""
+    v = synth.uniform_pm1(seed, synth.TAG_X, n)
+    rng = np.random.default_rng(seed)
+    if kind == "zeros":
+        v[:] = 0.0
+        v[1::2] = -0.0
+    elif kind == "sevenths":
+        v[::7] = 0.0
+    elif kind == "infinite":
+        v[:] = np.inf
+    elif kind == "mixed":
+        at = rng.permutation(n)
+        for k, s in enumerate((0.0, -0.0, np.inf, -np.inf, np.nan, 5e-324, -1e-310, 1e300, -1e-300)):
+            v[at[k * (n // 97):(k + 1) * (n // 97)]] = s
+    elif kind == "huge":
+        v *= 1e200
+    elif kind == "tiny":
+        v *= 1e-200
+    elif kind == "spread":
+        v = np.ldexp(v, rng.integers(-1070, 1024, n))
+    return v
+
+
+def same(got, want):
+    got, want = (np.ascontiguousarray(a, np.float64) for a in (got, want))
+    nan = np.isnan(want)
+    return np.array_equal(np.isnan(got), nan) and \
+        np.array_equal(got.view(np.uint64)[~nan], want.view(np.uint64)[~nan])
+
+
+def at(host, shift):
+    t = torch.empty(len(host) + 8, dtype=torch.float64, device="cuda")[shift:shift + len(host)]
+    return t.copy_(torch.from_numpy(host))
+
+
+@pytest.mark.parametrize("kind", KINDS)
+@pytest.mark.parametrize("shifts", [(0, 0, 0), (2, 0, 2), (0, 1, 3), (1, 1, 1)])
+@pytest.mark.parametrize("n", [1027, 100003, (1 << 20) + 1])
+def test_single_calls(n, shifts, kind):
+    xh, yh = data(kind, n, 21 + n % 13), synth.uniform_pm1(5, synth.TAG_Y, n)
+    x, y = at(xh, shifts[0]), at(yh, shifts[1])
+    for alpha in (0.7, -2.0 ** 600, 3e-308, 1e308, 0.0):
+        with np.errstate(all="ignore"):
+            want, want_xx = oracle.wxpy(alpha, xh, yh), oracle.wxpy(alpha, xh, xh)
+        w = at(np.zeros(n), shifts[2])
+        wx.wxpy(alpha, x, y, w)
+        assert same(w.cpu().numpy(), want), alpha
+        wx.wxpy(alpha, x, x, w)
+        assert same(w.cpu().numpy(), want_xx), alpha
+
+
+@pytest.mark.parametrize("kind", KINDS)
+@pytest.mark.parametrize("entry", ["launch", "once", "noalloc"])
+@pytest.mark.parametrize("shifts", [(0, 0, 0), (3, 0, 1)])
+@pytest.mark.parametrize("lengths", [[5, 1, 70001, 4099], [300] * 500, [40000] * 260])
+def test_batches(entry, kind, shifts, lengths):
+    total = sum(lengths)
+    starts = np.concatenate([[0], np.cumsum(lengths)[:-1]]).astype(np.int64)
+    xh, yh = data(kind, total, 31), synth.uniform_pm1(6, synth.TAG_Y, total)
+    alphas = np.resize([0.7, -2.0 ** 600, 3e-308, 1e308, 0.0, -0.3], len(lengths))
+    x, y, w = at(xh, shifts[0]), at(yh, shifts[1]), at(np.full(total, 7.25), shifts[2])
+    table = wx.desc_table(lengths, alphas, *(t.data_ptr() + 8 * starts for t in (x, y, w)))
+    dev = wx.table_to_device(table)
+    if entry == "noalloc":
+        binding.wxpy_batch_noalloc(dev, len(lengths))
+    elif entry == "once":
+        wx.wxpy_batch(table, dev)
+    else:
+        wx.wxpy_batch_plan_create(table).launch(dev)
+    torch.cuda.synchronize()
+    with np.errstate(all="ignore"):
+        want = np.repeat(alphas, lengths) * xh + yh  # two roundings, as the oracle's loop
+    assert same(w.cpu().numpy(), want)
