@@ -105,16 +105,23 @@ WX_EMU_FN uint64_t add_rn_with(uint64_t ua, uint64_t ub, Hw hw) {
 // RN(a + b) with the cheapest checks, for kernels that move a few of many sums:
 // ORs into `away` a word whose top bit is set when the operands leave the fast
 // path (the bits are then meaningless): the larger magnitude's exponent field
-// outside [512, 1535], a gap of more than 30 between the two (zeros always),
-// or a difference that cancels 20 bits or more.
+// outside [64, 2015], or a difference that cancels 20 bits or more.  Every gap
+// between the two is taken, and a zero or subnormal smaller one, which is 64 or
+// more below and counts as a number of that exponent field.
 //
 // Method, in 32-bit words.  The larger operand's significand, hidden bit at bit
-// 19 of the top word, and the smaller one's shifted right by the gap are held
-// exactly in 96 bits; they are added, or subtracted as a two's complement when
-// the signs differ.  The sum's leading bit is at bit 20 or below, so one left
-// shift puts it there.  The lowest word is then all that is rounded away, and
-// adding one half to it carries into the significand exactly when it is at
-// least one half; it becomes 0 exactly on a tie, which clears the lowest bit.
+// 19 of the top word, and the smaller one's shifted right by the gap are held in
+// 96 bits; they are added, or subtracted as a two's complement when the signs
+// differ.  The shift is made in two parts, by up to 32 bits and by the rest, and
+// `lost` is not 0 exactly when bits of it leave the 96 (gaps of 33 and more;
+// from 63 on the smaller one counts as about that far below, and no bit of the
+// result depends on how far).  A sum with lost bits lies above the 96 bits by
+// less than one of them; a difference lies below, so its complement leaves out
+// the final one and then lies above as well.  The sum's leading bit is at bit 20
+// or below, so one left shift puts it there.  The lowest word is then all that
+// is rounded away, and adding one half to it carries into the significand
+// exactly when it is at least one half; it becomes 0 with nothing lost exactly
+// on a tie, which clears the lowest bit.
 WX_EMU_FN uint64_t add_rn_quick(uint64_t ua, uint64_t ub, uint32_t &away) {
     const uint32_t ah = (uint32_t)(ua >> 32), al = (uint32_t)ua;
     const uint32_t bh = (uint32_t)(ub >> 32), bl = (uint32_t)ub;
@@ -126,7 +133,10 @@ WX_EMU_FN uint64_t add_rn_quick(uint64_t ua, uint64_t ub, uint32_t &away) {
     const uint32_t d = (x + 0x100000u) >> 20;  // gap + 1
     const uint32_t hm = (H & 0xFFFFFu) | 0x100000u, lm = (L & 0xFFFFFu) | 0x100000u;
     const uint32_t m = (uint32_t)((int32_t)(ah ^ bh) >> 31);
-    const uint32_t t2 = lm >> (d & 31u), t1 = funnel_r(ll, lm, d & 31u), t0 = funnel_r(0u, ll, d & 31u);
+    const uint32_t e = d > 32u ? d - 32u : 0u;  // the shift's second part
+    const uint32_t r1 = funnel_rc(ll, lm, d), r0 = funnel_rc(0u, ll, d);
+    const uint32_t t2 = funnel_rc(lm, 0u, d), t1 = funnel_rc(r1, 0u, e), t0 = funnel_rc(r0, r1, e);
+    const uint32_t lost = funnel_rc(0u, r0, e);
     uint32_t s2, s1, s0;
 #ifdef __CUDA_ARCH__
     uint32_t drop;
@@ -135,16 +145,16 @@ WX_EMU_FN uint64_t add_rn_quick(uint64_t ua, uint64_t ub, uint32_t &away) {
         "addc.cc.u32 %1, %7, %8;\n\t"
         "addc.u32 %2, %9, %10;"
         : "=r"(s0), "=r"(s1), "=r"(s2), "=r"(drop)
-        : "r"(m), "r"(hl << 31), "r"(t0 ^ m), "r"(funnel_r(hl, hm, 1u)), "r"(t1 ^ m), "r"(hm >> 1),
+        : "r"(m & ~lost), "r"(hl << 31), "r"(t0 ^ m), "r"(funnel_r(hl, hm, 1u)), "r"(t1 ^ m), "r"(hm >> 1),
           "r"(t2 ^ m));
     const int lz = __clz((int)s2);
 #else
-    const uint64_t w0 = (uint64_t)(hl << 31) + (t0 ^ m) + (m & 1u);
+    const uint64_t w0 = (uint64_t)(hl << 31) + (t0 ^ m) + (lost == 0u ? m & 1u : 0u);
     const uint64_t w1 = (uint64_t)funnel_r(hl, hm, 1u) + (t1 ^ m) + (w0 >> 32);
     s0 = (uint32_t)w0, s1 = (uint32_t)w1, s2 = (hm >> 1) + (t2 ^ m) + (uint32_t)(w1 >> 32);
     const int lz = s2 ? __builtin_clz(s2) : 32;
 #endif
-    away |= ((H << 1) - (512u << 21)) | ((31u << 20) - 1u - x) | (s2 - 1u);
+    away |= (H - (64u << 20)) | ((2016u << 20) - 1u - H) | (s2 - 1u);
     const uint32_t n = (uint32_t)lz - 11u;  // left shift: leading bit to bit 20
     const uint32_t r = 32u - n;
     // left funnels as right ones of the neighbouring words (n in 0..20)
@@ -170,7 +180,7 @@ WX_EMU_FN uint64_t add_rn_quick(uint64_t ua, uint64_t ub, uint32_t &away) {
     lo = o1 + (g >> 31);
     hi = hw + (uint32_t)(lo < o1);
 #endif
-    lo = gs == 0u ? lo & ~1u : lo;
+    lo = (gs | lost) == 0u ? lo & ~1u : lo;
     return ((uint64_t)hi << 32) | lo;
 }
 

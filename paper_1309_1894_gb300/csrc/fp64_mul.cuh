@@ -39,6 +39,15 @@ WX_MUL_FN uint32_t funnel_r(uint32_t lo, uint32_t hi, uint32_t sh) {
 #endif
 }
 
+// The same for any sh, with no bits left of the word at 32 and more.
+WX_MUL_FN uint32_t funnel_rc(uint32_t lo, uint32_t hi, uint32_t sh) {
+#ifdef __CUDA_ARCH__
+    return __funnelshift_rc(lo, hi, sh);
+#else
+    return (uint32_t)((((uint64_t)hi << 32) | lo) >> (sh < 32u ? sh : 32u));
+#endif
+}
+
 // RN(a * b) in the integer pipelines (multiply-adds on the FMA pipeline, the
 // rest on the ALU).
 //

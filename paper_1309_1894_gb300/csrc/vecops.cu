@@ -44,10 +44,22 @@ namespace wx {
 namespace {
 
 // Coefficients of one launch: as doubles for the FP64 instructions and split
-// once on the host for the integer-pipeline products.
+// once on the host for the integer-pipeline products, whose operands' range
+// (`from` in each split, `span` here) is the one that suits all of them.
 struct Coefs {
     double d[8];
     MulCoef m[8];
+    uint32_t span;
+};
+
+// What tells that a thread's elements left the fast path of the integer
+// pipelines: the products' distance (mul_rn_range), and the sums' word
+// (add_rn_quick).
+struct Leave {
+    uint32_t far = 0, gap = 0;
+    __device__ __forceinline__ bool left(const Coefs &c) const {
+        return far >= c.span || (int32_t)gap < 0;
+    }
 };
 
 template <int NIN>
@@ -74,10 +86,11 @@ __device__ __forceinline__ double double_of(uint64_t b) { return __longlong_as_d
 // p[j] = RN(c_j * e[F + j]), j < K, F = NIN - K (the data operands follow any
 // others).  PM = 1: integer-pipeline products, one out-of-line fallback to the
 // hardware instruction for the whole element when any of them leaves the
-// fast path.  At n = 2^26 (GB300) the windowed products (mul_rn_quick) took
-// axpbypcz from 0.92 to 0.965 of the measured peak and maxpy with 4 / 8 terms
-// from 0.87 / 0.74 to 0.89 / 0.755, against the fully checked ones; there the
-// sums keep the FP64 pipeline at the rate a plain chain of sums reaches.
+// fast path.  At n = 2^26 (GB300) products with one range test for all of them
+// (mul_rn_range) took axpbypcz from 0.92 to 0.965 of the measured peak and maxpy
+// with 4 / 8 terms from 0.87 / 0.74 to 0.89 / 0.755, against the fully checked
+// ones; there the sums keep the FP64 pipeline at the rate a plain chain of sums
+// reaches.
 template <int PM, int K, int NIN>
 __device__ __forceinline__ void products(const Coefs &c, const double (&e)[NIN], double (&p)[K]) {
     constexpr int F = NIN - K;
@@ -85,11 +98,11 @@ __device__ __forceinline__ void products(const Coefs &c, const double (&e)[NIN],
 #pragma unroll
         for (int j = 0; j < K; ++j) p[j] = __dmul_rn(c.d[j], e[F + j]);
     } else {
-        uint32_t away = 0;
+        uint32_t far = 0;
         uint64_t b[K];
 #pragma unroll
-        for (int j = 0; j < K; ++j) b[j] = mul_rn_quick(c.m[j], bits_of(e[F + j]), away);
-        if ((int32_t)away < 0) {
+        for (int j = 0; j < K; ++j) b[j] = mul_rn_range(c.m[j], bits_of(e[F + j]), far);
+        if (far >= c.span) {
 #pragma unroll
             for (int j = 0; j < K; ++j) b[j] = mul_rn_hw_bits(bits_of(c.d[j]), bits_of(e[F + j]));
         }
@@ -99,14 +112,21 @@ __device__ __forceinline__ void products(const Coefs &c, const double (&e)[NIN],
 }
 
 // The fast path of the integer-pipeline products alone: p[j] as in
-// products<1>, with the top bit of `away` set when any of them left the fast
-// path (its bits are then meaningless and the caller recomputes the element).
+// products<1>; one that left the fast path shows in l.far (its bits are then
+// meaningless and the caller recomputes the element).  Two distances and the
+// largest so far in one instruction: maxpy with 8 terms, n = 2^24, 251 us against
+// 257 with one at a time (GB300).
 template <int K, int NIN>
 __device__ __forceinline__ void products_fast(const Coefs &c, const double (&e)[NIN], double (&p)[K],
-                                              uint32_t &away) {
+                                              Leave &l) {
     constexpr int F = NIN - K;
 #pragma unroll
-    for (int j = 0; j < K; ++j) p[j] = double_of(mul_rn_quick(c.m[j], bits_of(e[F + j]), away));
+    for (int j = 0; j < K; j += 2) {
+        uint32_t d0 = 0, d1 = 0;
+        p[j] = double_of(mul_rn_range(c.m[j], bits_of(e[F + j]), d0));
+        if (j + 1 < K) p[j + 1] = double_of(mul_rn_range(c.m[j + 1], bits_of(e[F + j + 1]), d1));
+        l.far = __vimax3_u32(d0, d1, l.far);
+    }
 }
 
 template <int OFF>
@@ -120,9 +140,9 @@ struct AxpbyOp {
         return add_sel<OFF>(p[0], p[1], 1);
     }
     __device__ __forceinline__ static double apply_fast(const Coefs &c, const double (&e)[kIn], int,
-                                                        uint32_t &away) {
+                                                        Leave &l) {
         double p[2];
-        products_fast(c, e, p, away);
+        products_fast(c, e, p, l);
         return add_sel<OFF>(p[0], p[1], 1);
     }
 };
@@ -139,9 +159,9 @@ struct AxpbypczOp {
         return add_sel<OFF>(s1, p[2], OFF == 1 ? 0 : 1);
     }
     __device__ __forceinline__ static double apply_fast(const Coefs &c, const double (&e)[kIn], int,
-                                                        uint32_t &away) {
+                                                        Leave &l) {
         double p[3];
-        products_fast(c, e, p, away);
+        products_fast(c, e, p, l);
         const double s1 = add_sel<OFF>(p[0], p[1], 1);
         return add_sel<OFF>(s1, p[2], OFF == 1 ? 0 : 1);
     }
@@ -151,14 +171,16 @@ struct AxpbypczOp {
 // integer pipeline on the staged kernel's fast path, for the two elements of a
 // pair.  The FP64 pipeline does 1.7 sums per clock and SM whatever the code
 // (5.0e11/s), so m sums per 8(m + 2) bytes hold these kernels to 0.92 of the HBM
-// peak with 4 terms and 0.76 with 8; an integer sum is about 45 ALU operations,
-// and there is ALU time left for one or two in sixteen.  n = 2^26 (GB300), us
-// with none / these: 4 terms 532 / 502, 5 660 / 611, 6 802 / 751, 7 929 / 856,
-// 8 1056 / 973; with 3 terms one of six is slower, 408 / 414.
+// peak with 4 terms and 0.76 with 8; an integer sum is about 50 ALU operations,
+// and there is ALU time left for one or two in sixteen.  n = 2^24 (GB300), us
+// with none / these: 4 terms 137 / 133, 5 169 / 159, 6 204 / 191, 7 237 / 221,
+// 8 269 / 246; with 3 terms one of six is slower.  Which of them matters, by
+// where it falls among the other sums: 8 terms with sums 0 and 0 264, 3 and 3
+// 252.
 template <int M>
 __device__ constexpr unsigned integer_sums(int q) {
-    constexpr unsigned k[7][2] = {{0, 0}, {0, 0}, {0, 1u << 2}, {0, 1u << 3},
-                                  {0, 1u << 2}, {1u << 0, 1u << 3}, {1u << 3, 1u << 3}};
+    constexpr unsigned k[7][2] = {{0, 0}, {0, 0}, {1u << 1, 0}, {1u << 3, 0},
+                                  {0, 1u << 3}, {0, 1u << 3}, {1u << 2, 1u << 5}};
     return k[M - 2][q];
 }
 
@@ -176,14 +198,14 @@ struct MaxpyOp {
         return acc;
     }
     __device__ __forceinline__ static double apply_fast(const Coefs &c, const double (&e)[kIn], int q,
-                                                        uint32_t &away) {
+                                                        Leave &l) {
         double p[M];
-        products_fast(c, e, p, away);
+        products_fast(c, e, p, l);
         double acc = e[0];
 #pragma unroll
         for (int j = 0; j < M; ++j) {
             if (OFF == 0 && (integer_sums<M>(q) >> j & 1u))
-                acc = double_of(add_rn_quick(j ? opaque_bits(acc) : bits_of(acc), bits_of(p[j]), away));
+                acc = double_of(add_rn_quick(j ? opaque_bits(acc) : bits_of(acc), bits_of(p[j]), l.gap));
             else
                 acc = add_sel<OFF>(acc, p[j], j + 1);
         }
@@ -377,11 +399,11 @@ __device__ __forceinline__ double ld_shared_1(const double *p) {
 // input whose offset from the output is an odd number of elements is copied from
 // one element earlier (bit k of `odd`), and its 16-byte pairs would straddle the
 // output's; single accesses, 256 contiguous bytes a warp, are free of bank
-// conflicts at either offset.  Returns whether the first of the two is there;
-// the second is too, but for MIXED where it says so.
+// conflicts at either offset.  The second element is there if the first is, but
+// for MIXED where it says so.
 template <class Op, int PM, int EPT, bool MIXED>
 __device__ __forceinline__ void staged_pair(const Coefs &cf, const double *sb, double *out, int len,
-                                            int c, int j, unsigned odd, uint32_t &away) {
+                                            int c, int j, unsigned odd, Leave &l) {
     constexpr int NIN = Op::kIn;
     using SS = StageShape<NIN, EPT, MIXED>;
     const int p = (MIXED ? c : 2 * c) + 512 * j;
@@ -403,7 +425,7 @@ __device__ __forceinline__ void staged_pair(const Coefs &cf, const double *sb, d
         double e[NIN];
 #pragma unroll
         for (int k = 0; k < NIN; ++k) e[k] = v[k][q];
-        if constexpr (PM == 1) r[q] = Op::apply_fast(cf, e, q, away);
+        if constexpr (PM == 1) r[q] = Op::apply_fast(cf, e, q, l);
         else r[q] = Op::template apply<0>(cf, e);
     }
     if constexpr (MIXED) {
@@ -427,7 +449,7 @@ __device__ __noinline__ void staged_tile_fp64(double d0, double d1, double d2, d
     Coefs cf;  // the FP64 products read only the doubles
     cf.d[0] = d0, cf.d[1] = d1, cf.d[2] = d2, cf.d[3] = d3;
     cf.d[4] = d4, cf.d[5] = d5, cf.d[6] = d6, cf.d[7] = d7;
-    uint32_t none = 0;
+    Leave none;
     for (int j = 0; j < EPT / 2; ++j)
         staged_pair<Op, 0, EPT, MIXED>(cf, sb, out, len, c, j, odd, none);
 }
@@ -442,16 +464,18 @@ __device__ __noinline__ void staged_tile_fp64(double d0, double d1, double d2, d
 template <class Op, int PM, int EPT, bool MIXED>
 __device__ __forceinline__ bool staged_tile(const Coefs &cf, const double *sb, double *out, int len,
                                             int c, unsigned odd) {
-    uint32_t away = 0;
+    Leave l;
 #pragma unroll
     for (int j = 0; j < EPT / 2; ++j)
-        staged_pair<Op, PM, EPT, MIXED>(cf, sb, out, len, c, j, odd, away);
+        staged_pair<Op, PM, EPT, MIXED>(cf, sb, out, len, c, j, odd, l);
+    bool left = false;
     if constexpr (PM == 1) {
-        if ((int32_t)away < 0)
+        left = l.left(cf);
+        if (left)
             staged_tile_fp64<Op, EPT, MIXED>(cf.d[0], cf.d[1], cf.d[2], cf.d[3], cf.d[4], cf.d[5],
                                              cf.d[6], cf.d[7], sb, out, len, c, odd);
     }
-    return (int32_t)away < 0;
+    return left;
 }
 
 template <class Op, int EPT, bool MIXED>
@@ -541,7 +565,7 @@ __global__ void __launch_bounds__(kStagedThreads, (StageShape<Op::kIn, EPT, MIXE
             // element zero, maxpy with 4 terms, n = 2^26 (GB300): 1065 us
             // against 1557.
             bool left = false;
-            if ((int)slot < a.pm && fp64 == 0) 
+            if ((int)slot < a.pm && fp64 == 0)
                 left = staged_tile<Op, 1, EPT, MIXED>(a.cf, sb, out, len, threadIdx.x, a.odd);
             else staged_tile<Op, 0, EPT, MIXED>(a.cf, sb, out, len, threadIdx.x, a.odd);
             fp64 = __popc(__ballot_sync(0xffffffffu, left)) > 8 ? 16 : fp64 > 0 ? fp64 - 1 : 0;
@@ -630,14 +654,21 @@ int launch_ew(const double *const *in, double *out, int64_t n, const double *coe
     a.n = n;
     a.pm = pm;
     a.drop_tile = g_drop_tile.load();
+    uint32_t from = 0, to = ~0u;
     for (int k = 0; k < 8; ++k) {
         a.cf.d[k] = k < ncoef ? coef[k] : 0.0;
         uint64_t b;
         std::memcpy(&b, &a.cf.d[k], 8);
         a.cf.m[k] = mul_coef_of(b);
-        // a coefficient without an exponent window (zero, say): FP64 products
-        if (k < ncoef && a.cf.m[k].win == 0) a.pm = 0;
+        if (k < ncoef) {
+            from = std::max(from, a.cf.m[k].from);
+            to = std::min(to, a.cf.m[k].from + a.cf.m[k].span);
+        }
     }
+    // coefficients that share no range (one of them zero, say): FP64 products
+    a.cf.span = to > from ? to - from : 0u;
+    if (ncoef > 0 && a.cf.span == 0) a.pm = 0;
+    for (MulCoef &m : a.cf.m) m.from = from;
     cudaError_t e = injected_launch_error();
     if (e != cudaSuccess) return fail_cuda(e, "vector kernel launch");
     a.odd = 0;

@@ -89,3 +89,49 @@ def test_batches(entry, kind, shifts, lengths):
     with np.errstate(all="ignore"):
         want = np.repeat(alphas, lengths) * xh + yh  # two roundings, as the oracle's loop
     assert same(w.cpu().numpy(), want)
+
+
+# Lengths: less than a tile per SM; several tiles per warp, so that warps switch
+# to FP64 products or sums and back.
+@pytest.mark.parametrize("kind", KINDS)
+@pytest.mark.parametrize("n,shifts", [(4099, (0, 0, 0)), (100003, (0, 1, 2)), (6_000_001, (1, 1, 1)),
+                                      (6_000_001, (0, 1, 0))])
+def test_streaming_siblings(n, shifts, kind):
+    xh, yh, zh = (data(k, n, 41 + j) for j, k in enumerate((kind, "uniform", "uniform")))
+    x, y, z = (at(v, s) for v, s in zip((xh, yh, zh), shifts))
+    for c in ((0.7, -0.2, 0.3), (2.0 ** 600, 1e-300, -1.0), (0.5, 0.0, 1e308)):
+        with np.errstate(all="ignore"):
+            want2, want3 = oracle.axpby(c[0], c[1], xh, yh), oracle.axpbypcz(*c, xh, yh, zh)
+        y2, z3 = at(yh, shifts[1]), at(zh, shifts[2])
+        wx.wxpy_axpby(c[0], c[1], x, y2)
+        wx.wxpy_axpbypcz(*c, x, y, z3)
+        assert same(y2.cpu().numpy(), want2) and same(z3.cpu().numpy(), want3), c
+    wx.wxpy_vecops_status()  # no wait ran out
+
+
+@pytest.mark.parametrize("m", [2, 3, 4, 5, 6, 7, 8])
+@pytest.mark.parametrize("kind,scale", [("uniform", 1e-12), ("uniform", 2.0 ** -31), ("uniform", 1e12),
+                                        ("y zero", 1.0), ("y infinite", 1.0), ("cancelling", 1.0),
+                                        ("mixed", 1.0), ("sevenths", 1e-12), ("spread", 1.0)])
+@pytest.mark.parametrize("n,shifts", [(4099, (0, 0)), (2_000_003, (0, 0)), (2_000_003, (1, 0))])
+def test_maxpy_sums(n, shifts, m, kind, scale):
+    """Terms far below and above the vector they are added to, a zero vector, and
+    sums that cancel: the integer sums leave their path in some elements or all."""
+    special = kind if kind in KINDS else "uniform"
+    xs = [data(special if j == 1 else "uniform", n, 51 + j) * scale for j in range(m)]
+    yh = data("uniform", n, 50)
+    al = [0.75, -1.5, 1.25, -0.625, 1.875, -0.3125, 0.5625, -1.0625][:m]
+    if kind == "y zero":
+        yh[:] = 0.0
+        yh[::3] = -0.0
+    elif kind == "y infinite":
+        yh[1::5] = np.inf
+    elif kind == "cancelling":
+        for j in range(1, m):
+            xs[j][::2] = xs[j - 1][::2] * (-al[j - 1] / al[j]) * (1 + 2.0 ** -40)
+    with np.errstate(all="ignore"):
+        want = oracle.maxpy(al, xs, yh)
+    y = at(yh, shifts[0])
+    wx.wxpy_maxpy(al, [at(v, shifts[1]) for v in xs], y)
+    assert same(y.cpu().numpy(), want)
+    wx.wxpy_vecops_status()  # no wait ran out
