@@ -172,15 +172,19 @@ WX_MUL_FN uint64_t mul_rn_quick(const MulCoef &c, uint64_t ub, uint32_t &away) {
     return round_product(top, (uint32_t)x, (uint32_t)p00, c.k + (bh & 0xFFF00000u), &t);
 }
 
-// The same over the whole range of operands whose product is in the normal range
-// whatever t and the rounding: `far` becomes the largest distance of their
-// exponent fields above the range's first (modulo 2^32, so a field below it is
-// far as well), and the products made so far are meaningless once it is
-// c.span or more.  One coefficient for all of them.
+// How far b's exponent field lies above the first of the range of operands whose
+// product with the coefficient is in the normal range whatever t and the rounding
+// (modulo 2^32, so a field below it is far as well); c.span or more: outside.
+WX_MUL_FN uint32_t mul_distance(const MulCoef &c, uint64_t ub) {
+    return ((uint32_t)(ub >> 32) << 1) - c.from;
+}
+
+// The same product over that whole range: `far` becomes the largest distance so
+// far, and the products made are meaningless once it is c.span or more.
 WX_MUL_FN uint64_t mul_rn_range(const MulCoef &c, uint64_t ub, uint32_t &far) {
     const uint32_t bh = (uint32_t)(ub >> 32), bl = (uint32_t)ub;
     const uint32_t b1 = (bh & 0xFFFFFu) | 0x100000u;
-    const uint32_t d = (bh << 1) - c.from;
+    const uint32_t d = mul_distance(c, ub);
     far = d > far ? d : far;
     const uint64_t p00 = (uint64_t)c.lo * bl;
     const uint64_t x = (uint64_t)c.hi * bl + (uint64_t)c.lo * b1 + (p00 >> 32);

@@ -87,11 +87,11 @@ enum Deal {
 //              to the end of the row, and only its accesses are single ones
 //   kElements  positions 128 warp + lane + 32 q, so that the 8-byte accesses of
 //              a warp are contiguous
-template <int KIND, bool EMU, int DEAL, bool EARLY>
+template <int KIND, int MODE, int DEAL, bool EARLY>
 __device__ __forceinline__ void row_terms(const ReduceArgs &a, int64_t row, double (&t)[4],
                                           bool &left) {
     if constexpr (DEAL == kVectors) {
-        vector_terms<KIND, EMU, true, EARLY>(a, row + 4 * threadIdx.x, t, left);
+        vector_terms<KIND, MODE, true, EARLY>(a, row + 4 * threadIdx.x, t, left);
     } else if constexpr (DEAL == kShifted) {
         const int64_t i = row + 4 * (int)threadIdx.x - a.shift;
         double x[4], y[4], z[4], w[4];
@@ -108,7 +108,7 @@ __device__ __forceinline__ void row_terms(const ReduceArgs &a, int64_t row, doub
                 if constexpr (KIND == 1) z[q] = a.z[e];
             }
         }
-        elements4<KIND, EMU, EARLY>(a, x, y, z, w, t, left);
+        elements4<KIND, MODE, EARLY>(a, x, y, z, w, t, left);
         if (threadIdx.x != 0) {
             st4(a.w + i, w);
         } else {
@@ -117,7 +117,11 @@ __device__ __forceinline__ void row_terms(const ReduceArgs &a, int64_t row, doub
         }
     } else {
         const int64_t i0 = row + 128 * (threadIdx.x >> 5) + (threadIdx.x & 31);
-        constexpr int G = EMU ? 2 : 1;  // elements loaded together
+        constexpr int G = MODE != kFp64 ? 2 : 1;  // elements loaded together
+        // Single elements have no test for four x at once.  norm2 takes one for each
+        // product: every seventh element zero, n = 2^26, 440 us against 563, and
+        // 364 against 361 without.  dot has no register for it (515 against 428).
+        constexpr int kOf = MODE == kInteger && KIND == 0 ? (int)kIntegerEach : MODE;
 #pragma unroll
         for (int g = 0; g < 4; g += G) {
             double x[G], y[G], z[G];
@@ -136,7 +140,7 @@ __device__ __forceinline__ void row_terms(const ReduceArgs &a, int64_t row, doub
                 t[g + q] = 0.0;
                 if (i < a.n) {
                     double w;
-                    element<KIND, EMU>(a, x[q], y[q], KIND == 1 ? z[q] : 0.0, w, t[g + q], left);
+                    element<KIND, kOf>(a, x[q], y[q], KIND == 1 ? z[q] : 0.0, w, t[g + q], left);
                     a.w[i] = w;
                 }
             }
@@ -148,8 +152,8 @@ __device__ __forceinline__ void row_terms(const ReduceArgs &a, int64_t row, doub
 // the node of position p of the rows at red[p]; node: 128 doubles.
 // SUML (norm2 only): the first SUML of the three in-thread tree levels run as
 // integer-pipeline sums of non-negative values.  *left: the threads with an
-// element off the integer products' fast path.
-template <int KIND, int DEAL, bool EMU, int SUML = 0, bool EARLY = false>
+// element off the integer products' fast path (see elements4).
+template <int KIND, int DEAL, int MODE, int SUML = 0, bool EARLY = false>
 __device__ double tile_sum(const ReduceArgs &a, int64_t tile, double *red, double *node, int *left) {
     static_assert(SUML == 0 || KIND == 0, "integer tree sums need non-negative terms");
     const int t = threadIdx.x, lane = t & 31;
@@ -167,8 +171,8 @@ __device__ double tile_sum(const ReduceArgs &a, int64_t tile, double *red, doubl
         for (int m = 0; m < 2; ++m) {
             const int j = h + 2 * m;
             double lo[4], hi[4];
-            row_terms<KIND, EMU, DEAL, EARLY>(a, t0 + 1024 * j, lo, mine);
-            row_terms<KIND, EMU, DEAL, EARLY>(a, t0 + 1024 * (j + 4), hi, mine);
+            row_terms<KIND, MODE, DEAL, EARLY>(a, t0 + 1024 * j, lo, mine);
+            row_terms<KIND, MODE, DEAL, EARLY>(a, t0 + 1024 * (j + 4), hi, mine);
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
                 rp[q] = rc[q];
@@ -217,28 +221,45 @@ __device__ double tile_sum(const ReduceArgs &a, int64_t tile, double *red, doubl
 // the block and bits 6..0 on four values per lane took 51 warp instructions
 // and four block barriers more per tile, of which 36 and one are left:
 // norm2 at n = 2^26 (GB300) went from 309 to 289 us.
-template <int KIND, int DEAL, int SUML, bool EARLY>
+//
+// ALL: every full tile with integer products (mul_sixteenths 16, the default).
+// Data that keeps leaving their fast path pays for both kinds of product: after a
+// tile where a quarter of the threads did, the block takes other ones for sixteen
+// tiles.  With a test before the update's products (EARLY, see elements4) it is
+// the terms that left, infinities say, and both products move to FP64.  Without,
+// it is x more often than not, zeros say, and only the update's product moves:
+// three FP64 operations per element against four.  Every seventh element zero,
+// n = 2^26, norm2 / dot: 434 / 433 us, against 553 / 536 with both products moved
+// in either case, and 443 / 448 with a test per product everywhere.
+//
+// The last, ragged tile follows the loop: in it, and with the choice by tile that
+// ALL leaves out, norm2 took 298 us for the 282 it takes.
+template <int KIND, int DEAL, int SUML, bool EARLY, bool ALL>
 __global__ void __launch_bounds__(kThreads, 4) wxpy_reduce_kernel(const ReduceArgs a) {
+    constexpr int kOther = ALL && !EARLY && DEAL != kElements ? kTermInteger : kFp64;
     __shared__ __align__(16) double red[2][1024];  // two tiles in turn: one block barrier per tile
     __shared__ double node[128];
     pdl_enter();
     const int64_t full = a.n / kTile;        // tiles with every element present
     unsigned slot = (blockIdx.x * 7u) & 15u;  // block-uniform rotation of the pipe choice
-    int turn = 0, fp64 = 0;
-    for (int64_t tile = blockIdx.x; tile < a.ntiles; tile += gridDim.x, turn ^= 1) {
+    int turn = 0, other = 0;
+    for (int64_t tile = blockIdx.x; tile < full; tile += gridDim.x, turn ^= 1) {
         double s;
         int left = 0;
-        if (tile >= full) s = tile_sum<KIND, kElements, false>(a, tile, red[turn], node, &left);
-        else if ((int)slot < a.mul_sixteenths && fp64 == 0)
-            s = tile_sum<KIND, DEAL, true, SUML, EARLY>(a, tile, red[turn], node, &left);
-        else s = tile_sum<KIND, DEAL, false, SUML>(a, tile, red[turn], node, &left);
-        // Data that keeps leaving the fast path (zeros, say) pays for both kinds of
-        // product: after a tile where a quarter of the threads did, the block takes
-        // FP64 products for sixteen tiles.  Every seventh element zero, n = 2^26:
-        // 552 us against 683 without, and 576 before with a test per product.
-        fp64 = left > kThreads / 4 ? 16 : fp64 > 0 ? fp64 - 1 : 0;
+        if (other > 0 || (!ALL && (int)slot >= a.mul_sixteenths)) {
+            s = tile_sum<KIND, DEAL, kOther, SUML>(a, tile, red[turn], node, &left);
+            other -= other > 0;
+        } else {
+            s = tile_sum<KIND, DEAL, kInteger, SUML, EARLY>(a, tile, red[turn], node, &left);
+            if (left > kThreads / 4) other = 16;
+        }
         if (threadIdx.x == 0) a.partial[tile] = s;
-        slot = (slot + 1u) & 15u;
+        if (!ALL) slot = (slot + 1u) & 15u;
+    }
+    if (full < a.ntiles && full % gridDim.x == blockIdx.x) {
+        int left = 0;
+        const double s = tile_sum<KIND, kElements, kFp64>(a, full, red[turn], node, &left);
+        if (threadIdx.x == 0) a.partial[full] = s;
     }
 }
 
@@ -539,10 +560,10 @@ cudaError_t launch_staged(const ReduceArgs &a, const DeviceProps *dp, cudaStream
     return cudaGetLastError();
 }
 
-template <int KIND, int DEAL, int SUML, bool EARLY>
-cudaError_t launch_block(const ReduceArgs &a, const DeviceProps *dp, cudaStream_t s) {
+template <int KIND, int DEAL, int SUML, bool EARLY, bool ALL>
+cudaError_t launch_block_form(const ReduceArgs &a, const DeviceProps *dp, cudaStream_t s) {
     static std::atomic<int> cached[64];
-    auto kernel = &wxpy_reduce_kernel<KIND, DEAL, SUML, EARLY>;
+    auto kernel = &wxpy_reduce_kernel<KIND, DEAL, SUML, EARLY, ALL>;
     const int dev = dp->device;
     int nb = dev >= 0 && dev < 64 ? cached[dev].load(std::memory_order_relaxed) : 0;
     if (nb <= 0) {
@@ -555,6 +576,12 @@ cudaError_t launch_block(const ReduceArgs &a, const DeviceProps *dp, cudaStream_
     }
     const int64_t grid = std::max<int64_t>(1, std::min<int64_t>((int64_t)dp->sm_count * nb, a.ntiles));
     return launch_pdl(kernel, (unsigned)grid, kThreads, s, a);
+}
+
+template <int KIND, int DEAL, int SUML, bool EARLY>
+cudaError_t launch_block(const ReduceArgs &a, const DeviceProps *dp, cudaStream_t s) {
+    return a.mul_sixteenths == 16 ? launch_block_form<KIND, DEAL, SUML, EARLY, true>(a, dp, s)
+                                  : launch_block_form<KIND, DEAL, SUML, EARLY, false>(a, dp, s);
 }
 
 std::atomic<int> g_reduce_mul{-1};
@@ -652,8 +679,8 @@ int launch_reduce(int64_t n, double alpha, const double *x, const double *y, dou
     uint64_t ab;
     std::memcpy(&ab, &alpha, 8);
     a.ca = mul_coef_of(ab);
-    // an alpha without an exponent window (zero, say): FP64 products
-    a.mul_sixteenths = a.ca.win != 0 ? cfg.mul : 0;
+    // an alpha without a range of operands (zero, say): FP64 products
+    a.mul_sixteenths = a.ca.span != 0 ? cfg.mul : 0;
     a.drop_chunk = g_reduce_drop.load();
     uintptr_t any = (uintptr_t)x | (uintptr_t)y | (uintptr_t)w | (KIND == 1 ? (uintptr_t)z : 0);
     const bool vec = (any & 31u) == 0;
@@ -667,12 +694,14 @@ int launch_reduce(int64_t n, double alpha, const double *x, const double *y, dou
         if (e == cudaSuccess && a.ntiles == 1) return WXPY_OK;
     } else if (variant == 0) {
         const int suml = KIND == 0 && vec ? std::min(cfg.suml, 3) : 0;  // the in-thread levels
-        // blocks of a tile or two: the early test (elements4)
-        const bool brief = a.ntiles <= 8 * (int64_t)dp->sm_count;
+        // The early test (elements4) in norm2 of four tiles per block and fewer, where
+        // it costs nothing and most tiles of a block would be ones that find out:
+        // 2^24 elements 83 / 85 us without / with it, every seventh zero 134 / 115.
+        const bool brief = a.ntiles <= 16 * (int64_t)dp->sm_count;
         if (!vec) {
-            e = !same   ? launch_block<KIND, kElements, 0, false>(a, dp, s)
-                : brief ? launch_block<KIND, kShifted, 0, true>(a, dp, s)
-                        : launch_block<KIND, kShifted, 0, false>(a, dp, s);
+            if (!same) e = launch_block<KIND, kElements, 0, false>(a, dp, s);
+            else if (KIND == 1 || brief) e = launch_block<KIND, kShifted, 0, true>(a, dp, s);
+            else if constexpr (KIND == 0) e = launch_block<KIND, kShifted, 0, false>(a, dp, s);
         } else if constexpr (KIND == 0) {
             e = suml == 0   ? (brief ? launch_block<0, kVectors, 0, true>(a, dp, s)
                                      : launch_block<0, kVectors, 0, false>(a, dp, s))

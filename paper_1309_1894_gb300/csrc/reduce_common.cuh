@@ -79,21 +79,47 @@ static __device__ __noinline__ ulonglong2 element_hw_bits(uint64_t alpha, uint64
     return make_ulonglong2(bits_of(w), bits_of(t));
 }
 
-// w and the term of one element.  EMU: both products in the integer pipelines,
-// with one fallback test for the element.  At n = 2^26 (GB300) the windowed
-// products with one test run norm2 / dot at 0.75 / 0.89 of the measured peak,
-// against 0.72 / 0.84 with the fully checked products and a test for each.
-// `left` is set when the element left the fast path.
-template <int KIND, bool EMU>
+static __device__ __noinline__ uint64_t mul_hw_bits(uint64_t ua, uint64_t ub) {
+    return bits_of(__dmul_rn(double_of(ua), double_of(ub)));
+}
+
+// Where an element's two products run: both on the FP64 pipeline, both in the
+// integer pipelines, or the term's alone there.
+enum Products : int { kFp64, kInteger, kIntegerEach, kTermInteger };
+
+// w and the term of one element.  kInteger: one fallback test for the element,
+// and `left` set when it left the fast path.  At n = 2^26 (GB300) products with
+// one test run norm2 / dot at 0.75 / 0.89 of the measured peak, against
+// 0.72 / 0.84 with the fully checked products and a test for each.  kIntegerEach:
+// a test for each all the same, so that x outside the range (zeros, say) pays for
+// no second sum, and `left` set by the term's alone.
+template <int KIND, int MODE>
 __device__ __forceinline__ void element(const ReduceArgs &a, double x, double y, double z,
                                         double &w, double &t, bool &left) {
-    if constexpr (EMU) {
-        uint32_t away = 0;
+    if constexpr (MODE == kTermInteger || MODE == kIntegerEach) {
+        if constexpr (MODE == kTermInteger) {
+            w = __dadd_rn(__dmul_rn(a.alpha, x), y);
+        } else {
+            uint32_t far = 0;
+            uint64_t pb = mul_rn_range(a.ca, bits_of(x), far);
+            if (far >= a.ca.span) pb = mul_hw_bits(bits_of(a.alpha), bits_of(x));
+            w = __dadd_rn(double_of(pb), y);
+        }
+        const uint64_t wb = opaque_bits(w), zb = KIND == 0 ? wb : bits_of(z);
         bool slow = false;
-        w = __dadd_rn(double_of(mul_rn_quick(a.ca, bits_of(x), away)), y);
+        uint64_t tb = KIND == 0 ? sqr_rn_core(wb, slow) : mul_rn_quick2(wb, zb, slow);
+        if (slow) {
+            tb = mul_hw_bits(wb, zb);
+            left = true;
+        }
+        t = double_of(tb);
+    } else if constexpr (MODE == kInteger) {
+        uint32_t far = 0;
+        bool slow = false;
+        w = __dadd_rn(double_of(mul_rn_range(a.ca, bits_of(x), far)), y);
         const uint64_t wb = opaque_bits(w);
         t = double_of(KIND == 0 ? sqr_rn_core(wb, slow) : mul_rn_quick2(wb, bits_of(z), slow));
-        if (slow || (int32_t)away < 0) {
+        if (slow || far >= a.ca.span) {
             const ulonglong2 r =
                 element_hw_bits<KIND>(bits_of(a.alpha), bits_of(x), bits_of(y), bits_of(z));
             w = double_of(r.x);
@@ -110,35 +136,28 @@ template <int KIND, bool EMU>
 __device__ __forceinline__ void element(const ReduceArgs &a, double x, double y, double z,
                                         double &w, double &t) {
     bool left;
-    element<KIND, EMU>(a, x, y, z, w, t, left);
+    element<KIND, EMU ? kInteger : kFp64>(a, x, y, z, w, t, left);
 }
 
-static __device__ __noinline__ uint64_t mul_hw_bits(uint64_t ua, uint64_t ub) {
-    return bits_of(__dmul_rn(double_of(ua), double_of(ub)));
-}
-
-// w and the terms of four elements.  EARLY: the window of the four x is tested
-// before their products, so that data outside it (zeros, say) pays for no second
-// update sum; it costs norm2 4 % on data inside (n = 2^26, 291 against 303 us),
-// dot nothing (both 3-4 % on vectors past the boundary).  Without it, element() by element, a grid of a tile or two per
-// block has no next tile to take with FP64 products: every seventh element zero,
-// 2^22 elements, norm2 / dot 56 / 57 us, with it 47 / 48.
-template <int KIND, bool EMU, bool EARLY>
+// w and the terms of four elements.  EARLY (of kInteger): the range of the four x
+// is tested before their products, so that data outside it (zeros, say) pays for
+// no second update sum, and `left` is set by the terms' products alone.  It costs
+// norm2 on data inside 2 % at 2^25 elements and 4 % at 2^26, dot nothing.
+template <int KIND, int MODE, bool EARLY>
 __device__ __forceinline__ void elements4(const ReduceArgs &a, const double (&x)[4],
                                           const double (&y)[4], const double (&z)[4],
                                           double (&w)[4], double (&t)[4], bool &left) {
-    if constexpr (EMU && EARLY) {
-        uint32_t away = 0;
+    if constexpr (MODE == kInteger && EARLY) {
+        uint32_t far = 0;
 #pragma unroll
-        for (int q = 0; q < 4; ++q) away |= ((uint32_t)(bits_of(x[q]) >> 32) << 1) - a.ca.win;
+        for (int q = 0; q < 4; ++q) far = max(far, mul_distance(a.ca, bits_of(x[q])));
         uint64_t pb[4];
-        if ((int32_t)away < 0) {
+        if (far >= a.ca.span) {
 #pragma unroll
             for (int q = 0; q < 4; ++q) pb[q] = mul_hw_bits(bits_of(a.alpha), bits_of(x[q]));
-            left = true;
         } else {
 #pragma unroll
-            for (int q = 0; q < 4; ++q) pb[q] = mul_rn_quick(a.ca, bits_of(x[q]), away);
+            for (int q = 0; q < 4; ++q) pb[q] = mul_rn_range(a.ca, bits_of(x[q]), far);
         }
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
@@ -155,7 +174,7 @@ __device__ __forceinline__ void elements4(const ReduceArgs &a, const double (&x)
     } else {
 #pragma unroll
         for (int q = 0; q < 4; ++q)
-            element<KIND, EMU>(a, x[q], y[q], KIND == 1 ? z[q] : 0.0, w[q], t[q], left);
+            element<KIND, MODE>(a, x[q], y[q], KIND == 1 ? z[q] : 0.0, w[q], t[q], left);
     }
 }
 
@@ -175,7 +194,7 @@ __device__ __forceinline__ void st4(double *p, const double (&v)[4]) {
 // Terms of the four elements base .. base + 3; w stored.  VEC: one 32-byte
 // co-aligned vector of every operand; else element by element with bounds,
 // +0 terms past n.
-template <int KIND, bool EMU, bool VEC, bool EARLY = false>
+template <int KIND, int MODE, bool VEC, bool EARLY = false>
 __device__ __forceinline__ void vector_terms(const ReduceArgs &a, int64_t base, double (&t)[4],
                                              bool &left) {
     if constexpr (VEC) {
@@ -183,7 +202,7 @@ __device__ __forceinline__ void vector_terms(const ReduceArgs &a, int64_t base, 
         ld4(a.x + base, x);
         ld4(a.y + base, y);
         if constexpr (KIND == 1) ld4(a.z + base, z);
-        elements4<KIND, EMU, EARLY>(a, x, y, z, w, t, left);
+        elements4<KIND, MODE, EARLY>(a, x, y, z, w, t, left);
         st4(a.w + base, w);
     } else {
 #pragma unroll
@@ -192,7 +211,7 @@ __device__ __forceinline__ void vector_terms(const ReduceArgs &a, int64_t base, 
             if (i < a.n) {
                 const double zi = KIND == 1 ? a.z[i] : 0.0;
                 double wi;
-                element<KIND, EMU>(a, a.x[i], a.y[i], zi, wi, t[q]);
+                element<KIND, MODE>(a, a.x[i], a.y[i], zi, wi, t[q], left);
                 a.w[i] = wi;
             } else {
                 t[q] = 0.0;
@@ -204,7 +223,7 @@ __device__ __forceinline__ void vector_terms(const ReduceArgs &a, int64_t base, 
 template <int KIND, bool EMU, bool VEC>
 __device__ __forceinline__ void vector_terms(const ReduceArgs &a, int64_t base, double (&t)[4]) {
     bool left;
-    vector_terms<KIND, EMU, VEC>(a, base, t, left);
+    vector_terms<KIND, EMU ? kInteger : kFp64, VEC>(a, base, t, left);
 }
 
 // Bits 6..0 of a tile's tree, by one warp, from the 128 node values that bits

@@ -135,3 +135,48 @@ def test_maxpy_sums(n, shifts, m, kind, scale):
     wx.wxpy_maxpy(al, [at(v, shifts[1]) for v in xs], y)
     assert same(y.cpu().numpy(), want)
     wx.wxpy_vecops_status()  # no wait ran out
+
+
+# Tiles of 8192 elements: the cluster form; the block form with one tile and with
+# a few per block, whose later tiles take other products where the earlier ones
+# left the integer pipelines; every way the offsets deal the elements.
+@pytest.mark.parametrize("kind", KINDS)
+@pytest.mark.parametrize("tiles", [2, 130, 300, 2500])
+@pytest.mark.parametrize("shifts", [(0, 0, 0, 0), (1, 1, 1, 1), (0, 1, 2, 3)])
+def test_reductions(tiles, shifts, kind):
+    n = tiles * 8192 - 100
+    xh, yh, zh = (data(k, n, 61 + j) for j, k in enumerate((kind, "uniform", "uniform")))
+    x, y, z = (at(v, s) for v, s in zip((xh, yh, zh), shifts))
+    w = at(np.zeros(n), shifts[3])
+    for alpha in (0.7, 0.0) if tiles > 1000 else (0.7, -2.0 ** 600, 3e-308, 0.0):
+        with np.errstate(all="ignore"):
+            (w2, n2), (w3, d3) = oracle.wxpy_norm2(alpha, xh, yh), oracle.wxpy_dot(alpha, xh, yh, zh)
+        _, r = wx.wxpy_norm2(alpha, x, y, w=w)
+        assert same(w.cpu().numpy(), w2) and same(r.cpu().numpy(), np.array([n2])), alpha
+        _, r = wx.wxpy_dot(alpha, x, y, z, w=w)
+        assert same(w.cpu().numpy(), w3) and same(r.cpu().numpy(), np.array([d3])), alpha
+
+
+@pytest.mark.parametrize("shifts", [(0, 0, 0, 0), (1, 1, 1, 1), (0, 1, 2, 3)])
+def test_reductions_change_products_and_back(shifts):
+    """A stretch of zeros, one of infinities, ordinary data before, between and
+    after: every block meets each, and the terms' products leave in one alone."""
+    n = 5000 * 8192 + 7
+    xh, yh, zh = (data("uniform", n, 71 + j) for j in range(3))
+    xh[n // 5:2 * n // 5] = 0.0
+    xh[n // 2:n // 2 + 100] = np.inf
+    zh[3 * n // 5:4 * n // 5:2] = 0.0
+    yh[n // 5:n // 4] = 0.0
+    x, y, z = (at(v, s) for v, s in zip((xh, yh, zh), shifts))
+    w = at(np.zeros(n), shifts[3])
+    with np.errstate(all="ignore"):
+        (w2, n2), (w3, d3) = oracle.wxpy_norm2(0.7, xh, yh), oracle.wxpy_dot(0.7, xh, yh, zh)
+    for mul in (-1, 16, 8):
+        wx.wxpy_reduce_pipes(mul)
+        try:
+            _, r = wx.wxpy_norm2(0.7, x, y, w=w)
+            assert same(w.cpu().numpy(), w2) and same(r.cpu().numpy(), np.array([n2])), mul
+            _, r = wx.wxpy_dot(0.7, x, y, z, w=w)
+            assert same(w.cpu().numpy(), w3) and same(r.cpu().numpy(), np.array([d3])), mul
+        finally:
+            wx.wxpy_reduce_pipes(-1)
