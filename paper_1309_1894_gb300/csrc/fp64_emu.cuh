@@ -236,19 +236,37 @@ __device__ __forceinline__ void wxpy_vec_emu(double alpha, const double (&x)[VW]
     }
 }
 
+// How a vector of integer-pipeline products tells operands that it leaves out.
+// kTestEach: a test for each product, over its whole range of operands.  A
+// product's sum waits for its own x alone, which is what the single-call kernels
+// want, whose threads have one or two vectors: 2^20 elements 4.31 us on GB300, 16
+// bytes off 4.34, against 4.52 and 5.41 with one test for the vector.
+// kTestVector: one test for the vector, over the same range, in the batched
+// kernel's wide body: 4096 segments up to 2^18, 316 us, with every seventh element
+// zero 383, against 317 and 405.  kTestWindow: one test for the vector and half
+// the exponents (mul_rn_quick), in the batched body with three resident blocks,
+// which has no register to spare for more.
+enum ProductTest { kTestEach, kTestVector, kTestWindow };
+
 // The same with alpha's split `ca` at hand: EMU == 3 computes every product
-// RN(alpha*x) in the integer pipelines (fp64_mul.cuh; a vector with an operand
-// it leaves out takes the hardware multiply, out of line) and every sum on the
-// FP64 pipeline, which then carries one instruction per element.  The products
-// take every operand whose product is in the normal range, so that data of
-// 2^512 and more (an iteration that diverges, say) runs at the speed of any
-// other: 2^26 elements of 1e200 221 us on GB300, against 261 with the window of
-// mul_rn_quick, 2^20 4.5 against 6.6.  WINDOW: that window all the same, where
-// a kernel has no register to spare for the longer test.
-template <int VW, int EMU, bool WINDOW = false>
+// RN(alpha*x) in the integer pipelines (fp64_mul.cuh; operands it leaves out take
+// the hardware multiply, out of line) and every sum on the FP64 pipeline, which
+// then carries one instruction per element.
+template <int VW, int EMU, ProductTest TEST = kTestEach>
 __device__ __forceinline__ void wxpy_vec_emu(double alpha, const MulCoef &ca, const double (&x)[VW],
                                              const double (&y)[VW], double (&w)[VW], int base) {
-    if constexpr (EMU == 3) {
+    if constexpr (EMU == 3 && TEST == kTestEach) {
+#pragma unroll
+        for (int k = 0; k < VW; ++k) {
+            const uint64_t xb = (uint64_t)__double_as_longlong(x[k]);
+            uint32_t far = 0;
+            uint64_t p = mul_rn_range(ca, xb, far);
+            if (far >= ca.span) p = mul_rn_hw_bits((uint64_t)__double_as_longlong(alpha), xb);
+            w[k] = __dadd_rn(__longlong_as_double((long long)p), y[k]);
+        }
+    } else if constexpr (EMU == 3) {
+        static_assert(VW % 2 == 0, "the fallback takes two at a time");
+        constexpr bool WINDOW = TEST == kTestWindow;
         uint32_t far = WINDOW && ca.win == 0 ? 1u << 31 : 0u;
         uint64_t p[VW];
 #pragma unroll
@@ -260,14 +278,10 @@ __device__ __forceinline__ void wxpy_vec_emu(double alpha, const MulCoef &ca, co
             const uint64_t ab = (uint64_t)__double_as_longlong(alpha);
 #pragma unroll
             for (int k = 0; k < VW; k += 2) {  // out of line
-                if constexpr (VW == 1) {
-                    p[k] = mul_rn_hw_bits(ab, (uint64_t)__double_as_longlong(x[k]));
-                } else {
-                    const ulonglong2 r = mul2_rn_hw_bits(ab, (uint64_t)__double_as_longlong(x[k]),
-                                                         (uint64_t)__double_as_longlong(x[k + 1]));
-                    p[k] = r.x;
-                    p[k + 1] = r.y;
-                }
+                const ulonglong2 r = mul2_rn_hw_bits(ab, (uint64_t)__double_as_longlong(x[k]),
+                                                     (uint64_t)__double_as_longlong(x[k + 1]));
+                p[k] = r.x;
+                p[k + 1] = r.y;
             }
         }
 #pragma unroll

@@ -21,13 +21,13 @@ namespace wx {
 // of 256 threads) or, for batches of long tiles, four (two blocks).
 constexpr int kTileU = 2, kTileWideU = 4;
 
-// Whether the integer-pipeline products take the operands of a window only (see
-// wxpy_vec_emu).  Three resident blocks leave no register for the test of the
-// whole range: with it 1024 segments up to 2^16 stored back to back took 34.8 us
-// without a host's plan and 27.6 with one, against 34.1 and 27.3 (GB300), while
-// the wide body takes it at no cost.
+// How the integer-pipeline products test their operands (see ProductTest).  Three
+// resident blocks leave no register for the test of the whole range: with it 1024
+// segments up to 2^16 stored back to back took 34.8 us without a host's plan and
+// 27.6 with one, against 34.1 and 27.3 (GB300), while the wide body takes it at no
+// cost.
 template <int MAXU>
-constexpr bool kWindow = MAXU == kTileU;
+constexpr ProductTest kTileTest = MAXU == kTileU ? kTestWindow : kTestVector;
 
 __device__ __forceinline__ void tile_scalar(const double *x, const double *y, double *w,
                                             double alpha, int64_t e) {
@@ -61,7 +61,7 @@ __device__ __forceinline__ void tile_body4(const double *x, const double *y, dou
         for (int u = 0; u < MAXU; ++u) {
             const int64_t c = c0 + 32 * u;
             if (u < U && c < nch) {
-                wxpy_vec_emu<4, EMU, kWindow<MAXU>>(alpha, ca, xv[u], yv[u], wv[u], 0);
+                wxpy_vec_emu<4, EMU, kTileTest<MAXU>>(alpha, ca, xv[u], yv[u], wv[u], 0);
                 st_vec<4, 2>(w + c * 4, wv[u]);
             }
         }
@@ -93,7 +93,7 @@ __device__ __forceinline__ void tile_elements(const double *x, const double *y, 
 #pragma unroll
         for (int g = 0; g < kTileElems / 4; ++g) {
             double wv[4];
-            wxpy_vec_emu<4, EMU, kWindow<kTileU>>(alpha, ca, xv[g], yv[g], wv, 0);
+            wxpy_vec_emu<4, EMU, kTileTest<kTileU>>(alpha, ca, xv[g], yv[g], wv, 0);
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
                 const int64_t e = e0 + 32 * (4 * g + u);
