@@ -302,16 +302,20 @@ typedef struct wxpy_vecops_tune_result {
  * pristine inputs and compared with it bit for bit -- a single differing bit
  * rejects it -- and timed as the median of five runs of three back-to-back
  * calls, each run after an L2 flush.
- * The fastest verified split becomes the class's split for later calls that
- * leave wxpy_vecops_pipes at -1, and is saved and loaded with the tune cache
+ * The fastest verified split -- the default, unless a candidate is more than
+ * half a percent faster -- becomes the class's split for later calls that leave
+ * wxpy_vecops_pipes at -1 and fall into the same size range as n: below 2^23
+ * elements, where the L2 serves most of a call, or from there on.  Search both
+ * sizes to tune both.  It is saved and loaded with the tune cache
  * (wxpy_tune_cache_save / _load).  `results` (WXPY_VEC_CLASSES entries) may
  * be NULL.  Allocates about 11 n doubles of scratch while it runs, on the
  * current device.  Errors: WXPY_EINVAL (n <= 0), WXPY_ENOMEM, WXPY_ECUDA,
  * WXPY_EMISMATCH (every candidate of a class rejected). */
 int wxpy_vecops_tune(int64_t n, wxpy_vecops_tune_result *results);
 
-/* The searched split of a class (-1, -1 when not searched); set installs one
- * (add 0..2, mul 0..16) or clears it (-1, -1). */
+/* The searched split of a class (-1, -1 when not searched), of the size range
+ * stored last; set installs one (add 0..2, mul 0..16) for every size, or clears
+ * both ranges (-1, -1). */
 int wxpy_vecops_tuned_get(int op_class, int *add_offload, int *mul_sixteenths);
 int wxpy_vecops_tuned_set(int op_class, int add_offload, int mul_sixteenths);
 
@@ -407,15 +411,18 @@ typedef struct wxpy_reduce_tune_result {
  * integer tree levels in the fastest warp-tiled shape) is run once and compared with it bit for bit -- a single
  * differing bit of w or of the result rejects it -- and timed as the median
  * of five runs of three back-to-back calls, each run after an L2 flush.  The fastest verified configuration
- * becomes the operation's configuration for later calls whose knobs are left
- * at -1, and is saved and loaded with the tune cache.  `results` (2 entries)
+ * -- the default, unless a candidate is more than half a percent faster -- becomes
+ * the operation's configuration for later calls whose knobs are left at -1 and that
+ * fall into the same size range as n: up to 2^21 elements, where kernel 0 takes its
+ * cluster form, or above.  It is saved and loaded with the tune cache.  `results` (2 entries)
  * may be NULL.  Allocates about 5 n doubles of scratch while it runs, on the
  * current device.  Errors: WXPY_EINVAL (n <= 0), WXPY_ENOMEM, WXPY_ECUDA,
  * WXPY_EMISMATCH (every configuration rejected). */
 int wxpy_reduce_tune(int64_t n, wxpy_reduce_tune_result *results);
 
 /* The searched configuration of a reduction (kind 0 norm2, 1 dot; all -1
- * when not searched); set installs one or clears it (all -1). */
+ * when not searched), of the size range stored last; set installs one for every
+ * size, or clears both ranges (all -1). */
 int wxpy_reduce_tuned_get(int kind, int *variant, int *mul_sixteenths, int *sum_levels);
 int wxpy_reduce_tuned_set(int kind, int variant, int mul_sixteenths, int sum_levels);
 
@@ -830,12 +837,21 @@ int wxpy_debug_inject_launch_error(int cuda_error, int count);
  * flight.  -1 (the default) turns it off.  Process-wide. */
 int wxpy_debug_vecops_drop_tile(int64_t tile);
 
+/* The split a call of the class on n elements would run under (wxpy_vecops_pipes,
+ * else the searched split of its size range, else the default).  Host only. */
+int wxpy_debug_vecops_split(int op_class, int64_t n, int *add_offload, int *mul_sixteenths);
+
 /* Staged reductions launched after this call stop issuing copies before
  * chunk `chunk` (1024 elements; chunk c of tile t is 8t + c), so the owning
  * block's consumers' bounded waits run out and wxpy_reduce_status() reports
  * WXPY_ETIMEOUT; no copy is left in flight.  -1 (the default) turns it off.
  * Process-wide. */
 int wxpy_debug_reduce_drop_chunk(int64_t chunk);
+
+/* The configuration a reduction (kind 0 norm2, 1 dot) of n elements would run
+ * under, likewise.  Host only. */
+int wxpy_debug_reduce_config(int kind, int64_t n, int *variant, int *mul_sixteenths,
+                             int *sum_levels);
 
 #ifdef __cplusplus
 }

@@ -169,6 +169,9 @@ SIGNATURES = {
     "wxpy_vecops_tuned_get": (_INT, [_INT, ctypes.POINTER(_INT), ctypes.POINTER(_INT)]),
     "wxpy_vecops_tuned_set": (_INT, [_INT, _INT, _INT]),
     "wxpy_debug_vecops_drop_tile": (_INT, [_I64]),
+    "wxpy_debug_vecops_split": (_INT, [_INT, _I64, ctypes.POINTER(_INT), ctypes.POINTER(_INT)]),
+    "wxpy_debug_reduce_config": (_INT, [_INT, _I64, ctypes.POINTER(_INT), ctypes.POINTER(_INT),
+                                        ctypes.POINTER(_INT)]),
     "wxpy_host": (_INT, [_I64, _D, _P, _P, _P, _P]),
     "wxpy_host_config": (_INT, [_I64, _INT, _INT]),
     "wxpy_batch_launch_get": (_INT, [ctypes.POINTER(_INT), ctypes.POINTER(_INT)]),
@@ -541,6 +544,22 @@ def wxpy_vecops_tuned_set(op_class: int, add_offload: int, mul_sixteenths: int) 
 def wxpy_vecops_status() -> None:
     """Raises WxpyError(WXPY_ETIMEOUT) when a staged vector kernel's bounded wait ran out."""
     check(lib().wxpy_vecops_status(), "wxpy_vecops_status")
+
+
+def wxpy_debug_vecops_split(op_class: int, n: int) -> tuple[int, int]:
+    """(add_offload, mul_sixteenths) that a call of the class on n elements would run under."""
+    a, m = _INT(), _INT()
+    check(lib().wxpy_debug_vecops_split(op_class, n, ctypes.byref(a), ctypes.byref(m)),
+          "wxpy_debug_vecops_split")
+    return a.value, m.value
+
+
+def wxpy_debug_reduce_config(kind: int, n: int) -> tuple[int, int, int]:
+    """(variant, mul_sixteenths, sum_levels) that a reduction of n elements would run under."""
+    v, m, l = _INT(), _INT(), _INT()
+    check(lib().wxpy_debug_reduce_config(kind, n, ctypes.byref(v), ctypes.byref(m),
+                                         ctypes.byref(l)), "wxpy_debug_reduce_config")
+    return v.value, m.value, l.value
 
 
 def wxpy_debug_vecops_drop_tile(tile: int) -> None:

@@ -143,8 +143,12 @@ int vecops_inputs(int cls);
 int vecops_run(int cls, int64_t n, const double *coef, const double *const *in, double *out,
                VecPipes p, cudaStream_t s);
 VecPipes vecops_default(int cls, int64_t n);
-bool vecops_tuned_load(int cls, VecPipes *p);
-void vecops_tuned_store(int cls, const VecPipes *p);  // nullptr clears
+// A search's winner is used for calls of the size range it was found in, 0 or 1:
+// the best split of a class is another one where the L2 serves the call and where
+// HBM does.  range -1 stores for both; a load of -1 is of the last one stored.
+int vecops_range(int64_t n);
+bool vecops_tuned_load(int cls, int range, VecPipes *p);
+void vecops_tuned_store(int cls, int range, const VecPipes *p);  // nullptr clears
 
 // reduce.cu: the fused reductions (kind 0 norm2, 1 dot) under an explicit
 // configuration, and the table of searched configurations.
@@ -158,8 +162,15 @@ bool reduce_config_valid(int kind, ReduceConfig c);
 int reduce_run(int kind, int64_t n, double alpha, const double *x, const double *y, double *w,
                const double *z, double *result, void *workspace, int64_t ws_bytes, ReduceConfig c,
                cudaStream_t s);
-bool reduce_tuned_load(int kind, ReduceConfig *c);
-void reduce_tuned_store(int kind, const ReduceConfig *c);  // nullptr clears
+// By size range as the sibling kernels' splits: 0 where a call takes the cluster
+// form unless told otherwise, 1 above.
+int reduce_range(int64_t n);
+bool reduce_tuned_load(int kind, int range, ReduceConfig *c);
+void reduce_tuned_store(int kind, int range, const ReduceConfig *c);  // nullptr clears
+
+// The searches keep a built-in choice that their best candidate does not beat by
+// more than the timing's noise.
+constexpr double kSearchNoise = 1.005;
 
 cudaError_t launch_reference(unsigned grid, unsigned tpb, const SingleArgs &a, cudaStream_t s);
 SingleEntry single_entry(int vw, int offload, int u_idx, int gs, int cache, int xy);

@@ -588,7 +588,9 @@ std::atomic<int> g_reduce_mul{-1};
 std::atomic<long long> g_reduce_drop{-1};
 std::atomic<int> g_reduce_variant{-1};
 std::atomic<int> g_reduce_sum_levels{-1};
-std::atomic<int> g_reduce_tuned[2] = {-1, -1};  // (variant << 10) | (suml << 5) | mul
+// by size range and kind: (variant << 10) | (suml << 5) | mul
+std::atomic<int> g_reduce_tuned[2][2] = {{-1, -1}, {-1, -1}};
+std::atomic<int> g_reduce_last[2];  // per kind, the range stored last
 constexpr int kDefaultSumLevels = 0;
 constexpr int kReduceVariants = 7;  // 0 register-loaded, 1..3 staged, 4..6 warp-tiled
 // Measured on GB300 at n = 2^26 with every product in the integer pipelines
@@ -619,9 +621,9 @@ bool overlaps(const void *a, int64_t abytes, const void *b, int64_t bbytes) {
 
 // The configuration of a call: each knob set explicitly (>= 0) wins, then the
 // searched configuration of the operation, then the built-in default.
-ReduceConfig config_for(int kind) {
+ReduceConfig config_for(int kind, int64_t n) {
     ReduceConfig c = reduce_default(kind);
-    reduce_tuned_load(kind, &c);
+    reduce_tuned_load(kind, reduce_range(n), &c);
     const int v = g_reduce_variant.load(), m = g_reduce_mul.load(), l = g_reduce_sum_levels.load();
     if (v >= 0) c.variant = v;
     if (m >= 0) c.mul = m;
@@ -689,7 +691,8 @@ int launch_reduce(int64_t n, double alpha, const double *x, const double *y, dou
     const bool same = (diff & 31u) == 0;  // one offset modulo 32 bytes for all
     a.shift = (int)(((uintptr_t)w >> 3) & 3u);
     const int variant = vec ? cfg.variant : 0;
-    if (variant == 0 && cfg.suml == 0 && a.ntiles <= (vec || same ? kSplitTiles : kSplitTilesMixed)) {
+    const bool levels = KIND == 0 && vec && cfg.suml > 0;  // integer tree levels apply
+    if (variant == 0 && !levels && a.ntiles <= (vec || same ? kSplitTiles : kSplitTilesMixed)) {
         e = launch_reduce_split(KIND, vec, a, s);
         if (e == cudaSuccess && a.ntiles == 1) return WXPY_OK;
     } else if (variant == 0) {
@@ -735,9 +738,11 @@ bool reduce_config_valid(int kind, ReduceConfig c) {
            c.suml >= 0 && c.suml <= 6 && (kind == 0 || c.suml == 0);
 }
 
-bool reduce_tuned_load(int kind, ReduceConfig *c) {
+int reduce_range(int64_t n) { return n <= kSplitTiles * kTile ? 0 : 1; }
+
+bool reduce_tuned_load(int kind, int range, ReduceConfig *c) {
     if (kind < 0 || kind > 1) return false;
-    const int v = g_reduce_tuned[kind].load();
+    const int v = g_reduce_tuned[range < 0 ? g_reduce_last[kind].load() : range][kind].load();
     if (v < 0) return false;
     c->variant = v >> 10;
     c->suml = (v >> 5) & 31;
@@ -745,9 +750,13 @@ bool reduce_tuned_load(int kind, ReduceConfig *c) {
     return true;
 }
 
-void reduce_tuned_store(int kind, const ReduceConfig *c) {
+void reduce_tuned_store(int kind, int range, const ReduceConfig *c) {
     if (kind < 0 || kind > 1) return;
-    g_reduce_tuned[kind].store(c ? (c->variant << 10) | (c->suml << 5) | c->mul : -1);
+    for (int r = 0; r < 2; ++r)
+        if (range < 0 || range == r) {
+            g_reduce_tuned[r][kind].store(c ? (c->variant << 10) | (c->suml << 5) | c->mul : -1);
+            g_reduce_last[kind].store(r);
+        }
 }
 
 int reduce_run(int kind, int64_t n, double alpha, const double *x, const double *y, double *w,
@@ -772,14 +781,14 @@ int64_t wxpy_reduce_workspace_bytes(int64_t n) {
 int wxpy_norm2(int64_t n, double alpha, const double *x, const double *y, double *w,
                double *result, void *workspace, int64_t workspace_bytes, void *stream) {
     return launch_reduce<0>(n, alpha, x, y, w, nullptr, result, workspace, workspace_bytes,
-                            config_for(0), (cudaStream_t)stream);
+                            config_for(0, n), (cudaStream_t)stream);
 }
 
 int wxpy_dot(int64_t n, double alpha, const double *x, const double *y, double *w,
              const double *z, double *result, void *workspace, int64_t workspace_bytes,
              void *stream) {
     return launch_reduce<1>(n, alpha, x, y, w, z, result, workspace, workspace_bytes,
-                            config_for(1), (cudaStream_t)stream);
+                            config_for(1, n), (cudaStream_t)stream);
 }
 
 int wxpy_reduce_status(void) {
@@ -794,6 +803,17 @@ int wxpy_reduce_status(void) {
     if (fault)
         return fail(WXPY_ETIMEOUT, "a staged reduction's bounded wait ran out (mask %u: 1 producer, "
                     "2 consumer, 4 exchange)", fault);
+    return WXPY_OK;
+}
+
+int wxpy_debug_reduce_config(int kind, int64_t n, int *variant, int *mul_sixteenths,
+                             int *sum_levels) {
+    if (kind < 0 || kind > 1 || n < 0 || !variant || !mul_sixteenths || !sum_levels)
+        return fail(WXPY_EINVAL, "bad reduction kind %d or size", kind);
+    const ReduceConfig c = config_for(kind, n);
+    *variant = c.variant;
+    *mul_sixteenths = c.mul;
+    *sum_levels = c.suml;
     return WXPY_OK;
 }
 

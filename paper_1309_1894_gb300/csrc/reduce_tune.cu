@@ -172,9 +172,17 @@ int tune_kind(int kind, int64_t n, RScratch &sc, wxpy_reduce_tune_result *res) {
     if (kind == 0)
         for (int l = 2; l <= 6; l += 2)
             if ((st = consider(ReduceConfig{wbest, bmul, l})) != WXPY_OK) return st;
+    // The default, verified among the candidates, stays unless they beat it.
+    const ReduceConfig def = reduce_default(kind);
     double def_us = 0.0;
-    if ((st = time_config(kind, n, reduce_default(kind), sc, &def_us)) != WXPY_OK) return st;
-    reduce_tuned_store(kind, &best);
+    unsigned long long bad = 0;
+    if ((st = run_checked(kind, n, def, sc, &bad)) != WXPY_OK) return st;
+    if ((st = time_config(kind, n, def, sc, &def_us)) != WXPY_OK) return st;
+    if (!bad && def_us < best_us * kSearchNoise) {
+        best = def;
+        best_us = def_us;
+    }
+    reduce_tuned_store(kind, reduce_range(n), &best);
     if (res) {
         res->kind = kind;
         res->variant = best.variant;
@@ -237,7 +245,7 @@ int wxpy_reduce_tuned_get(int kind, int *variant, int *mul_sixteenths, int *sum_
     if (kind < 0 || kind > 1 || !variant || !mul_sixteenths || !sum_levels)
         return fail(WXPY_EINVAL, "bad reduction kind %d", kind);
     ReduceConfig c{-1, -1, -1};
-    reduce_tuned_load(kind, &c);
+    reduce_tuned_load(kind, -1, &c);
     *variant = c.variant;
     *mul_sixteenths = c.mul;
     *sum_levels = c.suml;
@@ -247,14 +255,14 @@ int wxpy_reduce_tuned_get(int kind, int *variant, int *mul_sixteenths, int *sum_
 int wxpy_reduce_tuned_set(int kind, int variant, int mul_sixteenths, int sum_levels) {
     if (kind < 0 || kind > 1) return fail(WXPY_EINVAL, "bad reduction kind %d", kind);
     if (variant == -1 && mul_sixteenths == -1 && sum_levels == -1) {
-        reduce_tuned_store(kind, nullptr);
+        reduce_tuned_store(kind, -1, nullptr);
         return WXPY_OK;
     }
     const ReduceConfig c{variant, mul_sixteenths, sum_levels};
     if (!reduce_config_valid(kind, c))
         return fail(WXPY_EINVAL, "bad reduction configuration (%d, %d, %d)", variant,
                     mul_sixteenths, sum_levels);
-    reduce_tuned_store(kind, &c);
+    reduce_tuned_store(kind, -1, &c);
     return WXPY_OK;
 }
 

@@ -324,10 +324,9 @@ int tune_impl(int64_t n, unsigned flags, wxpy_tune_result *out) {
     // the timing's noise the default, whose shape was chosen over all offsets of the
     // class where the search sees one set of them (mixed offsets at 2^28: a shape
     // 0.3 % faster than the default on one set is 8 % slower on two others).
-    constexpr double kNoise = 1.005;
     Variant chosen = best.v;
     double chosen_us = best_us;
-    if (def_us < best_us * kNoise) {
+    if (def_us < best_us * kSearchNoise) {
         chosen = dv;
         chosen_us = def_us;
     }
@@ -437,14 +436,19 @@ int cache_save(const char *path) {
         out += "\n  \"vecops\": [";
         bool vfirst = true;
         for (int c = 0; c < WXPY_VEC_CLASSES; ++c) {
-            VecPipes vp;
-            if (!vecops_tuned_load(c, &vp)) continue;
-            char buf[120];
-            std::snprintf(buf, sizeof buf,
-                          "%s\n    {\"class\": %d, \"add_offload\": %d, \"mul_sixteenths\": %d}",
-                          vfirst ? "" : ",", c, vp.add, vp.mul);
-            out += buf;
-            vfirst = false;
+            VecPipes v[2];
+            const bool have[2] = {vecops_tuned_load(c, 0, &v[0]), vecops_tuned_load(c, 1, &v[1])};
+            const bool both = have[0] && have[1] && v[0].add == v[1].add && v[0].mul == v[1].mul;
+            for (int range = 0; range < 2; ++range) {
+                if (!have[range] || (both && range)) continue;
+                char buf[140], sizes[24] = "";
+                if (!both) std::snprintf(sizes, sizeof sizes, ", \"sizes\": %d", range + 1);
+                std::snprintf(buf, sizeof buf,
+                              "%s\n    {\"class\": %d, \"add_offload\": %d, \"mul_sixteenths\": %d%s}",
+                              vfirst ? "" : ",", c, v[range].add, v[range].mul, sizes);
+                out += buf;
+                vfirst = false;
+            }
         }
         out += "\n  ],";
     }
@@ -452,15 +456,21 @@ int cache_save(const char *path) {
         out += "\n  \"reduce\": [";
         bool rfirst = true;
         for (int k = 0; k < 2; ++k) {
-            ReduceConfig rc;
-            if (!reduce_tuned_load(k, &rc)) continue;
-            char buf[140];
-            std::snprintf(buf, sizeof buf,
-                          "%s\n    {\"kind\": %d, \"variant\": %d, \"mul_sixteenths\": %d, "
-                          "\"sum_levels\": %d}",
-                          rfirst ? "" : ",", k, rc.variant, rc.mul, rc.suml);
-            out += buf;
-            rfirst = false;
+            ReduceConfig v[2];
+            const bool have[2] = {reduce_tuned_load(k, 0, &v[0]), reduce_tuned_load(k, 1, &v[1])};
+            const bool both = have[0] && have[1] && v[0].variant == v[1].variant &&
+                              v[0].mul == v[1].mul && v[0].suml == v[1].suml;
+            for (int range = 0; range < 2; ++range) {
+                if (!have[range] || (both && range)) continue;
+                char buf[160], sizes[24] = "";
+                if (!both) std::snprintf(sizes, sizeof sizes, ", \"sizes\": %d", range + 1);
+                std::snprintf(buf, sizeof buf,
+                              "%s\n    {\"kind\": %d, \"variant\": %d, \"mul_sixteenths\": %d, "
+                              "\"sum_levels\": %d%s}",
+                              rfirst ? "" : ",", k, v[range].variant, v[range].mul, v[range].suml, sizes);
+                out += buf;
+                rfirst = false;
+            }
         }
         out += "\n  ],";
     }
@@ -567,8 +577,13 @@ int cache_load(const char *path, const char *expect_device) {
             }
         }
     }
-    // Optional searched splits of the sibling kernels.
-    std::vector<std::pair<int, VecPipes>> vec;
+    // Optional searched splits of the sibling kernels; "sizes": 1 or 2, the range of
+    // call sizes of an entry, every size without it.
+    struct VecEntry {
+        int cls, range;
+        VecPipes p;
+    };
+    std::vector<VecEntry> vec;
     size_t vpos = s.find("\"vecops\"");
     if (vpos != std::string::npos) {
         const size_t vend = s.find(']', vpos);
@@ -581,12 +596,19 @@ int cache_load(const char *path, const char *expect_device) {
                 !find_int(s, q, r, "add_offload", &a) || !find_int(s, q, r, "mul_sixteenths", &m) ||
                 c < 0 || c >= WXPY_VEC_CLASSES || a < 0 || a > 2 || m < 0 || m > 16)
                 return fail(WXPY_EINVAL, "%s: malformed vecops entry", path);
-            vec.push_back({(int)c, VecPipes{(int)a, (int)m}});
+            long long sizes = 0;
+            if (find_int(s, q, r, "sizes", &sizes) && (sizes < 1 || sizes > 2))
+                return fail(WXPY_EINVAL, "%s: malformed vecops entry", path);
+            vec.push_back({(int)c, (int)sizes - 1, VecPipes{(int)a, (int)m}});
             q = r;
         }
     }
     // Optional searched configurations of the fused reductions.
-    std::vector<std::pair<int, ReduceConfig>> red;
+    struct ReduceEntry {
+        int kind, range;
+        ReduceConfig c;
+    };
+    std::vector<ReduceEntry> red;
     size_t rpos = s.find("\"reduce\"");
     if (rpos != std::string::npos) {
         const size_t rend = s.find(']', rpos);
@@ -600,7 +622,10 @@ int cache_load(const char *path, const char *expect_device) {
                 !find_int(s, q, r, "sum_levels", &l) || k < 0 || k > 1 ||
                 !reduce_config_valid((int)k, ReduceConfig{(int)v, (int)m, (int)l}))
                 return fail(WXPY_EINVAL, "%s: malformed reduce entry", path);
-            red.push_back({(int)k, ReduceConfig{(int)v, (int)m, (int)l}});
+            long long sizes = 0;
+            if (find_int(s, q, r, "sizes", &sizes) && (sizes < 1 || sizes > 2))
+                return fail(WXPY_EINVAL, "%s: malformed reduce entry", path);
+            red.push_back({(int)k, (int)sizes - 1, ReduceConfig{(int)v, (int)m, (int)l}});
             q = r;
         }
     }
@@ -609,8 +634,8 @@ int cache_load(const char *path, const char *expect_device) {
         g_tuned_launch_bound[entries[i].first].store(entry_lb[i]);
     }
     if (have_batch) set_batch_shape(bs);
-    for (auto &cv : vec) vecops_tuned_store(cv.first, &cv.second);
-    for (auto &rc : red) reduce_tuned_store(rc.first, &rc.second);
+    for (auto &v : vec) vecops_tuned_store(v.cls, v.range, &v.p);
+    for (auto &v : red) reduce_tuned_store(v.kind, v.range, &v.c);
     return WXPY_OK;
 }
 
@@ -675,8 +700,8 @@ int wxpy_tune_set(int tune_key, int variant_id) {
 int wxpy_tune_clear(void) {
     for (auto &t : g_tuned) t.store(-1);
     for (auto &t : g_tuned_launch_bound) t.store(0);
-    for (int c = 0; c < WXPY_VEC_CLASSES; ++c) vecops_tuned_store(c, nullptr);
-    for (int k = 0; k < 2; ++k) reduce_tuned_store(k, nullptr);
+    for (int c = 0; c < WXPY_VEC_CLASSES; ++c) vecops_tuned_store(c, -1, nullptr);
+    for (int k = 0; k < 2; ++k) reduce_tuned_store(k, -1, nullptr);
     return WXPY_OK;
 }
 

@@ -721,13 +721,17 @@ int launch_ew(const double *const *in, double *out, int64_t n, const double *coe
 // either leaves the operation's searched split, else its default (below).
 std::atomic<int> g_vec_add{-1};
 std::atomic<int> g_vec_mul{-1};
-std::atomic<int> g_vec_tuned[WXPY_VEC_CLASSES] = {-1, -1, -1, -1, -1, -1, -1, -1, -1, -1};
+std::atomic<int> g_vec_tuned[2][WXPY_VEC_CLASSES] = {{-1, -1, -1, -1, -1, -1, -1, -1, -1, -1},
+                                                     {-1, -1, -1, -1, -1, -1, -1, -1, -1, -1}};
+std::atomic<int> g_vec_last[WXPY_VEC_CLASSES];  // the range stored last
+
+constexpr int64_t kLongCall = (int64_t)1 << 23;  // elements: HBM's side of vecops_default
 
 using Pipes = VecPipes;
 
 Pipes pipes_for(int cls, int64_t n) {
     Pipes p = vecops_default(cls, n);
-    vecops_tuned_load(cls, &p);
+    vecops_tuned_load(cls, vecops_range(n), &p);
     const int add = g_vec_add.load(), mul = g_vec_mul.load();
     if (add >= 0) p.add = add;
     if (mul >= 0) p.mul = mul;
@@ -754,7 +758,7 @@ int maxpy_group(int64_t n, const double *alpha, const double *const *in, Pipes p
 // 19.1 / 84.5 / 332, 14/16 7.3 / 21.6 / 82.1 / 313.
 VecPipes vecops_default(int cls, int64_t n) {
     if (cls == WXPY_VEC_PMULT) return {0, 4};
-    const bool short_call = n < ((int64_t)1 << 23);
+    const bool short_call = vecops_range(n) == 0;
     if (cls == WXPY_VEC_AXPBYPCZ) return {0, short_call ? 16 : 15};
     if (cls == WXPY_VEC_AXPBY) return {0, short_call ? 16 : 10};
     return {0, cls + 1 == 2 && !short_call ? 14 : 16};  // maxpy with cls + 1 terms
@@ -766,18 +770,24 @@ int vecops_inputs(int cls) {
     return cls + 2;  // y and cls + 1 x vectors
 }
 
-bool vecops_tuned_load(int cls, VecPipes *p) {
+int vecops_range(int64_t n) { return n < kLongCall ? 0 : 1; }
+
+bool vecops_tuned_load(int cls, int range, VecPipes *p) {
     if (cls < 0 || cls >= WXPY_VEC_CLASSES) return false;
-    const int v = g_vec_tuned[cls].load();
+    const int v = g_vec_tuned[range < 0 ? g_vec_last[cls].load() : range][cls].load();
     if (v < 0) return false;
     p->add = v >> 5;
     p->mul = v & 31;
     return true;
 }
 
-void vecops_tuned_store(int cls, const VecPipes *p) {
+void vecops_tuned_store(int cls, int range, const VecPipes *p) {
     if (cls < 0 || cls >= WXPY_VEC_CLASSES) return;
-    g_vec_tuned[cls].store(p ? (p->add << 5) | p->mul : -1);
+    for (int r = 0; r < 2; ++r)
+        if (range < 0 || range == r) {
+            g_vec_tuned[r][cls].store(p ? (p->add << 5) | p->mul : -1);
+            g_vec_last[cls].store(r);
+        }
 }
 
 int vecops_run(int cls, int64_t n, const double *coef, const double *const *in, double *out,
@@ -891,6 +901,15 @@ int wxpy_vecops_status(void) {
     if (fault)
         return fail(WXPY_ETIMEOUT, "a staged vector kernel's bounded wait ran out (%s)",
                     fault & 1u ? (fault & 2u ? "producer and consumers" : "producer") : "consumers");
+    return WXPY_OK;
+}
+
+int wxpy_debug_vecops_split(int op_class, int64_t n, int *add_offload, int *mul_sixteenths) {
+    if (op_class < 0 || op_class >= WXPY_VEC_CLASSES || n < 0 || !add_offload || !mul_sixteenths)
+        return fail(WXPY_EINVAL, "bad vector class %d or size", op_class);
+    const Pipes p = pipes_for(op_class, n);
+    *add_offload = p.add;
+    *mul_sixteenths = p.mul;
     return WXPY_OK;
 }
 

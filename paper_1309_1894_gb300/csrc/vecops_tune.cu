@@ -9,7 +9,8 @@
 // of the all-FP64 split on the same inputs; a split whose output differs by a
 // single bit is rejected.  Candidates per class: the product share 0, 2, ..,
 // 16 sixteenths with the sums in FP64, then the sums every other one or all
-// in the integer pipeline at the best product share.  Timing: median of five
+// in the integer pipeline at the best product share; the default split stays
+// where none of them beats it.  Timing: median of five
 // runs of three back-to-back calls, each run after an L2 flush and a short
 // device delay, with the in-place output restored from a pristine copy before
 // every run.
@@ -192,9 +193,17 @@ int tune_class(int cls, int64_t n, VScratch &sc, wxpy_vecops_tune_result *res) {
             if ((st = consider(VecPipes{add, mul})) != WXPY_OK) return st;
     }
     if (!have) return fail(WXPY_EMISMATCH, "every split of vector class %d differed", cls);
+    // The default, whose share need not be among the candidates; kept unless they
+    // beat it.
+    const VecPipes def = vecops_default(cls, n);
     double def_us = 0.0;
-    if ((st = time_split(c, n, vecops_default(cls, n), sc, &def_us)) != WXPY_OK) return st;
-    vecops_tuned_store(cls, &best);
+    if ((st = run_checked(c, n, def, sc, false, &bad)) != WXPY_OK) return st;
+    if ((st = time_split(c, n, def, sc, &def_us)) != WXPY_OK) return st;
+    if (!bad && def_us < best_us * kSearchNoise) {
+        best = def;
+        best_us = def_us;
+    }
+    vecops_tuned_store(cls, vecops_range(n), &best);
     if (res) {
         res->op_class = cls;
         res->add_offload = best.add;
@@ -263,7 +272,7 @@ int wxpy_vecops_tuned_get(int op_class, int *add_offload, int *mul_sixteenths) {
     if (op_class < 0 || op_class >= WXPY_VEC_CLASSES || !add_offload || !mul_sixteenths)
         return fail(WXPY_EINVAL, "bad vector class %d", op_class);
     VecPipes p{-1, -1};
-    vecops_tuned_load(op_class, &p);
+    vecops_tuned_load(op_class, -1, &p);
     *add_offload = p.add;
     *mul_sixteenths = p.mul;
     return WXPY_OK;
@@ -273,14 +282,14 @@ int wxpy_vecops_tuned_set(int op_class, int add_offload, int mul_sixteenths) {
     if (op_class < 0 || op_class >= WXPY_VEC_CLASSES)
         return fail(WXPY_EINVAL, "bad vector class %d", op_class);
     if (add_offload == -1 && mul_sixteenths == -1) {
-        vecops_tuned_store(op_class, nullptr);
+        vecops_tuned_store(op_class, -1, nullptr);
         return WXPY_OK;
     }
     if (add_offload < 0 || add_offload > 2 || mul_sixteenths < 0 || mul_sixteenths > 16 ||
         (op_class == WXPY_VEC_PMULT && add_offload != 0))
         return fail(WXPY_EINVAL, "bad split (%d, %d)", add_offload, mul_sixteenths);
     const VecPipes p{add_offload, mul_sixteenths};
-    vecops_tuned_store(op_class, &p);
+    vecops_tuned_store(op_class, -1, &p);
     return WXPY_OK;
 }
 
