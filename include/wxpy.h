@@ -637,7 +637,11 @@ int wxpy_batch_tune(int bucket_min, int bucket_max, unsigned flags,
 
 /* The batch shape table: per bucket tile length (0 or a multiple of 32, at
  * most 2^30) and unroll (1, 2, 4: 32-byte vectors of x and of y in flight per
- * lane per pass).  Host only; no device touched. */
+ * lane per pass).  A batch runs with four in flight if a bucket that it has a
+ * problem in was set to 4 (by a call, the search or a cache file).  Buckets never
+ * set are reported as 4 and run with four where the tiles of a plan (or of a
+ * server's batch) hold 2048 elements and more on average, else with two.
+ * wxpy_batch_noalloc reads no table of the host's and always has two.  Host only; no device touched. */
 int wxpy_batch_shape_get(int bucket, int *tile_elems, int *unroll);
 int wxpy_batch_shape_set(int bucket, int tile_elems, int unroll);
 int wxpy_batch_shape_reset(void);
@@ -830,6 +834,10 @@ int wxpy_fill_uniform(int64_t n, uint64_t seed, uint32_t tag, int64_t start,
  * cudaError_t `cuda_error` (returned as WXPY_ECUDA) without touching the GPU.
  * count = 0 clears it.  Process-wide. */
 int wxpy_debug_inject_launch_error(int cuda_error, int count);
+
+/* The 32-byte vectors of x and of y in flight per lane, 4 or 2, that a plan of the
+ * table would run with (wxpy_batch_shape_set).  The table is validated as by wxpy_batch_plan_create.  Host only. */
+int wxpy_debug_batch_vectors(const wxpy_desc *host_table, int64_t count, int *vectors);
 
 /* Staged vector kernels launched after this call stop issuing copies at tile
  * `tile` (in the block that owns it), so that block's consumers' bounded wait

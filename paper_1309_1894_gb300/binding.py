@@ -168,6 +168,7 @@ SIGNATURES = {
     "wxpy_vecops_tune": (_INT, [_I64, ctypes.POINTER(VecopsTuneResult)]),
     "wxpy_vecops_tuned_get": (_INT, [_INT, ctypes.POINTER(_INT), ctypes.POINTER(_INT)]),
     "wxpy_vecops_tuned_set": (_INT, [_INT, _INT, _INT]),
+    "wxpy_debug_batch_vectors": (_INT, [ctypes.c_void_p, _I64, ctypes.POINTER(_INT)]),
     "wxpy_debug_vecops_drop_tile": (_INT, [_I64]),
     "wxpy_debug_vecops_split": (_INT, [_INT, _I64, ctypes.POINTER(_INT), ctypes.POINTER(_INT)]),
     "wxpy_debug_reduce_config": (_INT, [_INT, _I64, ctypes.POINTER(_INT), ctypes.POINTER(_INT),
@@ -544,6 +545,14 @@ def wxpy_vecops_tuned_set(op_class: int, add_offload: int, mul_sixteenths: int) 
 def wxpy_vecops_status() -> None:
     """Raises WxpyError(WXPY_ETIMEOUT) when a staged vector kernel's bounded wait ran out."""
     check(lib().wxpy_vecops_status(), "wxpy_vecops_status")
+
+
+def wxpy_debug_batch_vectors(table) -> int:
+    """Vectors of x and of y in flight per lane (4 or 2) that a plan of the table would run with."""
+    v = _INT()
+    check(lib().wxpy_debug_batch_vectors(table.ctypes.data, len(table), ctypes.byref(v)),
+          "wxpy_debug_batch_vectors")
+    return v.value
 
 
 def wxpy_debug_vecops_split(op_class: int, n: int) -> tuple[int, int]:

@@ -67,27 +67,33 @@ __global__ void __launch_bounds__(256, MAXU == kTileU ? 3 : 2) wxpy_seg_kernel(c
 
 using SegKernelFn = void (*)(SegParams);
 
-// Long tiles: 2048 elements and more on average.
-static SegKernelFn seg_kernel_fn(int offload, int64_t ntiles, int64_t elems) {
-    const bool wide = elems >= 2048 * ntiles;
+static SegKernelFn seg_kernel_fn(int offload, bool wide) {
     return offload == 3 ? (wide ? &wxpy_seg_kernel<3, kTileWideU> : &wxpy_seg_kernel<3, kTileU>)
            : offload    ? (wide ? &wxpy_seg_kernel<1, kTileWideU> : &wxpy_seg_kernel<1, kTileU>)
                         : (wide ? &wxpy_seg_kernel<0, kTileWideU> : &wxpy_seg_kernel<0, kTileU>);
 }
 
-static cudaError_t seg_launch(int offload, unsigned grid, int threads, int64_t elems,
+static cudaError_t seg_launch(int offload, unsigned grid, int threads, bool wide,
                               const SegParams &sp, cudaStream_t s) {
-    return launch_pdl(seg_kernel_fn(offload, sp.ntiles, elems), grid, (unsigned)threads, s, sp);
+    return launch_pdl(seg_kernel_fn(offload, wide), grid, (unsigned)threads, s, sp);
 }
 
 // The same tiles without a list: the warp finds its tile's segment in the
 // per-segment plan (seg_search.cuh).  For one-shot calls, whose list would be
 // built and copied for a single launch.
-template <int EMU>
-__global__ void __launch_bounds__(256, 3)
+template <int EMU, int MAXU>
+__global__ void __launch_bounds__(256, MAXU == kTileU ? 3 : 2)
     wxpy_seg_search_kernel(const wxpy_desc *table, const SegPlan *plan, int64_t count) {
     pdl_enter();
-    run_plan_tiles<EMU>(table, plan, count);
+    run_plan_tiles<EMU, MAXU>(table, plan, count);
+}
+
+using SearchKernelFn = void (*)(const wxpy_desc *, const SegPlan *, int64_t);
+
+static SearchKernelFn search_kernel_fn(int offload, bool wide) {
+    return offload == 3 ? (wide ? &wxpy_seg_search_kernel<3, kTileWideU> : &wxpy_seg_search_kernel<3, kTileU>)
+           : offload    ? (wide ? &wxpy_seg_search_kernel<1, kTileWideU> : &wxpy_seg_search_kernel<1, kTileU>)
+                        : (wide ? &wxpy_seg_search_kernel<0, kTileWideU> : &wxpy_seg_search_kernel<0, kTileU>);
 }
 
 // ---------------------------------------------------------------- shapes
@@ -108,7 +114,7 @@ BatchShape default_batch_shape() {
                     // 1103 with half the sums (at its best grid)
     for (int b = 0; b < kBuckets; ++b) {
         s.tile_elems[b] = b < 13 ? 0 : 8192;
-        s.unroll_log2[b] = 2;
+        s.unroll_log2[b] = -1;
     }
     return s;
 }
@@ -190,8 +196,27 @@ static int64_t tile_len_of(const BatchShape &shape, int64_t n, int64_t t_cap) {
     return std::min<int64_t>(std::min<int64_t>(T, t_cap), kMaxTileElems);
 }
 
-static int unroll_log2_of(const BatchShape &shape, int64_t n) {
-    return std::min<int>(2, std::max<int>(0, shape.unroll_log2[bucket_of(n)]));
+int unroll_log2_of(const BatchShape &shape, int64_t n) {
+    const int ul = shape.unroll_log2[bucket_of(n)];
+    return ul < 0 ? 2 : std::min<int>(2, ul);
+}
+
+// Four vectors in flight where a segment's bucket asks for them, set or found by
+// the search.  Buckets left at the built-in unroll take what is faster for the
+// batch (see wxpy_seg_kernel): four from 2048 elements per tile on average, else
+// two.  A one-shot call passes no elements: where a warp searches for its tiles, two
+// are as fast or faster throughout (4096 segments up to 2^18 / 2^20: 353 / 1155 us
+// against 362 / 1150).
+bool wide_body(const wxpy_desc *t, int64_t count, const BatchShape &shape, int64_t ntiles,
+               int64_t elems) {
+    bool built_in = false;
+    for (int64_t s = 0; s < count; ++s) {
+        if (t[s].n <= 0) continue;
+        const int ul = shape.unroll_log2[bucket_of(t[s].n)];
+        if (ul >= 2) return true;
+        built_in = built_in || ul < 0;
+    }
+    return built_in && elems >= 2048 * ntiles;
 }
 
 // Blocks of a launch over `ntiles` tiles of `elems` elements in all.  Where the
@@ -259,8 +284,8 @@ int64_t build_tiles(const wxpy_desc *t, int64_t count, const BatchShape &shape, 
 }
 
 cudaError_t launch_segmented(const wxpy_desc *dev_table, const TileRec *tiles, int64_t ntiles,
-                             int64_t elems, unsigned *status, const BatchShape &shape, int sm_count,
-                             cudaStream_t s) {
+                             int64_t elems, bool wide, unsigned *status, const BatchShape &shape,
+                             int sm_count, cudaStream_t s) {
     if (ntiles == 0) return cudaSuccess;
     const unsigned grid = batch_grid(shape, sm_count, ntiles, elems);
     cudaError_t e = injected_launch_error();
@@ -270,7 +295,7 @@ cudaError_t launch_segmented(const wxpy_desc *dev_table, const TileRec *tiles, i
     sp.tiles = tiles;
     sp.ntiles = ntiles;
     sp.status = status;
-    return seg_launch(shape.offload, grid, shape.threads, elems, sp, s);
+    return seg_launch(shape.offload, grid, shape.threads, wide, sp, s);
 }
 
 }  // namespace wx
@@ -286,6 +311,7 @@ struct wxpy_batch_plan {
     TileRec *d_tiles = nullptr;
     unsigned *d_status = nullptr;
     unsigned grid = 0;
+    bool wide = false;
     // graph of the launch, with the table it was built for
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
@@ -332,6 +358,7 @@ int wxpy_batch_plan_create(const wxpy_desc *host_table, int64_t count, wxpy_batc
     p->total_elems = build_tiles(host_table, count, p->shape, true, &tiles);
     p->ntiles = (int64_t)tiles.size();
     p->grid = batch_grid(p->shape, dp->sm_count, p->ntiles, p->total_elems);
+    p->wide = wide_body(host_table, count, p->shape, p->ntiles, p->total_elems);
     cudaError_t e = cudaMalloc(&p->d_status, 256);
     if (e == cudaSuccess && p->ntiles > 0)
         e = cudaMalloc(&p->d_tiles, sizeof(TileRec) * (size_t)p->ntiles);
@@ -359,7 +386,7 @@ int wxpy_batch_launch(wxpy_batch_plan *plan, const wxpy_desc *dev_table, void *s
     if (!dev_table) return fail(WXPY_EINVAL, "null device table");
     cudaError_t e = injected_launch_error();
     if (e == cudaSuccess)
-        e = seg_launch(plan->shape.offload, plan->grid, plan->shape.threads, plan->total_elems,
+        e = seg_launch(plan->shape.offload, plan->grid, plan->shape.threads, plan->wide,
                        params_of(plan, dev_table), (cudaStream_t)stream);
     if (e != cudaSuccess) return fail_cuda(e, "batch kernel launch");
     return WXPY_OK;
@@ -374,7 +401,7 @@ int wxpy_batch_graph_launch(wxpy_batch_plan *plan, const wxpy_desc *dev_table, v
     SegParams sp = params_of(plan, dev_table);
     void *args[] = {&sp};
     cudaKernelNodeParams kp = {};
-    kp.func = (void *)seg_kernel_fn(plan->shape.offload, plan->ntiles, plan->total_elems);
+    kp.func = (void *)seg_kernel_fn(plan->shape.offload, plan->wide);
     kp.gridDim = dim3(plan->grid);
     kp.blockDim = dim3(plan->shape.threads);
     kp.sharedMemBytes = 0;
@@ -458,9 +485,8 @@ int wxpy_batch(const wxpy_desc *host_table, const wxpy_desc *dev_table, int64_t 
         const unsigned grid = batch_grid(shape, dp->sm_count, ntiles, total);
         const unsigned threads = (unsigned)shape.threads;
         const SegPlan *d_plan = (const SegPlan *)buf;
-        e = shape.offload == 3 ? launch_pdl(&wxpy_seg_search_kernel<3>, grid, threads, s, dev_table, d_plan, count)
-            : shape.offload    ? launch_pdl(&wxpy_seg_search_kernel<1>, grid, threads, s, dev_table, d_plan, count)
-                               : launch_pdl(&wxpy_seg_search_kernel<0>, grid, threads, s, dev_table, d_plan, count);
+        const bool wide = wide_body(host_table, count, shape, ntiles, 0);
+        e = launch_pdl(search_kernel_fn(shape.offload, wide), grid, threads, s, dev_table, d_plan, count);
     }
     cudaError_t e2 = cudaFreeAsync(buf, s);
     if (e != cudaSuccess) return fail_cuda(e, "batch launch");
@@ -601,10 +627,11 @@ int run_shape(SynthBatch &sb, const BatchShape &shape, const DeviceProps &dp, in
     sp.tiles = (const TileRec *)sb.tiles.p;
     sp.ntiles = ntiles;
     sp.status = (unsigned *)sb.status.p;
+    const bool wide = wide_body(sb.host.data(), (int64_t)sb.host.size(), shape, ntiles, sb.elems);
     // verification run on a poisoned output
     cudaError_t e = cudaMemsetAsync(sb.w.p, 0xff, (size_t)sb.slots * 8, s);
     if (e == cudaSuccess) e = cudaMemsetAsync(sb.count.p, 0, 8, s);
-    if (e == cudaSuccess) e = seg_launch(shape.offload, grid, shape.threads, sb.elems, sp, s);
+    if (e == cudaSuccess) e = seg_launch(shape.offload, grid, shape.threads, wide, sp, s);
     if (e != cudaSuccess) return fail_cuda(e, "batch search launch");
     if ((st = launch_count_mismatch((const double *)sb.w.p, (const double *)sb.wref.p, sb.slots,
                                     (unsigned long long *)sb.count.p, s)))
@@ -615,7 +642,7 @@ int run_shape(SynthBatch &sb, const BatchShape &shape, const DeviceProps &dp, in
     std::vector<float> ms(reps);
     for (int r = 0; r < reps; ++r) {
         cudaEventRecord(e0, s);
-        seg_launch(shape.offload, grid, shape.threads, sb.elems, sp, s);
+        seg_launch(shape.offload, grid, shape.threads, wide, sp, s);
         cudaEventRecord(e1, s);
         if ((e = cudaEventSynchronize(e1)) != cudaSuccess) return fail_cuda(e, "batch search timing");
         cudaEventElapsedTime(&ms[r], e0, e1);
@@ -626,6 +653,9 @@ int run_shape(SynthBatch &sb, const BatchShape &shape, const DeviceProps &dp, in
 }
 
 }  // namespace
+
+// As the shape table reports it: 4 for the built-in one.
+static int unroll_of(int log2) { return log2 < 0 ? 4 : 1 << log2; }
 
 int batch_tune_impl(int bmin, int bmax, unsigned flags, wxpy_batch_tune_result *out) {
     TraceRange trace("wxpy_batch_tune");
@@ -669,7 +699,8 @@ int batch_tune_impl(int bmin, int bmax, unsigned flags, wxpy_batch_tune_result *
         int8_t best_u = shape.unroll_log2[b];
         for (int32_t T : kTiles) {
             if (T != 0 && T >= ((int64_t)2 << b)) continue;  // no cut: same as whole segment
-            for (int8_t ul = 0; ul < 3; ++ul) {
+            for (int8_t ul = -1; ul < 3; ++ul) {
+                if (ul < 0 && T != builtin.tile_elems[b]) continue;  // the built-in shape
                 if (quick && (ul == 0 || (T != 0 && T != 8192))) continue;
                 BatchShape cand = shape;
                 cand.tile_elems[b] = T;
@@ -682,7 +713,7 @@ int batch_tune_impl(int bmin, int bmax, unsigned flags, wxpy_batch_tune_result *
                     ++rejected;
                     continue;
                 }
-                if (T == builtin.tile_elems[b] && ul == builtin.unroll_log2[b]) plain_us[b] = us;
+                if (ul < 0) plain_us[b] = us;
                 if (us < best_us) {
                     best_us = us;
                     best_tile = T;
@@ -695,7 +726,7 @@ int batch_tune_impl(int bmin, int bmax, unsigned flags, wxpy_batch_tune_result *
         shape.unroll_log2[b] = best_u;
         if (out) {
             out->tile_elems[b] = best_tile;
-            out->unroll[b] = 1 << best_u;
+            out->unroll[b] = unroll_of(best_u);
             out->us[b] = best_us;
             out->gbs[b] = 24.0 * (double)sb.elems / (best_us * 1e-6) / 1e9;
         }
@@ -736,7 +767,7 @@ int batch_tune_impl(int bmin, int bmax, unsigned flags, wxpy_batch_tune_result *
         if (out) {
             for (int b = bmin; b <= bmax && best_plain; ++b) {
                 out->tile_elems[b] = shape.tile_elems[b];
-                out->unroll[b] = 1 << shape.unroll_log2[b];
+                out->unroll[b] = unroll_of(shape.unroll_log2[b]);
                 out->gbs[b] *= out->us[b] / plain_us[b];
                 out->us[b] = plain_us[b];
             }
@@ -767,7 +798,7 @@ extern "C" int wxpy_batch_shape_get(int bucket, int *tile_elems, int *unroll) {
         return wx::fail(WXPY_EINVAL, "bad bucket %d", bucket);
     const wx::BatchShape s = wx::current_batch_shape();
     *tile_elems = s.tile_elems[bucket];
-    *unroll = 1 << s.unroll_log2[bucket];
+    *unroll = wx::unroll_of(s.unroll_log2[bucket]);
     return WXPY_OK;
 }
 
@@ -781,6 +812,17 @@ extern "C" int wxpy_batch_shape_set(int bucket, int tile_elems, int unroll) {
     s.tile_elems[bucket] = tile_elems;
     s.unroll_log2[bucket] = (int8_t)ul;
     wx::set_batch_shape(s);
+    return WXPY_OK;
+}
+
+extern "C" int wxpy_debug_batch_vectors(const wxpy_desc *host_table, int64_t count, int *vectors) {
+    if (!vectors) return wx::fail(WXPY_EINVAL, "null argument");
+    const int st = wx::validate_table(host_table, count);
+    if (st != WXPY_OK) return st;
+    const wx::BatchShape shape = wx::current_batch_shape();
+    std::vector<wx::TileRec> tiles;
+    const int64_t elems = wx::build_tiles(host_table, count, shape, true, &tiles);
+    *vectors = wx::wide_body(host_table, count, shape, (int64_t)tiles.size(), elems) ? 4 : 2;
     return WXPY_OK;
 }
 

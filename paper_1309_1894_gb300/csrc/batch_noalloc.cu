@@ -158,7 +158,7 @@ __global__ void __cluster_dims__(BLOCKS, 1, 1) __launch_bounds__(1024)
 __global__ void __launch_bounds__(256, 3) na_run_kernel(const wxpy_desc *table, int64_t count,
                                                         const NaScratch *sc) {
     pdl_enter();
-    run_plan_tiles<3>(table, sc->plan, count);
+    run_plan_tiles<3, kTileU>(table, sc->plan, count);
 }
 
 constexpr int kMaxDev = 64;

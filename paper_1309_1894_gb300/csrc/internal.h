@@ -95,8 +95,13 @@ struct BatchShape {
     int blocks_per_sm;             // grid = blocks_per_sm * sm_count (capped by tiles)
     int offload;                   // integer pipelines: 0 none, 1 half the sums, 3 every product
     int32_t tile_elems[kBuckets];  // per size bucket of a segment; 0 = whole segment
-    int8_t unroll_log2[kBuckets];  // per size bucket: log2 of the unroll
+    int8_t unroll_log2[kBuckets];  // per size bucket: log2 of the unroll; -1: by the batch
 };
+// Of a segment of n elements: log2 of the vectors in flight its tiles ask for.
+int unroll_log2_of(const BatchShape &shape, int64_t n);
+// Whether the launch takes the body with four vectors in flight (batch.cu).
+bool wide_body(const wxpy_desc *t, int64_t count, const BatchShape &shape, int64_t ntiles,
+               int64_t elems);
 BatchShape default_batch_shape();
 BatchShape current_batch_shape();
 void set_batch_shape(const BatchShape &s);
@@ -107,10 +112,10 @@ int64_t tile_cap(int64_t elems);
 int64_t fill_tiles(const wxpy_desc *t, int64_t count, const BatchShape &shape, int64_t t_cap,
                    TileRec *out, int64_t cap);
 // One launch of the segmented kernel over `ntiles` device tile records of `elems`
-// elements in all.
+// elements in all; wide: see wide_body.
 cudaError_t launch_segmented(const wxpy_desc *dev_table, const TileRec *tiles, int64_t ntiles,
-                             int64_t elems, unsigned *status, const BatchShape &shape, int sm_count,
-                             cudaStream_t s);
+                             int64_t elems, bool wide, unsigned *status, const BatchShape &shape,
+                             int sm_count, cudaStream_t s);
 
 // api.cu: NVTX ranges on (WXPY_NVTX=1), read once; see trace.h.
 bool trace_enabled();

@@ -38,14 +38,14 @@ __device__ __forceinline__ int64_t find_segment(const SegPlan *plan, int64_t cou
 }
 
 // One tile; one that would pass the n of the descriptor it reads is skipped.
-template <int EMU>
+template <int EMU, int MAXU>
 __device__ __forceinline__ void run_plan_tile(const wxpy_desc &d, const SegPlan &sp, int64_t t,
                                               int lane) {
     const int64_t T = sp.tile_len(), begin = (t - sp.first_tile) * T;
     const int64_t len = min(T, sp.n - begin);
     if (len > 0 && begin + len <= d.n)
-        tile_wxpy<EMU>(d.x + begin, d.y + begin, d.w + begin, d.alpha, len, lane,
-                       1 << (sp.len_ul >> 30));
+        tile_wxpy<EMU, MAXU>(d.x + begin, d.y + begin, d.w + begin, d.alpha, len, lane,
+                             1 << (sp.len_ul >> 30));
 }
 
 // Every tile of a plan of `count` segments (plan[count].first_tile: the tile
@@ -54,7 +54,7 @@ __device__ __forceinline__ void run_plan_tile(const wxpy_desc &d, const SegPlan 
 // time (40000 segments up to 1024 elements 85 us against 115 on GB300).  Else
 // warp k takes tiles k, k + W, .. and searches for each, so that the warps of an
 // SM work on neighbouring memory (4096 segments up to 2^20: 1141 us against 1210).
-template <int EMU>
+template <int EMU, int MAXU>
 __device__ __forceinline__ void run_plan_tiles(const wxpy_desc *table, const SegPlan *plan,
                                                int64_t count) {
     const int lane = threadIdx.x & 31;
@@ -69,7 +69,7 @@ __device__ __forceinline__ void run_plan_tiles(const wxpy_desc *table, const Seg
     for (int64_t s = 0; t < end; t += step) {
         if (s == 0 || !runs) s = find_segment(plan, count, t, s, lane);
         while (plan[s + 1].first_tile <= t) ++s;
-        run_plan_tile<EMU>(table[s], plan[s], t, lane);
+        run_plan_tile<EMU, MAXU>(table[s], plan[s], t, lane);
     }
 }
 

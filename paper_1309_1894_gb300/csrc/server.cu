@@ -626,7 +626,7 @@ cudaError_t launch_batch(wxpy_server *sv, Slot &s, const std::vector<Request *> 
             const int b = 63 - __builtin_clzll((unsigned long long)r->n);
             T = std::min<int64_t>(shape.tile_elems[b] > 0 ? shape.tile_elems[b] : r->n,
                                   kMaxTileElems);
-            ulog = std::min<int>(2, std::max<int>(0, shape.unroll_log2[b]));
+            ulog = unroll_log2_of(shape, r->n);
         }
         h_plan[i] = ServePlan{nplan, T, ulog, 0};
         if (r->src_kind < 0) nplan += (r->n + T - 1) / T;
@@ -660,6 +660,7 @@ cudaError_t launch_batch(wxpy_server *sv, Slot &s, const std::vector<Request *> 
                                  s.host<TileRec>(s.off_tiles), s.cap_tiles);
         }
     }
+    const bool wide = !fused && wide_body(h_table, count, shape, ntiles, elems);
     // One upload: status word (zero), descriptors, seeds, plan, and the tiles.
     *s.host<unsigned>(0) = 0u;
     const size_t up = fused ? s.off_tiles : s.off_tiles + sizeof(TileRec) * (size_t)ntiles;
@@ -711,7 +712,7 @@ cudaError_t launch_batch(wxpy_server *sv, Slot &s, const std::vector<Request *> 
     // (b) one segmented launch over the batch: reads x, y, writes w; its
     // status word (uploaded as zero) comes back with the batch
     unsigned *d_status = s.dev<unsigned>(0);
-    e = launch_segmented(d_table, s.dev<TileRec>(s.off_tiles), ntiles, elems, d_status, shape,
+    e = launch_segmented(d_table, s.dev<TileRec>(s.off_tiles), ntiles, elems, wide, d_status, shape,
                          sv->sm_count, s.stream);
     if (e != cudaSuccess) return e;
     sv->launches += 1;

@@ -426,8 +426,10 @@ int cache_save(const char *path) {
         out += buf;
         out += "\n  \"batch\": [";
         for (int b = 0; b < kBuckets; ++b) {
-            std::snprintf(buf, sizeof buf, "%s\n    {\"bucket\": %d, \"tile\": %d, \"unroll_log2\": %d}",
-                          b ? "," : "", b, bs.tile_elems[b], (int)bs.unroll_log2[b]);
+            const bool built_in = bs.unroll_log2[b] < 0;
+            std::snprintf(buf, sizeof buf, "%s\n    {\"bucket\": %d, \"tile\": %d, \"unroll_log2\": %d%s}",
+                          b ? "," : "", b, bs.tile_elems[b], built_in ? 2 : (int)bs.unroll_log2[b],
+                          built_in ? ", \"built_in\": 1" : "");
             out += buf;
         }
         out += "\n  ],";
@@ -556,7 +558,10 @@ int cache_load(const char *path, const char *expect_device) {
                 b < 0 || b >= kBuckets || tile < 0 || tile > (1 << 30) || (tile % 32) || ul < 0 || ul > 2)
                 return fail(WXPY_EINVAL, "%s: malformed batch entry", path);
             bs.tile_elems[b] = (int32_t)tile;
-            bs.unroll_log2[b] = (int8_t)ul;
+            long long built_in = 0;
+            if (find_int(s, q, r, "built_in", &built_in) && (built_in < 0 || built_in > 1))
+                return fail(WXPY_EINVAL, "%s: malformed batch entry", path);
+            bs.unroll_log2[b] = (int8_t)(built_in ? -1 : ul);
             q = r;
         }
         have_batch = true;
