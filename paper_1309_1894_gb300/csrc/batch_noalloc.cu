@@ -28,6 +28,7 @@
 #include <cstdint>
 #include <mutex>
 
+#include "cluster.cuh"
 #include "internal.h"
 #include "seg_search.cuh"
 
@@ -78,8 +79,8 @@ __device__ __forceinline__ void cluster_gather(int64_t *slot, int64_t v, int ran
             asm volatile("st.shared::cluster.s64 [%0], %1;" ::"r"(remote), "l"(v) : "memory");
         }
     }
-    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    cluster_arrive();
+    cluster_wait();
 }
 
 // 1. Tile length, tile counts, exclusive prefix over the segments, by one
@@ -95,9 +96,9 @@ __global__ void __cluster_dims__(BLOCKS, 1, 1) __launch_bounds__(1024)
     __shared__ int64_t elems[BLOCKS], tiles_of[BLOCKS];
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, rank = blockIdx.x;
     // no block's shared memory is written before it has started
-    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    cluster_arrive();
     pdl_enter();
-    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    cluster_wait();
     const int per = (int)((count + BLOCKS * 1024 - 1) / (BLOCKS * 1024));  // <= kPer
     const int64_t s0 = ((int64_t)rank * 1024 + tid) * per;
     int64_t n[kPer], total = 0;

@@ -14,6 +14,7 @@
 // elements behind one SM's FP64 pipeline (two sums each, 1.7 per clock: 5 us)
 // and eight dependent loads per thread; here a block holds 1024 elements and
 // every thread loads once.
+#include "cluster.cuh"
 #include "reduce_common.cuh"
 #include "single_kernel.cuh"
 
@@ -22,14 +23,6 @@ namespace {
 
 constexpr int kColumns = 8;         // blocks of a cluster
 constexpr int kSplitThreads = 256;  // eight rows, one warp each
-
-__device__ __forceinline__ void cluster_arrive() {
-    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-}
-
-__device__ __forceinline__ void cluster_wait() {
-    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
 
 // Stores v at `p` (an address of this block's shared memory) in block 0 of the cluster.
 __device__ __forceinline__ void st_first_block(double *p, double v) {

@@ -1,4 +1,4 @@
-"""The hand-over of a shared-memory stage to the copy that refills it (no GPU).
+"""Orderings that no test could provoke reliably, read from the sources (no GPU).
 
 The consumer warps of the staged kernels read a ring stage and then arrive on
 its "empty" barrier, after which a bulk copy may overwrite it.  The arrival,
@@ -36,3 +36,12 @@ def test_every_consumed_stage_is_released():
     used = {name: re.findall(r"mbar_arrive_warp\(smem_addr\(&(\w+)\[", text) for name, text in sources()}
     assert {n: sorted(u) for n, u in used.items() if u} == {
         "vecops.cu": ["empty"], "reduce.cu": ["empty", "xempty", "xfull"]}
+
+
+def test_cluster_barriers_bring_the_warp_together_first():
+    """The aligned cluster barrier is undefined for a warp that is not converged;
+    one thread of a block stores its value just before it."""
+    plain = {name: len(re.findall(r"barrier\.cluster\.", text)) for name, text in sources()}
+    assert {n: c for n, c in plain.items() if c} == {"cluster.cuh": 2}
+    text = dict(sources())["cluster.cuh"]
+    assert len(re.findall(r'__syncwarp\(\);\s*asm volatile\("barrier\.cluster\.', text)) == 2
