@@ -242,7 +242,7 @@ Variant default_variant(const CallClass &c, int64_t n) {
     // 224.6, 885.9 before.
     Variant v{16, 1, 256, 0, 0, -1, 1, 3};
     const bool xy = (c.alias & WXPY_ALIAS_XY) != 0;
-    const bool one_wave = n > ((int64_t)3 << 18) && n <= (int64_t)152 * 8 * 1024;
+    const bool one_wave = n > ((int64_t)3 << 18) && n <= (int64_t)kSmCount * 8 * 1024;
     if (n <= 4096 && c.align >= 16) {
         // The smallest calls are launches: 1.31 to 1.43 against 1.69 before.
         // Narrower accesses are faster (one element per thread 0.94 to 1.18); they
@@ -388,7 +388,7 @@ int launch_piece(const Variant &v, const DeviceProps &dp, int xy, int64_t n, dou
     // axpbypcz, norm2 and dot in turn on 131072 elements: 16.5 us a round when it
     // starts early, 15.0 late; larger grids hide its launch: two calls each on 2^18
     // and 2^19 15.3 us early, 17.4 late, 2^20 4.5 against 5.1).
-    a.late = grid * threads <= (int64_t)dp.sm_count * 256;
+    a.late = ends_at_once(grid, threads, dp.sm_count);
     cudaError_t e = set_carveout(ent.func, dp.device, v.carveout);
     if (e != cudaSuccess) return fail_cuda(e, "cudaFuncSetAttribute(carveout)");
     e = injected_launch_error();

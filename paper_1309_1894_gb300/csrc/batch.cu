@@ -175,17 +175,8 @@ int validate_table(const wxpy_desc *t, int64_t count) {
     return WXPY_OK;
 }
 
-// Batches of kTargetTiles x 8192 elements and more keep the shape's tiles.
-// Smaller ones are cut into shorter tiles (down to 256 elements), so that their
-// warps still spread over every SM: with 8192-element tiles a lone problem of
-// 65536 elements would run on one block.
-constexpr int64_t kTargetTiles = 4864;  // 152 SMs x 4 blocks x 8 warps
-
 int64_t tile_cap(int64_t elems) {
-    int64_t t = 8192;
-    if (elems / t >= kTargetTiles) return kMaxTileElems;
-    while (t > 256 && elems / t < kTargetTiles) t >>= 1;
-    return t;
+    return elems / kSpreadTile >= kTargetTiles ? kMaxTileElems : spread_tile(elems);
 }
 
 static int bucket_of(int64_t v) { return 63 - __builtin_clzll((unsigned long long)v); }

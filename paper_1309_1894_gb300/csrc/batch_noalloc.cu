@@ -13,7 +13,7 @@
 //
 // The plan is made on the device, in the caller's stream, in two launches:
 //   1. a cluster of blocks sums the table's lengths, picks the tile length that
-//      spreads the batch over the GPU (the rule of batch.cu's tile_cap), and
+//      spreads the batch over the GPU (spread_tile), and
 //      scans the tile counts into a per-segment plan;
 //   2. a grid of warps runs the tiles; a warp finds its first tile's segment
 //      in the plan, so no per-tile list is written and read.
@@ -36,9 +36,6 @@ namespace wx {
 namespace {
 
 constexpr int64_t kNaMaxSegments = 65536;  // largest table this entry accepts
-constexpr int64_t kNaTile = 8192;          // elements per tile of a large batch
-constexpr int64_t kNaTargetTiles = 4864;   // as batch.cu: warps to keep busy
-
 constexpr int kPlanBlocks = 8;             // one cluster plans a table
 constexpr int kPer = 8;                    // segments per thread of it, at most
 static_assert((int64_t)kPlanBlocks * 1024 * kPer >= kNaMaxSegments, "the plan holds the table");
@@ -118,8 +115,7 @@ __global__ void __cluster_dims__(BLOCKS, 1, 1) __launch_bounds__(1024)
     cluster_gather<BLOCKS>(elems, total, rank);
     total = 0;
     for (int r = 0; r < BLOCKS; ++r) total += elems[r];
-    int64_t len = kNaTile;
-    while (len > 256 && total / len < kNaTargetTiles) len >>= 1;
+    const int64_t len = spread_tile(total);
     const int shift = 63 - __clzll(len);
     int64_t mine = 0;
 #pragma unroll

@@ -81,7 +81,32 @@ int run_variant(const Variant &v, const CallClass &c, int64_t n, double alpha,
 // Launch gate for fault injection: returns cudaSuccess or the injected error.
 cudaError_t injected_launch_error();
 
+constexpr int kSmCount = 152;  // GB300; rules that have no device at hand
+
+// A grid that fills at most an eighth of the GPU's threads lets the next launch
+// start after its work, not before (launch_piece): the family's kernels and the
+// reference kernel that their timings are compared with.
+inline bool ends_at_once(int64_t grid, int threads, int sm_count) {
+    return grid * threads <= (int64_t)sm_count * 256;
+}
+
 // ---- batched launch (batch.cu) ----
+// Batches of kTargetTiles x 8192 elements and more keep their tiles.  Smaller ones
+// are cut into shorter tiles (down to 256 elements), so that their warps still
+// spread over every SM: with 8192-element tiles a lone problem of 65536 elements
+// would run on one block.
+constexpr int64_t kTargetTiles = (int64_t)kSmCount * 4 * 8;  // four blocks of eight warps
+constexpr int64_t kSpreadTile = 8192;
+
+#ifdef __CUDACC__
+__host__ __device__
+#endif
+inline int64_t spread_tile(int64_t elems) {
+    int64_t t = kSpreadTile;
+    while (t > 256 && elems / t < kTargetTiles) t >>= 1;
+    return t;
+}
+
 // One work item of the segmented launch.
 struct TileRec {
     int64_t begin;    // first element of the tile within its segment

@@ -1,7 +1,7 @@
 // reference.cu -- the reference variant (paper Sec. 2: the plain code whose
 // outputs every variant is compared with): one element per thread, plain
 // loads and stores, the two hardware-rounded FP64 operations.
-#include "single_kernel.cuh"
+#include "internal.h"
 
 namespace wx {
 
@@ -21,7 +21,7 @@ __global__ void wxpy_reference_kernel(const SingleArgs a) {
 
 cudaError_t launch_reference(unsigned grid, unsigned tpb, const SingleArgs &a, cudaStream_t s) {
     SingleArgs r = a;
-    r.late = (int64_t)grid * tpb <= 152 * 256;  // the family's rule (launch_piece), 152 SMs
+    r.late = ends_at_once(grid, (int)tpb, kSmCount);
     return launch_pdl(&wxpy_reference_kernel, grid, tpb, s, r);
 }
 
