@@ -184,7 +184,9 @@ WX_MUL_FN uint32_t mul_distance(const MulCoef &c, uint64_t ub) {
 WX_MUL_FN uint64_t mul_rn_range(const MulCoef &c, uint64_t ub, uint32_t &far) {
     const uint32_t bh = (uint32_t)(ub >> 32), bl = (uint32_t)ub;
     const uint32_t b1 = (bh & 0xFFFFFu) | 0x100000u;
-    const uint32_t d = mul_distance(c, ub);
+    // mul_distance(c, ub), from the word at hand: by way of ub the compiler orders the
+    // wide maxpy groups another way, which is 2 % slower (GB300)
+    const uint32_t d = (bh << 1) - c.from;
     far = d > far ? d : far;
     const uint64_t p00 = (uint64_t)c.lo * bl;
     const uint64_t x = (uint64_t)c.hi * bl + (uint64_t)c.lo * b1 + (p00 >> 32);
