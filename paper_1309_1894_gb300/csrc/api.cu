@@ -239,17 +239,20 @@ Variant default_variant(const CallClass &c, int64_t n) {
     // to hide latency with and a long one ends on small blocks.  2^17 1.56, 2^19
     // 2.74, 2^22 14.9, 2^24 56.5, 2^26 221.9, 2^28 881.0, against 1.72, 3.01, 15.4,
     // 57.0, 222.6, 880.6 for the best 32-byte shape and 2.20, 3.38, 16.0, 57.1,
-    // 224.6, 885.9 before.
+    // 224.6, 885.9 before.  (These and the figures below were taken with one range
+    // test per vector; with one per product 2^20 takes 4.24 us, 16 bytes off 4.29, and
+    // up to 2^14 a twentieth less.)
     Variant v{16, 1, 256, 0, 0, -1, 1, 3};
     const bool xy = (c.alias & WXPY_ALIAS_XY) != 0;
     const bool one_wave = n > ((int64_t)3 << 18) && n <= (int64_t)kSmCount * 8 * 1024;
     if (n <= 4096 && c.align >= 16) {
-        // The smallest calls are launches: 1.31 to 1.43 against 1.69 before.
-        // Narrower accesses are faster (one element per thread 0.94 to 1.18); they
-        // are left to forced variants and to the search, because with one as the
-        // default no cell would count as launch-bound any more: the search marks a
-        // cell where the plain reference kernel is within its tie band of the best
-        // shape, and its choice and the saved one follow that mark.
+        // The smallest calls are mostly launch: 1.31 to 1.43 against 1.69 before.  The
+        // shape still matters: narrower accesses are faster, one element per thread
+        // 0.94 to 1.18.  They are left to forced variants and to the search, because
+        // the search marks a cell as launch-bound where the plain reference kernel is
+        // within its tie band of the best shape, and its choice and the saved one
+        // follow that mark; with one element per thread as the default no cell would
+        // have it any more.
         v = Variant{32, 1, 128, 0, 1, -1, 1, 3};
     } else if (c.align < 16) {
         // Offsets that differ by an odd number of elements.  The worst of the
@@ -270,7 +273,9 @@ Variant default_variant(const CallClass &c, int64_t n) {
         // 2.09); 2^16 1.31 with either
         v.threads = 128;
     } else if (one_wave) {
-        // one wave of 32-byte accesses: 2^20 4.56 against 4.73 (before: 6.05)
+        // one wave of 32-byte accesses: 2^20 4.56 against 4.73 (before: 6.05).  The
+        // upper end is the wave; the lower one lies between 2^19, where 16 bytes are
+        // ahead (2.74 against 3.01), and 2^20, at no measured point.
         v = Variant{32, 1, 256, 0, 1, -1, 1, 3};
     } else if (xy && n > ((int64_t)1 << 20)) {
         // x == y has one load per element in flight, and wants 32 bytes of it:

@@ -80,7 +80,7 @@ struct MulCoef {
 // The exponent window of mul_rn_quick: the 1024 exponent fields from first on,
 // every one of which gives a product in the normal range whatever t and the
 // rounding; 0 when the coefficient has no such window (it is not normal, or
-// 2^1020 or more in magnitude).  The window starts as near to 512 (values from
+// 2^1021 or more in magnitude).  The window starts as near to 512 (values from
 // 2^-511) as the coefficient's exponent allows.
 WX_MUL_FN int mul_window_first(uint64_t ua) {
     const int ea = (int)((ua >> 52) & 0x7FFu);
@@ -246,13 +246,6 @@ __device__ __forceinline__ uint64_t mul_rn_bits(uint64_t ua, uint64_t ub) {
     uint64_t bits = mul_rn_core(mul_coef_of(ua), ub, slow);
     if (slow) bits = mul_rn_hw_bits(ua, ub);
     return bits;
-}
-
-// Operands here are loaded data or kernel parameters, never the output of an
-// FP64 instruction, so their bits are taken directly (no opaque move).
-__device__ __forceinline__ double mul_rn_int(double a, double b) {
-    return __longlong_as_double((long long)mul_rn_bits((uint64_t)__double_as_longlong(a),
-                                                       (uint64_t)__double_as_longlong(b)));
 }
 
 #endif  // __CUDACC__

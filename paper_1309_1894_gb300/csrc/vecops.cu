@@ -11,11 +11,12 @@
 //   maxpy:     y = RN(... RN(RN(y + RN(a0*x0)) + RN(a1*x1)) ... + RN(a_{m-1}*x_{m-1}))
 //   pmult:     w = RN(x*y)
 //
-// One element-wise kernel template serves the three streaming operations: a
-// grid-stride loop over 32-byte vectors when every pointer shares its offset
-// modulo 32 bytes (the head peeled to that boundary and the tail finished
-// with scalars), else over single elements.  A pass loads every input before
-// it stores, so the output may be exactly one of the inputs.
+// axpby, axpbypcz and maxpy run as one template, the staged kernel below, with
+// pointers at any 8-byte offsets; with sums asked for in the integer pipeline and
+// offsets that differ by an odd number of elements they, like pointwise_mult where
+// offsets differ modulo 32 bytes, take single elements, and pointwise_mult else
+// 32-byte vectors.  Every form has an element's inputs loaded before its output is
+// stored, so the output may be exactly one of the inputs.
 //
 // Pipe balance.  On GB300 the FP64 pipeline issues about two operations per
 // clock per SM, and these kernels need more of it than wxpy does: axpbypcz
@@ -23,7 +24,7 @@
 // terms 2m operations per 8(m + 2) bytes.  Both are FP64-bound far below the
 // HBM roofline unless part of the arithmetic moves to the integer pipelines
 // (fp64_emu.cuh, fp64_mul.cuh).  A product costs about twenty ALU operations
-// there and a sum about seventy-five, so products are the cheaper ones to
+// there and a sum about fifty to seventy-five, so products are the cheaper ones to
 // move: a runtime fraction (in sixteenths) of each warp's loop iterations
 // computes all of its products in the integer pipeline, the rest in FP64;
 // the choice is uniform across the warp (no divergence) and rotates with the

@@ -81,7 +81,8 @@ def test_parity(kind, variant, mul, offs):
 def test_many_tiles_per_block(kind, variant, mul, offs):
     """2^24 + 12345 elements: several tiles per block of every kernel variant
     (every exchange slot and ring stage of the staged ones reused), a ragged
-    last tile; the 16-byte offsets take the element path."""
+    last tile; pointers at one offset past 32 bytes take variant 0's shifted vectors,
+    differing offsets its single elements."""
     wx.wxpy_reduce_variant(variant)
     wx.wxpy_reduce_pipes(mul)
     n = (1 << 24) + 12345
