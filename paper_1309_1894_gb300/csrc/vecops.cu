@@ -180,7 +180,7 @@ struct AxpbypczOp {
 // 252.
 template <int M>
 __device__ constexpr unsigned integer_sums(int q) {
-    constexpr unsigned k[7][2] = {{0, 0}, {0, 0}, {1u << 1, 0}, {1u << 3, 0},
+    constexpr unsigned k[7][2] = {{0, 0}, {0, 0}, {1u << 1, 0}, {1u << 2, 0},
                                   {0, 1u << 3}, {0, 1u << 3}, {1u << 2, 1u << 5}};
     return k[M - 2][q];
 }
