@@ -141,7 +141,7 @@ def test_maxpy_sums(n, shifts, m, kind, scale):
 # a few per block, whose later tiles take other products where the earlier ones
 # left the integer pipelines; every way the offsets deal the elements.
 @pytest.mark.parametrize("kind", KINDS)
-@pytest.mark.parametrize("tiles", [2, 130, 300, 2500])
+@pytest.mark.parametrize("tiles", [2, 130, 300, 1000, 2500])
 @pytest.mark.parametrize("shifts", [(0, 0, 0, 0), (1, 1, 1, 1), (0, 1, 2, 3)])
 def test_reductions(tiles, shifts, kind):
     n = tiles * 8192 - 100
