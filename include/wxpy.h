@@ -262,7 +262,8 @@ int wxpy_pointwise_mult(int64_t n, const double *x, const double *y, double *w, 
  * pointwise_mult): how much of their binary64 arithmetic runs as the exactly
  * rounded integer-pipeline operations instead of FP64 instructions.
  * add_offload: the sums (0 none -- but where its products run there too, one or
- * two in sixteen of a maxpy group of 4..8 terms -- 1 every other one, 2 all);
+ * two per pair of elements of a maxpy group of 4..8 terms -- 1 every other one,
+ * 2 all);
  * mul_sixteenths:
  * the fraction, in sixteenths, of each warp's loop iterations whose products
  * run there (0..16).  -1 in either leaves that part to the operation's

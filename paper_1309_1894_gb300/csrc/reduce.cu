@@ -594,16 +594,16 @@ std::atomic<int> g_reduce_last[2];  // per kind, the range stored last
 constexpr int kDefaultSumLevels = 0;
 constexpr int kReduceVariants = 7;  // 0 register-loaded, 1..3 staged, 4..6 warp-tiled
 // Measured on GB300 at n = 2^26 with every product in the integer pipelines
-// (GB/s of algorithmic bytes, norm2 / dot): register-loaded 5500 / 6115; staged
+// (GB/s of algorithmic bytes, norm2 / dot): register-loaded 5726 / 6430; staged
 // 4700 / 5136, 4604 / 4784, 4637 / 5194; warp-tiled 4599 / 5526, 5029 / 5286,
 // 4697 / 5838.
 constexpr int kDefaultVariant[2] = {0, 0};  // norm2, dot
 // Tiles up to which a call takes the cluster form (reduce_split.cu).  Measured on
-// GB300, norm2 / dot, us, cluster against block form: 2^21 elements 16.7 / 18.2
-// against 17.8 / 19.5, 2^22 30.3 / 31.6 against 28.1 / 31.5.  With offsets that
-// differ the block form reads single elements too: 2^22 32.2 / 37.0 against
-// 34.2 / 37.2, 2^23 59.9 / 69.5 against 63.2 / 70.4, 2^24 107.6 / 121.7 against
-// 108.1 / 122.4.
+// GB300, norm2 / dot, us, cluster against block form: 2^21 elements 17.0 / 19.0
+// against 17.9 / 19.3, 3 x 2^20 25.4 / 27.6 against 23.6 / 25.4.  With offsets that
+// differ the block form reads single elements too: 2^22 33.7 / 37.3 against
+// 34.4 / 39.5, 2^23 60.9 / 68.2 against 62.8 / 72.1, 2^24 108.4 / 123.0 against
+// 106.9 / 124.0.
 constexpr int64_t kSplitTiles = 256, kSplitTilesMixed = 1024;
 constexpr int kDefaultMulSixteenths = 16;  // measured fastest on GB300 (both operations)
 

@@ -29,8 +29,8 @@
 // computes all of its products in the integer pipeline, the rest in FP64;
 // the choice is uniform across the warp (no divergence) and rotates with the
 // iteration, so every SM sub-partition sees the same mix.  Sums can move too
-// (add offload 1: every other one, 2: all; 0: none, but for one or two of a wide
-// maxpy group's, see integer_sums).  Every split gives the same bits.
+// (add offload 1: every other one, 2: all; 0: none, but for one or two per pair of
+// elements of a wide maxpy group, see integer_sums).  Every split gives the same bits.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -173,8 +173,8 @@ struct AxpbypczOp {
 // pair.  The FP64 pipeline does 1.7 sums per clock and SM whatever the code
 // (5.0e11/s), so m sums per 8(m + 2) bytes hold these kernels to 0.92 of the HBM
 // peak with 4 terms and 0.76 with 8; an integer sum is about 50 ALU operations,
-// and there is ALU time left for one or two in sixteen.  n = 2^24 (GB300), us
-// with none / these: 4 terms 137 / 133, 5 169 / 159, 6 204 / 191, 7 237 / 221,
+// and there is ALU time left for one or two per pair of elements.  n = 2^24 (GB300), us
+// with none / these: 4 terms 137 / 133, 5 169 / 158, 6 204 / 191, 7 237 / 221,
 // 8 269 / 246; with 3 terms one of six is slower.  Which of them matters, by
 // where it falls among the other sums: 8 terms with sums 0 and 0 264, 3 and 3
 // 252.
