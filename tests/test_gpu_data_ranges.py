@@ -112,7 +112,8 @@ def test_streaming_siblings(n, shifts, kind):
 @pytest.mark.parametrize("m", [2, 3, 4, 5, 6, 7, 8])
 @pytest.mark.parametrize("kind,scale", [("uniform", 1e-12), ("uniform", 2.0 ** -31), ("uniform", 1e12),
                                         ("y zero", 1.0), ("y infinite", 1.0), ("cancelling", 1.0),
-                                        ("mixed", 1.0), ("sevenths", 1e-12), ("spread", 1.0)])
+                                        ("mixed", 1.0), ("sevenths", 1e-12), ("spread", 1.0),
+                                        ("ties", 1.0)])
 @pytest.mark.parametrize("n,shifts", [(4099, (0, 0)), (2_000_003, (0, 0)), (2_000_003, (1, 0))])
 def test_maxpy_sums(n, shifts, m, kind, scale):
     """Terms far below and above the vector they are added to, a zero vector, and
@@ -126,6 +127,16 @@ def test_maxpy_sums(n, shifts, m, kind, scale):
         yh[::3] = -0.0
     elif kind == "y infinite":
         yh[1::5] = np.inf
+    elif kind == "ties":
+        # half an ulp of the sum so far, exactly or missed by a bit far below, at gaps
+        # of 52 to 54 and beyond
+        rng = np.random.default_rng(n + m)
+        yh = (1.0 + rng.integers(0, 1 << 52, n) * 2.0 ** -52) * np.where(rng.random(n) < 0.1, 0, 1) + 1.0
+        al = [1.0, -1.0, 0.5, 2.0, -0.5, 1.0, -2.0, 0.25][:m]
+        for j in range(m):
+            half = 2.0 ** -52 * rng.choice([0.5, 1.0, 1.5, 2.0, 3.0, 2.0 ** -8], n)
+            xs[j] = half * (1 + rng.choice([0.0, 2.0 ** -52, 2.0 ** -20, -2.0 ** -53], n))
+            xs[j] *= rng.choice([-1.0, 1.0], n)
     elif kind == "cancelling":
         for j in range(1, m):
             xs[j][::2] = xs[j - 1][::2] * (-al[j - 1] / al[j]) * (1 + 2.0 ** -40)
