@@ -533,7 +533,7 @@ cudaError_t copy_in(const Request *r, cudaStream_t st) {
     return e;
 }
 
-// The driver's knowledge of an address (ptr_range.h); no context is needed.
+// What CUDA knows of an address (ptr_range.h); no context is needed.
 bool address_info(uint64_t p, AddressInfo *info) {
     using Fn = CUresult (*)(unsigned, CUpointer_attribute *, void **, CUdeviceptr);
     static const Fn get = [] {
